@@ -229,7 +229,8 @@ extern "C" fa_status fa_warp_lncc_adjoint(const fa_vol *fixed, const fa_vol *mov
     FA_CUDA_TRY(launch_header_reset(b.h, s));
     FA_CUDA_TRY(launch_warp(Im, uu, b.J, du ? b.grad : nullptr, d, s));
     FA_CUDA_TRY(launch_absmax2(I, b.J, N, b.h, s));
-    FA_CUDA_TRY(launch_lncc_forward(I, b.J, d, window, cc_eps, dIf != nullptr, b.h, b.lb, s));
+    FA_CUDA_TRY(launch_lncc_forward(I, b.J, d, window, cc_eps, true, dIf != nullptr, b.h, b.lb,
+                                    s));
     FA_CUDA_TRY(launch_loss_finalize(b.h, N, -1.0f, loss_dev, s));
     if (du || dIf || dIm)
         FA_CUDA_TRY(launch_lncc_backward(I, b.J, du ? b.grad : nullptr, d, window, b.h, b.lb,

@@ -411,7 +411,8 @@ cudaError_t affine_gradient(AffineWs &w, const fa_params *p, const float *If, co
     if (p->loss == FA_LOSS_LNCC) {
         e = launch_absmax2(If, w.J, d.N(), w.h, s);
         if (e == cudaSuccess)
-            e = launch_lncc_forward(If, w.J, d, p->window, p->cc_eps, false, w.h, w.lb, s);
+            e = launch_lncc_forward(If, w.J, d, p->window, p->cc_eps, want_grad, false, w.h, w.lb,
+                                    s);
         if (e == cudaSuccess && want_grad)
             e = launch_lncc_backward(If, w.J, w.grad, d, p->window, w.h, w.lb, nullptr, nullptr,
                                      w.g, s);

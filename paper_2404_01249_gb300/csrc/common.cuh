@@ -325,16 +325,19 @@ __device__ __forceinline__ long long quantize(float v, float scale) {
 // limited the exact-sum kernels; they use 32-bit conversions, integer
 // operations and FP32 adds, and give the same bits as that instruction.
 
-// uint64 -> float, rounded to nearest even: the leading 24 bits, rounded by
-// the 40 bits below them (a carry out of the mantissa raises the exponent).
+// The 64-bit value h 2^32 + l -> float, rounded to nearest even: its leading
+// 32 bits, the lowest of them ORed with "any bit below is set" (which decides
+// no tie it should not), take the 32-bit conversion's one rounding to 24 bits.
+__device__ __forceinline__ float u64_halves_to_float_rn(unsigned h, unsigned l) {
+    const unsigned hh = h ? h : l, ll = h ? l : 0u;
+    const int lz = __clz((int)hh) & 31;  // 0 stays 0
+    const unsigned top = __funnelshift_l(ll, hh, lz) | ((ll << lz) != 0u ? 1u : 0u);
+    return __uint2float_rn(top) * __uint_as_float((unsigned)((h ? 159 : 127) - lz) << 23);
+}
+
+// uint64 -> float, rounded to nearest even.
 __device__ __forceinline__ float u64_to_float_rn(unsigned long long u) {
-    if (u == 0ull) return 0.0f;
-    const int lz = __clzll((long long)u);
-    const unsigned long long m = u << lz;  // bit 63 set
-    unsigned mant = (unsigned)(m >> 40);   // 24 bits, the leading one included
-    const unsigned long long rest = m & 0xFFFFFFFFFFull, half = 1ull << 39;
-    mant += (rest > half || (rest == half && (mant & 1u))) ? 1u : 0u;
-    return __uint_as_float(((unsigned)(190 - lz) << 23) + (mant - 0x800000u));
+    return u64_halves_to_float_rn((unsigned)(u >> 32), (unsigned)u);
 }
 
 __device__ __forceinline__ float i64_to_float_rn(long long x) {
@@ -353,18 +356,47 @@ __device__ __forceinline__ void i64_to_ff(long long x, float &hi, float &lo) {
     lo = __fsub_rn(fl, __fsub_rn(hi, fh));
 }
 
-// n a - b c for int64 operands, formed exactly in 128 bits and rounded to
-// float (one rounding when the result fits 64 bits; otherwise the two halves
-// are scaled and added, within one float ulp).
+// n a - b c, formed exactly and rounded to float (one rounding when the
+// result fits 64 bits; otherwise the two halves are scaled and added, within
+// one float ulp).  For 0 < n < 2^13, |a| <= 2^62 and |b|, |c| < 2^40 (window
+// sums): the result fits 96 bits, so three 32-bit limbs replace 128-bit
+// products, without a branch.  NONNEG: the caller knows the result is not
+// negative (a variance).
+template <bool NONNEG = false>
 __device__ __forceinline__ float diff_i128_to_float(long long n, long long a, long long b,
                                                     long long c) {
-    const __int128 r = (__int128)n * a - (__int128)b * c;
-    const long long hi = (long long)(r >> 64);
-    const unsigned long long lo = (unsigned long long)r;
-    if (hi == 0) return u64_to_float_rn(lo);
-    if (hi == -1 && (long long)lo < 0) return i64_to_float_rn((long long)lo);
-    // |hi| < 2^24 here (|r| < 2^88), so its 32-bit conversion is exact
-    return fmaf(__int2float_rn((int)hi), 18446744073709551616.0f, u64_to_float_rn(lo));
+    const unsigned nn = (unsigned)n, a0 = (unsigned)a, b0 = (unsigned)b, c0 = (unsigned)c;
+    const int a1 = (int)(a >> 32), b1 = (int)(b >> 32), c1 = (int)(c >> 32);
+    // n a: low 32 bits of t, the rest in th
+    const unsigned long long t = (unsigned long long)a0 * nn;
+    const long long th = (long long)a1 * (int)nn + (long long)(t >> 32);
+    // b c: low 32 bits of p, the rest in q (two's complement limbs: the top
+    // limb takes back what reading negative c1, b1 as unsigned adds)
+    const unsigned long long p = (unsigned long long)b0 * c0;
+    unsigned long long q = (unsigned long long)b0 * (unsigned)c1 +
+                           (unsigned long long)(unsigned)b1 * c0 + (p >> 32);
+    q += (unsigned long long)((unsigned)b1 * (unsigned)c1 - (b0 & (unsigned)(c1 >> 31)) -
+                              (c0 & (unsigned)(b1 >> 31)))
+         << 32;
+    const unsigned long long u =
+        (unsigned long long)th - q - ((unsigned)t < (unsigned)p ? 1ull : 0ull);
+    int hi = (int)(u >> 32);
+    unsigned mid = (unsigned)u, lo = (unsigned)t - (unsigned)p;
+    unsigned sign = 0u;
+    if (!NONNEG) {  // a negative 64-bit result: its magnitude, and hi of zero
+        const unsigned m = hi == -1 && (int)mid < 0 ? 0xffffffffu : 0u;
+        const unsigned long long v =
+            ((((unsigned long long)mid << 32) | lo) ^ (((unsigned long long)m << 32) | m)) -
+            (((unsigned long long)m << 32) | m);
+        mid = (unsigned)(v >> 32);
+        lo = (unsigned)v;
+        hi = (int)((unsigned)hi & ~m);
+        sign = m & 0x80000000u;
+    }
+    const float f =
+        __uint_as_float(__float_as_uint(u64_halves_to_float_rn(mid, lo)) ^ sign);
+    // |hi| < 2^24, so its conversion is exact; hi = 0 leaves f
+    return fmaf(__int2float_rn(hi), 18446744073709551616.0f, f);
 }
 
 // ---------------------------------------------------------- float-float

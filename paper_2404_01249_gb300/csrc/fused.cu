@@ -13,23 +13,6 @@ namespace {
 
 // ================================================================ launching
 
-// Slab depth TZ minimising (waves x planes per CTA) for a z-marching kernel.
-int choose_tz(int D, int tiles_xy, int halo, int ctas_per_sm) {
-    const long long slots = (long long)num_sms() * (ctas_per_sm > 0 ? ctas_per_sm : 1);
-    int best = D;
-    long long bestcost = -1;
-    for (int tz = 1; tz <= D && tz <= 64; ++tz) {
-        const long long ctas = (long long)tiles_xy * ((D + tz - 1) / tz);
-        const long long waves = (ctas + slots - 1) / slots;
-        const long long cost = waves * (tz + 2 * halo);
-        if (bestcost < 0 || cost < bestcost) {
-            bestcost = cost;
-            best = tz;
-        }
-    }
-    return best;
-}
-
 // ------------------------------------------------------------- tile choices
 // Per (kernel, radius, compose variant, level grid): the slab depth TZ
 // (0: the cost model above) and, for K3/K4 on the TMA path, 32 x 16 tiles
@@ -64,7 +47,7 @@ TileChoice tile_choice(int kernel, int radius, int su, Dims d) {
 inline LaunchGeom geometry(int occ, int nw, int ty, int halo, Dims d, int tz = 0) {
     LaunchGeom g;
     const int gx = (d.W + FX - 1) / FX, gy = (d.H + ty - 1) / ty;
-    g.tz = tz > 0 ? (tz < d.D ? tz : d.D) : choose_tz(d.D, gx * gy, halo, occ);
+    g.tz = tz > 0 ? (tz < d.D ? tz : d.D) : choose_tz(d.D, gx * gy, 2.0f * halo, occ);
     g.grid = dim3(gx, gy, (d.D + g.tz - 1) / g.tz);
     g.block = dim3(FX, nw);
     return g;
@@ -150,62 +133,34 @@ bool tmap(CUtensorMap *m, const void *base, int esize, Dims d, int C, int bx, in
 namespace {
 
 
-template <int R>
 cudaError_t launch_k1(const float *If, const float *J, const long long *sI, const float *varI,
                       float *coef, WsHeader *h, Dims d, int window, float cc_eps, bool wc,
                       cudaStream_t s) {
-    const int bits = lncc_image_bits(window);
-    Maps mp{};
-    cudaError_t le;
-    using ST = K1S<R, K1_NW, K1_OPT, K1_ST_TMA>;
-    const bool tma = tmap(&mp.a, If, 4, d, 1, ST::BXW, ST::RY, 1) &&
-                     tmap(&mp.b, J, 4, d, 1, ST::BXW, ST::RY, 1);
-    const TileChoice tc = tile_choice(0, R, 0, d);
-    if (tma) {
-        auto kern = k_lncc_fwd<R, K1_NW, K1_OPT, K1_ST_TMA, true>;
-        static const int occ = prepare(kern, ST::bytes, ST::NT);
-        LaunchGeom g = geometry(occ, K1_NW, ST::TY, R, d, tc.tz);
-        le = launch_pdl(kern, g, ST::bytes, s, mp, If, J, sI, varI, coef, h, d.D, d.H, d.W, d.pitch(), g.tz,
-                                                bits, cc_eps, window, wc ? 1 : 0);
-    } else {
-        using SC = K1S<R, K1_NW, K1_OPT, K1_ST_CP>;
-        auto kern = k_lncc_fwd<R, K1_NW, K1_OPT, K1_ST_CP, false>;
-        static const int occ = prepare(kern, SC::bytes, SC::NT);
-        LaunchGeom g = geometry(occ, K1_NW, SC::TY, R, d, tc.tz);
-        le = launch_pdl(kern, g, SC::bytes, s, mp, If, J, sI, varI, coef, h, d.D, d.H, d.W, d.pitch(), g.tz,
-                                                bits, cc_eps, window, wc ? 1 : 0);
-    }
-    note_launch();
-    return le;
+    FwdArgs a{};
+    a.I = If;
+    a.J = J;
+    a.SI = const_cast<long long *>(sI);
+    a.varI = const_cast<float *>(varI);
+    a.coef = coef;
+    a.h = h;
+    a.cc_eps = cc_eps;
+    a.write_coef = wc;
+    return launch_window_fwd(kFwdGiven, a, d, window, tile_choice(0, window / 2, 0, d).tz, s);
 }
 
-// WDJ: the adjoint's variant, which also writes dL/dJ to dJout.
-template <int R, bool WDJ = false>
+// dJout (may be NULL): also write dL/dJ, which the adjoint's scatter needs.
 cudaError_t launch_k2(const float *If, const float *gJ, const float *J, const float *coef,
-                      WsHeader *h, float *g, Dims d, int window, cudaStream_t s,
-                      float *dJout = nullptr) {
-    const int cb = lncc_coef_bits(window);
-    Maps mp{};
-    cudaError_t le;
-    using ST = K2S<R, K2_NW, K2_OPT, K2_ST_TMA>;
-    const bool tma = tmap(&mp.a, coef, 4, d, 4, ST::BXW, ST::RY, 4);
-    const TileChoice tc = tile_choice(1, R, 0, d);
-    if (tma) {
-        auto kern = k_lncc_grad<R, K2_NW, K2_OPT, K2_ST_TMA, true, WDJ>;
-        static const int occ = prepare(kern, ST::bytes, ST::NT);
-        LaunchGeom gg = geometry(occ, K2_NW, ST::TY, R, d, tc.tz);
-        le = launch_pdl(kern, gg, ST::bytes, s, mp, If, gJ, J, coef, h, g, d.D, d.H, d.W, d.pitch(), gg.tz,
-                        cb, dJout);
-    } else {
-        using SC = K2S<R, K2_NW, K2_OPT, K2_ST_CP>;
-        auto kern = k_lncc_grad<R, K2_NW, K2_OPT, K2_ST_CP, false, WDJ>;
-        static const int occ = prepare(kern, SC::bytes, SC::NT);
-        LaunchGeom gg = geometry(occ, K2_NW, SC::TY, R, d, tc.tz);
-        le = launch_pdl(kern, gg, SC::bytes, s, mp, If, gJ, J, coef, h, g, d.D, d.H, d.W, d.pitch(), gg.tz,
-                        cb, dJout);
-    }
-    note_launch();
-    return le;
+                      const WsHeader *h, float *g, float *dJout, Dims d, int window,
+                      cudaStream_t s) {
+    GradArgs a{};
+    a.I = If;
+    a.J = J;
+    a.gJ = gJ;
+    a.coef = coef;
+    a.h = h;
+    a.g = g;
+    a.dJ = dJout;
+    return launch_window_grad(false, a, d, window, tile_choice(1, window / 2, 0, d).tz, s);
 }
 
 template <int RG, int NW, class TS>
@@ -305,54 +260,6 @@ cudaError_t launch_k4(const TU *u, const float *dir, TU *uo, const float *Im, fl
         return call;          \
     }
 
-cudaError_t dispatch_k1(const float *If, const float *J, const long long *sI, const float *varI,
-                        float *coef, WsHeader *h, Dims d, int window, float cc_eps, bool wc,
-                        cudaStream_t s) {
-    switch (window / 2) {
-        FA_CASE(0, (launch_k1<RR>(If, J, sI, varI, coef, h, d, window, cc_eps, wc, s)))
-        FA_CASE(1, (launch_k1<RR>(If, J, sI, varI, coef, h, d, window, cc_eps, wc, s)))
-        FA_CASE(2, (launch_k1<RR>(If, J, sI, varI, coef, h, d, window, cc_eps, wc, s)))
-        FA_CASE(3, (launch_k1<RR>(If, J, sI, varI, coef, h, d, window, cc_eps, wc, s)))
-        FA_CASE(4, (launch_k1<RR>(If, J, sI, varI, coef, h, d, window, cc_eps, wc, s)))
-        FA_CASE(5, (launch_k1<RR>(If, J, sI, varI, coef, h, d, window, cc_eps, wc, s)))
-        FA_CASE(6, (launch_k1<RR>(If, J, sI, varI, coef, h, d, window, cc_eps, wc, s)))
-        FA_CASE(7, (launch_k1<RR>(If, J, sI, varI, coef, h, d, window, cc_eps, wc, s)))
-    }
-    return cudaErrorInvalidValue;
-}
-
-cudaError_t dispatch_k2(const float *If, const float *gJ, const float *J, const float *coef,
-                        WsHeader *h, float *g, Dims d, int window, cudaStream_t s) {
-    switch (window / 2) {
-        FA_CASE(0, (launch_k2<RR>(If, gJ, J, coef, h, g, d, window, s)))
-        FA_CASE(1, (launch_k2<RR>(If, gJ, J, coef, h, g, d, window, s)))
-        FA_CASE(2, (launch_k2<RR>(If, gJ, J, coef, h, g, d, window, s)))
-        FA_CASE(3, (launch_k2<RR>(If, gJ, J, coef, h, g, d, window, s)))
-        FA_CASE(4, (launch_k2<RR>(If, gJ, J, coef, h, g, d, window, s)))
-        FA_CASE(5, (launch_k2<RR>(If, gJ, J, coef, h, g, d, window, s)))
-        FA_CASE(6, (launch_k2<RR>(If, gJ, J, coef, h, g, d, window, s)))
-        FA_CASE(7, (launch_k2<RR>(If, gJ, J, coef, h, g, d, window, s)))
-    }
-    return cudaErrorInvalidValue;
-}
-
-// The adjoint's K2 (windows 1..15): g and dL/dJ.
-cudaError_t dispatch_k2_dj(const float *If, const float *gJ, const float *J, const float *coef,
-                           WsHeader *h, float *g, float *dJ, Dims d, int window, cudaStream_t s) {
-    switch (window / 2) {
-        FA_CASE(0, (launch_k2<RR, true>(If, gJ, J, coef, h, g, d, window, s, dJ)))
-        FA_CASE(1, (launch_k2<RR, true>(If, gJ, J, coef, h, g, d, window, s, dJ)))
-        FA_CASE(2, (launch_k2<RR, true>(If, gJ, J, coef, h, g, d, window, s, dJ)))
-        FA_CASE(3, (launch_k2<RR, true>(If, gJ, J, coef, h, g, d, window, s, dJ)))
-        FA_CASE(4, (launch_k2<RR, true>(If, gJ, J, coef, h, g, d, window, s, dJ)))
-        FA_CASE(5, (launch_k2<RR, true>(If, gJ, J, coef, h, g, d, window, s, dJ)))
-        FA_CASE(6, (launch_k2<RR, true>(If, gJ, J, coef, h, g, d, window, s, dJ)))
-        FA_CASE(7, (launch_k2<RR, true>(If, gJ, J, coef, h, g, d, window, s, dJ)))
-    }
-    return cudaErrorInvalidValue;
-}
-
-
 template <class TS>
 cudaError_t dispatch_k3_ts(const float *g, TS *m, TS *v, float *dir, WsHeader *h, Dims d,
                            const GaussTaps &t, AdamConsts ac, int parity, cudaStream_t s) {
@@ -429,8 +336,8 @@ struct KTimer {
 }  // namespace
 
 void fused_carve(WsCarver &c, long long n, FusedBuffers *fb) {
-    fb->coef = c.take<float>(4 * n);  // also the first int64 scratch of the fixed statistics
-    fb->g = c.take<float>(4 * n);     // also the second one
+    fb->coef = c.take<float>(4 * n);
+    fb->g = c.take<float>(4 * n);  // three channels; the size callers allocate by
     fb->dir = c.take<float>(3 * n);
     fb->J = c.take<float>(n);
     fb->gJ = c.take<float>(3 * n);
@@ -441,11 +348,10 @@ void fused_carve(WsCarver &c, long long n, FusedBuffers *fb) {
 }
 
 cudaError_t fused_level_start(const float *If, const float *Im, const float *u, Dims d,
-                              const fa_params *p, const WsHeader *h, FusedBuffers &fb,
+                              const fa_params *p, WsHeader *h, FusedBuffers &fb,
                               cudaStream_t s) {
     if (p->loss == FA_LOSS_LNCC) {
-        cudaError_t e = launch_fixed_stats(If, d, p->window, h, (long long *)fb.coef,
-                                           (long long *)fb.g, fb.sI, fb.varI, s);
+        cudaError_t e = launch_fixed_stats(If, d, p->window, h, fb.sI, fb.varI, s);
         if (e != cudaSuccess) return e;
     }
     return launch_warp_field(Im, u, p->field_storage, fb.J, fb.gJ, d, s);
@@ -467,11 +373,11 @@ fa_status fused_iteration(FusedBuffers &fb, WsHeader *h, const fa_params *p, Dim
     const int parity = it.t & 1;
     if (p->loss == FA_LOSS_LNCC) {
         FA_CUDA_TRY(start(FA_K_FUSED_WARP_LNCC));
-        FA_CUDA_TRY(dispatch_k1(it.If, fb.J, fb.sI, fb.varI, fb.coef, h, d, p->window, p->cc_eps,
+        FA_CUDA_TRY(launch_k1(it.If, fb.J, fb.sI, fb.varI, fb.coef, h, d, p->window, p->cc_eps,
                                 true, s));
         FA_CUDA_TRY(stop(FA_K_FUSED_WARP_LNCC));
         FA_CUDA_TRY(start(FA_K_FUSED_LNCC_GRAD));
-        FA_CUDA_TRY(dispatch_k2(it.If, fb.gJ, fb.J, fb.coef, h, fb.g, d, p->window, s));
+        FA_CUDA_TRY(launch_k2(it.If, fb.gJ, fb.J, fb.coef, h, fb.g, nullptr, d, p->window, s));
         FA_CUDA_TRY(stop(FA_K_FUSED_LNCC_GRAD));
     } else if (p->loss == FA_LOSS_MI) {
         FA_CUDA_TRY(start(FA_K_FUSED_LNCC_GRAD));
@@ -530,9 +436,9 @@ fa_status fused_autotune_level(FusedBuffers &fb, WsHeader *h, const fa_params *p
     auto launch = [&](int kernel) -> cudaError_t {
         switch (kernel) {
             case 0:
-                return dispatch_k1(If, fb.J, fb.sI, fb.varI, fb.coef, h, d, p->window, p->cc_eps,
+                return launch_k1(If, fb.J, fb.sI, fb.varI, fb.coef, h, d, p->window, p->cc_eps,
                                    true, s);
-            case 1: return dispatch_k2(If, fb.gJ, fb.J, fb.coef, h, fb.g, d, p->window, s);
+            case 1: return launch_k2(If, fb.gJ, fb.J, fb.coef, h, fb.g, nullptr, d, p->window, s);
             case 2: return dispatch_k3(fb.g, m, v, p->state_storage, fb.dir, h, d, g3, ac, 0, s);
             default:
                 return dispatch_k4(u, fb.dir, u_alt, p->field_storage, Im, fb.J, fb.gJ, h, d, g4,
@@ -616,7 +522,7 @@ int fused_tile_choices(int32_t *out, int capacity) {
 
 cudaError_t fused_lncc_forward_only(const float *If, const FusedBuffers &fb, Dims d, int window,
                                     float cc_eps, WsHeader *h, cudaStream_t s) {
-    return dispatch_k1(If, fb.J, fb.sI, fb.varI, nullptr, h, d, window, cc_eps, false, s);
+    return launch_k1(If, fb.J, fb.sI, fb.varI, nullptr, h, d, window, cc_eps, false, s);
 }
 
 cudaError_t fused_warp_lncc_adjoint(const float *If, const float *Im, const float *u,
@@ -626,16 +532,14 @@ cudaError_t fused_warp_lncc_adjoint(const float *If, const float *Im, const floa
     cudaError_t e;
     if ((e = launch_warp(Im, u, fb.J, g ? fb.gJ : nullptr, d, s)) != cudaSuccess) return e;
     if ((e = launch_absmax2(If, fb.J, d.N(), h, s)) != cudaSuccess) return e;
-    if ((e = launch_fixed_stats(If, d, window, h, (long long *)fb.coef, (long long *)fb.g, fb.sI,
-                                fb.varI, s)) != cudaSuccess)
+    if ((e = launch_fixed_stats(If, d, window, h, fb.sI, fb.varI, s)) != cudaSuccess)
         return e;
-    if ((e = dispatch_k1(If, fb.J, fb.sI, fb.varI, fb.coef, h, d, window, cc_eps, g != nullptr,
+    if ((e = launch_k1(If, fb.J, fb.sI, fb.varI, fb.coef, h, d, window, cc_eps, g != nullptr,
                          s)) != cudaSuccess)
         return e;
     if ((e = launch_loss_finalize(h, d.N(), -1.0f, loss_dev, s)) != cudaSuccess) return e;
     if (!g) return cudaSuccess;
-    return dJ ? dispatch_k2_dj(If, fb.gJ, fb.J, fb.coef, h, g, dJ, d, window, s)
-              : dispatch_k2(If, fb.gJ, fb.J, fb.coef, h, g, d, window, s);
+    return launch_k2(If, fb.gJ, fb.J, fb.coef, h, g, dJ, d, window, s);
 }
 
 // Self-test of the bounded wait: one thread waits on an mbarrier that no

@@ -28,32 +28,16 @@ struct BGeom {
 struct BTaps {
     float w[2 * kMaxFusedRG + 1];
 };
-struct K1Job {
-    const float *If, *J;
-    const long long *SI;
-    const float *varI;
-    float *coef;
-    WsHeader *h;
-    BGeom g;
-    float cc_eps;
-};
+// K1 and K2 take every job's arguments as a single launch does.
 struct K1Batch {
-    CUtensorMap tm[2 * kMaxLockstepJobs];  // job k: I_f at 2k, J at 2k + 1
-    int n, bits, window, write_coef;
+    int n;
     int first[kMaxLockstepJobs + 1];
-    K1Job j[kMaxLockstepJobs];
-};
-struct K2Job {
-    const float *If, *gJ, *J, *coef;
-    float *g;
-    WsHeader *h;
-    BGeom geo;
+    FwdArgs j[kMaxLockstepJobs];
 };
 struct K2Batch {
-    CUtensorMap tm[kMaxLockstepJobs];  // job k: the A, B, C coefficients
-    int n, cbits;
+    int n;
     int first[kMaxLockstepJobs + 1];
-    K2Job j[kMaxLockstepJobs];
+    GradArgs j[kMaxLockstepJobs];
 };
 struct K3Job {
     const float *g;
@@ -129,26 +113,31 @@ __device__ __forceinline__ MapRef job_maps(const CUtensorMap *tm, int k) {
     return r;
 }
 
-template <int R, bool TMA>
-__global__ void __launch_bounds__(FX *K1_NW) k_lncc_fwd_batch(const __grid_constant__ K1Batch b) {
-    const int k = batch_job(b.first, b.n, (int)blockIdx.x);
-    const K1Job &j = b.j[k];
-    int bx, by, bz;
-    batch_tile(j.g, (int)blockIdx.x - b.first[k], bx, by, bz);
-    lncc_fwd_body<R, K1_NW, K1_OPT, TMA ? K1_ST_TMA : K1_ST_CP, TMA>(
-        job_maps<2, TMA>(b.tm, k), j.If, j.J, j.SI, j.varI, j.coef, j.h, j.g.D, j.g.H, j.g.W,
-        j.g.P, j.g.TZ, b.bits, j.cc_eps, b.window, b.write_coef, bx, by, bz);
+template <int R, class A>
+__device__ __forceinline__ void window_tile(const A &a, int t, int &bx, int &by, int &bz) {
+    const int gx = (a.W + FX - 1) / FX, gy = (a.H + WinTile<R>::TY - 1) / WinTile<R>::TY;
+    bx = t % gx;
+    const int r = t / gx;
+    by = r % gy;
+    bz = r / gy;
 }
 
-template <int R, bool TMA>
-__global__ void __launch_bounds__(FX *K2_NW) k_lncc_grad_batch(const __grid_constant__ K2Batch b) {
+template <int R>
+__global__ void __launch_bounds__(WinTile<R>::NT, fwd_min_ctas(R, kFwdGiven))
+    k_lncc_fwd_batch(const __grid_constant__ K1Batch b) {
     const int k = batch_job(b.first, b.n, (int)blockIdx.x);
-    const K2Job &j = b.j[k];
     int bx, by, bz;
-    batch_tile(j.geo, (int)blockIdx.x - b.first[k], bx, by, bz);
-    lncc_grad_body<R, K2_NW, K2_OPT, TMA ? K2_ST_TMA : K2_ST_CP, TMA>(
-        job_maps<1, TMA>(b.tm, k), j.If, j.gJ, j.J, j.coef, j.h, j.g, j.geo.D, j.geo.H, j.geo.W,
-        j.geo.P, j.geo.TZ, b.cbits, bx, by, bz);
+    window_tile<R>(b.j[k], (int)blockIdx.x - b.first[k], bx, by, bz);
+    lncc_fwd_body<R, kFwdGiven>(b.j[k], bx, by, bz);
+}
+
+template <int R>
+__global__ void __launch_bounds__(WinTile<R>::NT, grad_min_ctas(R))
+    k_lncc_grad_batch(const __grid_constant__ K2Batch b) {
+    const int k = batch_job(b.first, b.n, (int)blockIdx.x);
+    int bx, by, bz;
+    window_tile<R>(b.j[k], (int)blockIdx.x - b.first[k], bx, by, bz);
+    lncc_grad_body<R, false>(b.j[k], bx, by, bz);
 }
 
 template <class TS>
@@ -186,10 +175,10 @@ __global__ void __launch_bounds__(FX *K4B_NW, 2) k_compose_batch(
 // own depth), minimising (waves x planes per CTA) over the whole launch, whose
 // CTAs fill the GPU's resident slots together.  A coarse level of many jobs
 // then takes short slabs (more CTAs), a fine level long ones (less halo).
-int launch_tz(const Dims *d, int n, int ty, int halo, int occ) {
+int launch_tz(const Dims *d, int n, int ty, float extra, int occ) {
     const long long slots = (long long)num_sms() * (occ > 0 ? occ : 1);
     int best = 64;
-    long long bestcost = -1;
+    float bestcost = -1.0f;
     for (int tz = 1; tz <= 64; ++tz) {
         long long ctas = 0;
         for (int k = 0; k < n; ++k) {
@@ -197,8 +186,8 @@ int launch_tz(const Dims *d, int n, int ty, int halo, int occ) {
             const int t = tz < d[k].D ? tz : d[k].D;
             ctas += txy * ((d[k].D + t - 1) / t);
         }
-        const long long cost = (ctas + slots - 1) / slots * (tz + 2 * halo);
-        if (bestcost < 0 || cost < bestcost) {
+        const float cost = (float)((ctas + slots - 1) / slots) * ((float)tz + extra);
+        if (bestcost < 0.0f || cost < bestcost) {
             bestcost = cost;
             best = tz;
         }
@@ -219,8 +208,6 @@ int batch_geom(BGeom &g, Dims d, int ty, int tz) {
     return g.gx * g.gy * ((d.D + g.TZ - 1) / g.TZ);
 }
 
-BGeom *geom_of(K1Job &j) { return &j.g; }
-BGeom *geom_of(K2Job &j) { return &j.geo; }
 BGeom *geom_of(K3Job &j) { return &j.geo; }
 BGeom *geom_of(K4Job &j) { return &j.geo; }
 
@@ -243,7 +230,7 @@ template <class B>
 void batch_layout(B &b, const LockstepJob *jobs, const int *idx, int ty, int halo, int occ) {
     Dims dd[kMaxLockstepJobs];
     for (int k = 0; k < b.n; ++k) dd[k] = jobs[idx[k]].d;
-    const int tz = launch_tz(dd, b.n, ty, halo, occ);
+    const int tz = launch_tz(dd, b.n, ty, 2.0f * halo, occ);
     b.first[0] = 0;
     for (int k = 0; k < b.n; ++k) {
         BGeom &g = *geom_of(b.j[k]);
@@ -251,47 +238,51 @@ void batch_layout(B &b, const LockstepJob *jobs, const int *idx, int ty, int hal
     }
 }
 
-template <int R>
-cudaError_t launch_k1_batch(K1Batch &b, const LockstepJob *jobs, const int *idx, cudaStream_t s) {
-    using ST = K1S<R, K1_NW, K1_OPT, K1_ST_TMA>;
-    bool tma = true;
-    for (int k = 0; k < b.n && tma; ++k) {
-        const LockstepJob &q = jobs[idx[k]];
-        tma = tmap(&b.tm[2 * k], q.If, 4, q.d, 1, ST::BXW, ST::RY, 1) &&
-              tmap(&b.tm[2 * k + 1], q.fb->J, 4, q.d, 1, ST::BXW, ST::RY, 1);
+// Grid and slab depth of every job of a K1 or K2 launch.
+template <int R, class B>
+void window_layout(B &b, const LockstepJob *jobs, int occ) {
+    using G = WinTile<R>;
+    Dims dd[kMaxLockstepJobs];
+    for (int k = 0; k < b.n; ++k) dd[k] = jobs[k].d;
+    const int tz = launch_tz(dd, b.n, G::TY, window_slab_extra(R), occ);
+    b.first[0] = 0;
+    for (int k = 0; k < b.n; ++k) {
+        auto &a = b.j[k];
+        a.D = dd[k].D;
+        a.H = dd[k].H;
+        a.W = dd[k].W;
+        a.P = dd[k].pitch();
+        a.TZ = tz < a.D ? tz : a.D;
+        b.first[k + 1] = b.first[k] + (a.W + FX - 1) / FX * ((a.H + G::TY - 1) / G::TY) *
+                                          ((a.D + a.TZ - 1) / a.TZ);
     }
-    if (tma) {
-        auto kern = k_lncc_fwd_batch<R, true>;
-        static const int occ = prepare(kern, ST::bytes, ST::NT);
-        batch_layout(b, jobs, idx, ST::TY, R, occ);
-        return launch_batch(kern, b, ST::NT / FX, ST::bytes, s);
-    }
-    using SC = K1S<R, K1_NW, K1_OPT, K1_ST_CP>;
-    auto kern = k_lncc_fwd_batch<R, false>;
-    static const int occ = prepare(kern, SC::bytes, SC::NT);
-    batch_layout(b, jobs, idx, SC::TY, R, occ);
-    return launch_batch(kern, b, SC::NT / FX, SC::bytes, s);
+}
+
+template <class K, class B>
+cudaError_t launch_window_batch(K kern, const B &b, int threads, size_t smem, cudaStream_t s) {
+    LaunchGeom g;
+    g.grid = dim3((unsigned)b.first[b.n]);
+    g.block = dim3(threads);
+    g.tz = 0;
+    return launch_pdl(kern, g, smem, s, b);
 }
 
 template <int R>
-cudaError_t launch_k2_batch(K2Batch &b, const LockstepJob *jobs, const int *idx, cudaStream_t s) {
-    using ST = K2S<R, K2_NW, K2_OPT, K2_ST_TMA>;
-    bool tma = true;
-    for (int k = 0; k < b.n && tma; ++k) {
-        const LockstepJob &q = jobs[idx[k]];
-        tma = tmap(&b.tm[k], q.fb->coef, 4, q.d, 4, ST::BXW, ST::RY, 4);
-    }
-    if (tma) {
-        auto kern = k_lncc_grad_batch<R, true>;
-        static const int occ = prepare(kern, ST::bytes, ST::NT);
-        batch_layout(b, jobs, idx, ST::TY, R, occ);
-        return launch_batch(kern, b, ST::NT / FX, ST::bytes, s);
-    }
-    using SC = K2S<R, K2_NW, K2_OPT, K2_ST_CP>;
-    auto kern = k_lncc_grad_batch<R, false>;
-    static const int occ = prepare(kern, SC::bytes, SC::NT);
-    batch_layout(b, jobs, idx, SC::TY, R, occ);
-    return launch_batch(kern, b, SC::NT / FX, SC::bytes, s);
+cudaError_t launch_k1_batch(K1Batch &b, const LockstepJob *jobs, cudaStream_t s) {
+    constexpr size_t smem = FwdSmem<R, kFwdGiven>::bytes;
+    auto kern = k_lncc_fwd_batch<R>;
+    static const int occ = prepare(kern, smem, WinTile<R>::NT);
+    window_layout<R>(b, jobs, occ);
+    return launch_window_batch(kern, b, WinTile<R>::NT, smem, s);
+}
+
+template <int R>
+cudaError_t launch_k2_batch(K2Batch &b, const LockstepJob *jobs, cudaStream_t s) {
+    constexpr size_t smem = GradTile<R>::bytes;
+    auto kern = k_lncc_grad_batch<R>;
+    static const int occ = prepare(kern, smem, WinTile<R>::NT);
+    window_layout<R>(b, jobs, occ);
+    return launch_window_batch(kern, b, WinTile<R>::NT, smem, s);
 }
 
 template <int RG, class TS>
@@ -358,32 +349,32 @@ cudaError_t launch_k4_batch(K4Batch<SU ? 2 : 1> &b, const LockstepJob *jobs, con
         return call;          \
     }
 
-cudaError_t dispatch_k1_batch(int R, K1Batch &b, const LockstepJob *jobs, const int *idx,
+cudaError_t dispatch_k1_batch(int R, K1Batch &b, const LockstepJob *jobs,
                               cudaStream_t s) {
     switch (R) {
-        FA_CASE(0, launch_k1_batch<RR>(b, jobs, idx, s))
-        FA_CASE(1, launch_k1_batch<RR>(b, jobs, idx, s))
-        FA_CASE(2, launch_k1_batch<RR>(b, jobs, idx, s))
-        FA_CASE(3, launch_k1_batch<RR>(b, jobs, idx, s))
-        FA_CASE(4, launch_k1_batch<RR>(b, jobs, idx, s))
-        FA_CASE(5, launch_k1_batch<RR>(b, jobs, idx, s))
-        FA_CASE(6, launch_k1_batch<RR>(b, jobs, idx, s))
-        FA_CASE(7, launch_k1_batch<RR>(b, jobs, idx, s))
+        FA_CASE(0, launch_k1_batch<RR>(b, jobs, s))
+        FA_CASE(1, launch_k1_batch<RR>(b, jobs, s))
+        FA_CASE(2, launch_k1_batch<RR>(b, jobs, s))
+        FA_CASE(3, launch_k1_batch<RR>(b, jobs, s))
+        FA_CASE(4, launch_k1_batch<RR>(b, jobs, s))
+        FA_CASE(5, launch_k1_batch<RR>(b, jobs, s))
+        FA_CASE(6, launch_k1_batch<RR>(b, jobs, s))
+        FA_CASE(7, launch_k1_batch<RR>(b, jobs, s))
     }
     return cudaErrorInvalidValue;
 }
 
-cudaError_t dispatch_k2_batch(int R, K2Batch &b, const LockstepJob *jobs, const int *idx,
+cudaError_t dispatch_k2_batch(int R, K2Batch &b, const LockstepJob *jobs,
                               cudaStream_t s) {
     switch (R) {
-        FA_CASE(0, launch_k2_batch<RR>(b, jobs, idx, s))
-        FA_CASE(1, launch_k2_batch<RR>(b, jobs, idx, s))
-        FA_CASE(2, launch_k2_batch<RR>(b, jobs, idx, s))
-        FA_CASE(3, launch_k2_batch<RR>(b, jobs, idx, s))
-        FA_CASE(4, launch_k2_batch<RR>(b, jobs, idx, s))
-        FA_CASE(5, launch_k2_batch<RR>(b, jobs, idx, s))
-        FA_CASE(6, launch_k2_batch<RR>(b, jobs, idx, s))
-        FA_CASE(7, launch_k2_batch<RR>(b, jobs, idx, s))
+        FA_CASE(0, launch_k2_batch<RR>(b, jobs, s))
+        FA_CASE(1, launch_k2_batch<RR>(b, jobs, s))
+        FA_CASE(2, launch_k2_batch<RR>(b, jobs, s))
+        FA_CASE(3, launch_k2_batch<RR>(b, jobs, s))
+        FA_CASE(4, launch_k2_batch<RR>(b, jobs, s))
+        FA_CASE(5, launch_k2_batch<RR>(b, jobs, s))
+        FA_CASE(6, launch_k2_batch<RR>(b, jobs, s))
+        FA_CASE(7, launch_k2_batch<RR>(b, jobs, s))
     }
     return cudaErrorInvalidValue;
 }
@@ -478,38 +469,41 @@ fa_status fused_iteration_lockstep(int n, const LockstepJob *jobs, int t, cudaSt
     {
         K1Batch b;
         b.n = n;
-        b.bits = lncc_image_bits(p0->window);
-        b.window = p0->window;
-        b.write_coef = 1;
         for (int k = 0; k < n; ++k) {
             const LockstepJob &q = jobs[k];
-            K1Job &j = b.j[k];
-            j.If = q.If;
-            j.J = q.fb->J;
-            j.SI = q.fb->sI;
-            j.varI = q.fb->varI;
-            j.coef = q.fb->coef;
-            j.h = q.h;
-            j.cc_eps = q.p->cc_eps;
+            FwdArgs a{};
+            a.I = q.If;
+            a.J = q.fb->J;
+            a.SI = q.fb->sI;
+            a.varI = q.fb->varI;
+            a.coef = q.fb->coef;
+            a.h = q.h;
+            a.bits = lncc_image_bits(p0->window);
+            a.window = p0->window;
+            a.cc_eps = q.p->cc_eps;
+            a.write_coef = 1;
+            b.j[k] = a;
         }
-        FA_CUDA_TRY(dispatch_k1_batch(R, b, jobs, idx, s));
+        FA_CUDA_TRY(dispatch_k1_batch(R, b, jobs, s));
         note_launch();
     }
     {
         K2Batch b;
         b.n = n;
-        b.cbits = lncc_coef_bits(p0->window);
         for (int k = 0; k < n; ++k) {
             const LockstepJob &q = jobs[k];
-            K2Job &j = b.j[k];
-            j.If = q.If;
-            j.gJ = q.fb->gJ;
-            j.J = q.fb->J;
-            j.coef = q.fb->coef;
-            j.g = q.fb->g;
-            j.h = q.h;
+            GradArgs a{};
+            a.I = q.If;
+            a.J = q.fb->J;
+            a.gJ = q.fb->gJ;
+            a.coef = q.fb->coef;
+            a.h = q.h;
+            a.g = q.fb->g;
+            a.cbits = lncc_coef_bits(p0->window);
+            a.n = p0->window * p0->window * p0->window;
+            b.j[k] = a;
         }
-        FA_CUDA_TRY(dispatch_k2_batch(R, b, jobs, idx, s));
+        FA_CUDA_TRY(dispatch_k2_batch(R, b, jobs, s));
         note_launch();
     }
     const AdamConsts ac = adam_consts(p0, t);

@@ -19,8 +19,10 @@
 // adjoint window sums need A, B, C around every output, so K2 cannot join K1
 // without recomputing a much wider halo.
 //
-// Every kernel marches along z ("2.5-D" tiling): a CTA owns a 32 x TY tile of
-// (x, y) columns and a slab of TZ output planes.  A plane's inputs (the tile
+// K1 and K2 are in window.cuh; K3 and K4 are here.
+//
+// Every kernel marches along z ("2.5-D" tiling).  In K3 and K4 a CTA owns a
+// 32 x TY tile of (x, y) columns and a slab of TZ output planes.  A plane's inputs (the tile
 // plus its halo, and the operands of the plane's outputs) arrive NSTG - 1
 // planes ahead of use.  When the buffers' rows start on 16-byte boundaries
 // (a registration pads its levels' rows to a multiple of 4 floats) they come
@@ -45,18 +47,15 @@
 #include <type_traits>
 #include <math.h>
 
-#include <map>
-#include <mutex>
-
+#include "launch.cuh"
 #include "register.h"
 #include "validate.h"
+#include "window.cuh"
 
 namespace fa {
 
 namespace {
 
-
-constexpr int FX = 32;  // tile width along x (one warp)
 
 __host__ __device__ constexpr int halo4(int r) { return (r + 3) / 4 * 4; }
 __host__ __device__ constexpr size_t al128(size_t b) { return (b + 127) & ~size_t(127); }
@@ -154,17 +153,6 @@ __device__ __forceinline__ MapRef map_ref(const Maps &m) { return MapRef{&m.a, &
 // false when the field does not meet TMA's alignment rules.
 bool tmap(CUtensorMap *m, const void *base, int esize, Dims d, int C, int bx, int by, int bc);
 namespace {
-
-// Programmatic dependent launch: the fused kernels are launched so that a
-// kernel's CTAs may start while the previous kernel in the stream finishes.
-// Everything before pdl_wait() touches no data the previous kernel writes;
-// pdl_wait() returns once that kernel has completed and its writes are
-// visible.  pdl_trigger() lets the next kernel begin launching once every
-// CTA of this one has started.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
-__device__ __forceinline__ void pdl_trigger() {
-    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-}
 
 // For a CTA that has waited for the previous kernel (pdl_wait) and issued its
 // first copies and header loads (so that they are in flight while the status
@@ -311,117 +299,6 @@ __device__ __forceinline__ void gauss_x4(const float *pl, float *xb, const TT &t
     }
 }
 
-// Sliding window sums of 4 adjacent outputs from 4 + 2R values.
-template <int R, class T>
-__device__ __forceinline__ void slide4(const T *p, T s[4]) {
-    T a = 0;
-#pragma unroll
-    for (int t = 0; t <= 2 * R; ++t) a += p[t];
-    s[0] = a;
-#pragma unroll
-    for (int jj = 1; jj < 4; ++jj) {
-        a += p[2 * R + jj] - p[jj - 1];
-        s[jj] = a;
-    }
-}
-
-__device__ __forceinline__ void store_ll4(long long *d, const long long s[4]) {
-    ((longlong2 *)d)[0] = make_longlong2(s[0], s[1]);
-    ((longlong2 *)d)[1] = make_longlong2(s[2], s[3]);
-}
-
-// LNCC forward x pass on quantised planes qI, qJ [RY][BXW] (int32) ->
-// xL [3][RY][FX] int64: channel 0 sum J, 1 sum J^2, 2 sum I J.
-template <int R, int RY, int BXW, int COFF, int NT>
-__device__ __forceinline__ void box_x4_fwd(const int *qI, const int *qJ, long long *xL, int tid) {
-    constexpr int ITEMS = 3 * RY * 8, NL = (4 + COFF + 2 * R + 3) / 4, NV = 4 + 2 * R;
-    static_assert(28 + 4 * NL <= BXW, "row too short for the vector loads");
-#pragma unroll
-    for (int j = 0; j < (ITEMS + NT - 1) / NT; ++j) {
-        const int it = tid + j * NT;
-        if (ITEMS % NT != 0 && it >= ITEMS) break;
-        const int k = it & 7, rest = it >> 3, ry = rest % RY, c = rest / RY;
-        int vj[4 * NL], vi[4 * NL];
-        const int4 *sj = (const int4 *)(qJ + ry * BXW + 4 * k);
-#pragma unroll
-        for (int l = 0; l < NL; ++l) {
-            const int4 q = sj[l];
-            vj[4 * l] = q.x;
-            vj[4 * l + 1] = q.y;
-            vj[4 * l + 2] = q.z;
-            vj[4 * l + 3] = q.w;
-        }
-        long long out[4];
-        if (c == 0) {
-            int s4[4];
-            slide4<R, int>(vj + COFF, s4);
-#pragma unroll
-            for (int jj = 0; jj < 4; ++jj) out[jj] = s4[jj];
-        } else {
-            if (c == 2) {
-                const int4 *si = (const int4 *)(qI + ry * BXW + 4 * k);
-#pragma unroll
-                for (int l = 0; l < NL; ++l) {
-                    const int4 q = si[l];
-                    vi[4 * l] = q.x;
-                    vi[4 * l + 1] = q.y;
-                    vi[4 * l + 2] = q.z;
-                    vi[4 * l + 3] = q.w;
-                }
-            } else {
-#pragma unroll
-                for (int l = 0; l < 4 * NL; ++l) vi[l] = vj[l];
-            }
-            long long pr[NV];
-#pragma unroll
-            for (int tt = 0; tt < NV; ++tt) pr[tt] = (long long)vi[tt + COFF] * vj[tt + COFF];
-            slide4<R, long long>(pr, out);
-        }
-        store_ll4(xL + (c * RY + ry) * FX + 4 * k, out);
-    }
-}
-
-// LNCC adjoint x pass on quantised coefficients q [3][RY][BXW] (int64) ->
-// xL [3][RY][FX].
-template <int R, int RY, int BXW, int COFF, int NT>
-__device__ __forceinline__ void box_x4_adj(const long long *q, long long *xL, int tid) {
-    constexpr int ITEMS = 3 * RY * 8, NL = (4 + COFF + 2 * R + 1) / 2;
-    static_assert(28 + 2 * NL <= BXW, "row too short for the vector loads");
-#pragma unroll
-    for (int j = 0; j < (ITEMS + NT - 1) / NT; ++j) {
-        const int it = tid + j * NT;
-        if (ITEMS % NT != 0 && it >= ITEMS) break;
-        const int k = it & 7, rest = it >> 3, ry = rest % RY, c = rest / RY;
-        const longlong2 *src = (const longlong2 *)(q + (c * RY + ry) * BXW + 4 * k);
-        long long v[2 * NL];
-#pragma unroll
-        for (int l = 0; l < NL; ++l) {
-            const longlong2 a = src[l];
-            v[2 * l] = a.x;
-            v[2 * l + 1] = a.y;
-        }
-        long long out[4];
-        slide4<R, long long>(v + COFF, out);
-        store_ll4(xL + (c * RY + ry) * FX + 4 * k, out);
-    }
-}
-
-// y pass of this thread's outputs from xL [C][RY][FX].
-template <int R, int RY, int NW, int OPT>
-__device__ __forceinline__ void box_y3(const long long *xL, int wy, int tx, long long P[OPT][3]) {
-#pragma unroll
-    for (int o = 0; o < OPT; ++o) {
-        const long long *xi = xL + (wy + NW * o) * FX + tx;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            long long sum = 0;
-#pragma unroll
-            for (int t = 0; t <= 2 * R; ++t) sum += xi[c * RY * FX + t * FX];
-            P[o][c] = sum;
-        }
-    }
-}
-
 // Channels 0 and 1 of the y and z passes run as one packed FP32 pair
 // (__ffma2_rn: each component is exactly fmaf), channel 2 alone; every
 // channel's taps accumulate in the same order as a scalar loop would.
@@ -444,21 +321,6 @@ __device__ __forceinline__ void gauss_y3(const float *xb, const TT &t, int wy, i
         Q[o][1] = s01.y;
         Q[o][2] = s2;
     }
-}
-
-// Running z window sums: ring of the last NS plane results per output.
-template <int NS, int OPT, int NOUT, int NT>
-__device__ __forceinline__ void zslide(long long *ring, int slot, int tid,
-                                       const long long P[OPT][3], long long acc[OPT][3]) {
-    long long *rb = ring + slot * 3 * NOUT + tid;
-#pragma unroll
-    for (int o = 0; o < OPT; ++o)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            long long *r = rb + c * NOUT + o * NT;
-            acc[o][c] += P[o][c] - *r;
-            *r = P[o][c];
-        }
 }
 
 // Ring of the last NS in-plane results of this thread's outputs, [NS][3][NOUT]
@@ -498,455 +360,6 @@ __device__ __forceinline__ void gauss_z3(const float *ring_o, int newest, const 
 template <int NSTG>
 __device__ __forceinline__ void drain(unsigned long long *bar, int i, int np) {
     for (int j = i; j < i + NSTG && j < np; ++j) mbar_wait(bar + j % NSTG, (unsigned)(j / NSTG) & 1u);
-}
-
-// ====================================================================== K1
-template <int R, int NW, int OPT, int NSTG>
-struct K1S {
-    static constexpr int NT = FX * NW, TY = NW * OPT, RX = FX + 2 * R, RY = TY + 2 * R;
-    static constexpr int XB = halo4(R), BXW = FX + 2 * XB, COFF = XB - R;
-    static constexpr int NR = BXW * RY, NS = 2 * R + 1, NOUT = NT * OPT;
-    static constexpr size_t plane = al128((size_t)NR * 4);  // I_f plane, then J plane
-    static constexpr size_t st_bytes = 2 * plane;
-    static constexpr unsigned tx_plane = 2u * NR * 4;
-    static constexpr size_t o_st = 0;
-    static constexpr size_t o_ring = o_st + st_bytes * NSTG;             // [NS][3][NOUT] int64
-    static constexpr size_t o_xL = o_ring + (size_t)NS * 3 * NOUT * 8;   // [3][RY][FX] int64
-    static constexpr size_t o_q = o_xL + (size_t)3 * RY * FX * 8;        // [2][RY][BXW] int32
-    static constexpr size_t o_bar = al128(o_q + (size_t)2 * NR * 4);
-    static constexpr size_t bytes = o_bar + 8 * NSTG;
-};
-
-// K1's output voxel from its window sums acc = (S_J, S_JJ, S_IJ) and the
-// fixed image's S_I (a1) and variance: cc into the loss sum qcc (bad when cc
-// leaves [0, 2]), and with write_coef the adjoint coefficients A, B and C
-// (float-float) at cp[0], cp[N], cp[2N], cp[3N] with their running maxima.
-__device__ __forceinline__ void lncc_fwd_output(const long long acc[3], long long a1, float varI,
-                                                long long n, float nf, float inv_nf, float inv_s,
-                                                float cc_eps, int write_coef, float *cp,
-                                                long long N, unsigned long long &qcc, bool &bad,
-                                                float &mA, float &mB, float &mC) {
-    const long long a2 = acc[0];
-    const float varJ = diff_i128_to_float(n, acc[1], a2, a2) * inv_s * inv_s * inv_nf;
-    const float cross = diff_i128_to_float(n, acc[2], a1, a2) * inv_s * inv_s * inv_nf;
-    const float den = fmaf(varI, varJ, cc_eps);
-    const float rden = __frcp_rn(den);
-    const float cc = cross * cross * rden;
-    if (cc >= 0.0f && cc <= 2.0f)
-        qcc += (unsigned long long)quantize(cc, 4294967296.0f);  // cc in [0, 2]
-    else
-        bad = true;
-    if (write_coef) {
-        const float A = 2.0f * cross * rden;
-        const float B = -cc * varI * rden;
-        float Ch, Cl;
-        lncc_c_ff(A, B, a1, a2, inv_s, nf, inv_nf, Ch, Cl);
-        cp[0] = A;
-        cp[N] = B;
-        cp[2 * N] = Ch;
-        cp[3 * N] = Cl;
-        mA = fmaxf(mA, fabsf(A));
-        mB = fmaxf(mB, fabsf(B));
-        mC = fmaxf(mC, fabsf(Ch));
-    }
-}
-
-// The body of K1 for the CTA with tile coordinates (bx, by, bz).
-template <int R, int NW, int OPT, int NSTG, bool TMA>
-__device__ __forceinline__ void lncc_fwd_body(MapRef maps, const float *__restrict__ If,
-                                              const float *__restrict__ J,
-                                              const long long *__restrict__ SIg,
-                                              const float *__restrict__ varIg,
-                                              float *__restrict__ coef, WsHeader *__restrict__ h,
-                                              int D, int H, int W, int P, int TZ, int bits,
-                                              float cc_eps,
-                                              int window, int write_coef, int bx, int by, int bz) {
-    using S = K1S<R, NW, OPT, NSTG>;
-    constexpr int NT = S::NT, TY = S::TY, RX = S::RX, RY = S::RY, BXW = S::BXW, COFF = S::COFF,
-                  XB = S::XB, NR = S::NR, NS = S::NS, NOUT = S::NOUT;
-    constexpr int CS = (int)(S::plane / 4);
-    using G = Region<RY, RX, NW, BXW, COFF>;
-    extern __shared__ __align__(128) unsigned char smem[];
-    long long *ring = (long long *)(smem + S::o_ring);
-    long long *xL = (long long *)(smem + S::o_xL);
-    int *qI = (int *)(smem + S::o_q), *qJ = qI + NR;
-    unsigned long long *bar = (unsigned long long *)(smem + S::o_bar);
-    __shared__ float redf[32];
-    __shared__ unsigned long long redu[32];
-    __shared__ int flag;
-    auto stage = [&](int s) { return (float *)(smem + S::o_st + S::st_bytes * s); };
-
-    const int tx = threadIdx.x, wy = threadIdx.y, tid = wy * FX + tx;
-    const int x0 = bx * FX, y0 = by * TY, z0 = bz * TZ;
-    const int zend = min(z0 + TZ, D);
-    const long long N = (long long)D * H * P, HW = (long long)H * P;  // channel, plane strides
-    const long long n = (long long)window * window * window;
-    const float nf = (float)n, inv_nf = 1.0f / nf;
-    G rg;
-    if (!TMA) rg.init(wy, tx, y0 - R, x0 - R, H, W, P);
-    Outs<OPT, NW> ou;
-    ou.init(wy, tx, y0, x0, H, W, P);
-    if (TMA && tid == 0) {
-        for (int k = 0; k < NSTG; ++k) mbar_init(bar + k);
-        mbar_init_fence();
-    }
-    for (int k = tid; k < NS * 3 * NOUT; k += NT) ring[k] = 0;
-
-    long long acc[OPT][3];
-#pragma unroll
-    for (int o = 0; o < OPT; ++o)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) acc[o][c] = 0;
-
-    const int zs = z0 - R, np = zend - z0 + 2 * R;
-    auto issue = [&](int i) {
-        const int zp = zs + i, s = i % NSTG;
-        if (TMA) {
-            if (tid == 0 && i < np) {
-                mbar_expect(bar + s, S::tx_plane);
-                tma4(stage(s), maps.a, x0 - XB, y0 - R, zp, 0, bar + s);
-                tma4(stage(s) + CS, maps.b, x0 - XB, y0 - R, zp, 0, bar + s);
-            }
-        } else {
-            if (i < np) {
-                const bool zok = zp >= 0 && zp < D;
-                rg.template load<1>(stage(s), If, N, (long long)zp * HW, zok);
-                rg.template load<1>(stage(s) + CS, J, N, (long long)zp * HW, zok);
-            }
-            cp_commit();
-        }
-    };
-    // the outputs' operands S_I, var_I, loaded one plane ahead into registers
-    long long a1n[OPT][1];
-    float vIn[OPT][1];
-    auto fetch_ops = [&](int i) {
-        const int zo = zs + i - R;
-        if (i < np && zo >= z0 && zo < zend) {
-            ou.fetch(a1n, SIg, N, (long long)zo * HW);
-            ou.fetch(vIn, varIg, N, (long long)zo * HW);
-        }
-    };
-    // after the previous kernel: first copies, operands and header loads in
-    // flight together, then the status check
-    pdl_wait();
-    fetch_ops(0);
-#pragma unroll
-    for (int k = 0; k < NSTG - 1; ++k) issue(k);
-    const float amax =
-        fmaxf(__uint_as_float(h->absmax_bits[0]), __uint_as_float(h->absmax_bits[1]));
-    if (status_timed_out(h, tid, &flag)) {
-        drain_first<TMA, NSTG>(bar, np, tid);
-        return;
-    }
-    const int sh = fixed_shift(amax, bits);
-    const float scale = pow2f(sh), inv_s = pow2f(-sh);
-
-    unsigned long long qcc = 0;
-    float mA = 0.f, mB = 0.f, mC = 0.f;
-    bool bad = false;
-    int fail = -1, slot = 0;
-    for (int i = 0; i < np; ++i) {
-        const int zp = zs + i, z = zp - R, s = i % NSTG;
-        issue(i + NSTG - 1);
-        const bool out = z >= z0 && z < zend;
-        long long a1[OPT];
-        float vI[OPT];
-#pragma unroll
-        for (int o = 0; o < OPT; ++o) {
-            a1[o] = a1n[o][0];
-            vI[o] = vIn[o][0];
-        }
-        fetch_ops(i + 1);
-        bool ok = true;
-        if (TMA)
-            ok = mbar_wait(bar + s, (unsigned)(i / NSTG) & 1u);
-        else
-            cp_wait<NSTG - 1>();
-        const bool zin = zp >= 0 && zp < D;
-        if (zin) {
-            const float *sI = stage(s), *sJ = sI + CS;
-            if (TMA) {
-                for (int k = tid; k < NR; k += NT) {
-                    qI[k] = __float2int_rn(sI[k] * scale);
-                    qJ[k] = __float2int_rn(sJ[k] * scale);
-                }
-            } else {
-#pragma unroll
-                for (int j = 0; j < G::NJ; ++j)
-#pragma unroll
-                    for (int c = 0; c < G::NC; ++c) {  // own copies
-                        if (rg.off[j * G::NC + c] == -2) continue;
-                        const int k = rg.sbase + G::sofs(j, c);
-                        qI[k] = __float2int_rn(sI[k] * scale);
-                        qJ[k] = __float2int_rn(sJ[k] * scale);
-                    }
-            }
-        }
-        if (__syncthreads_or(!ok)) {
-            fail = i;
-            break;
-        }
-        long long P[OPT][3];
-        if (zin) {
-            box_x4_fwd<R, RY, BXW, COFF, NT>(qI, qJ, xL, tid);
-            __syncthreads();
-            box_y3<R, RY, NW, OPT>(xL, wy, tx, P);
-        } else {
-#pragma unroll
-            for (int o = 0; o < OPT; ++o)
-#pragma unroll
-                for (int c = 0; c < 3; ++c) P[o][c] = 0;
-        }
-        zslide<NS, OPT, NOUT, NT>(ring, slot, tid, P, acc);
-        slot = (slot + 1 == NS) ? 0 : slot + 1;
-        if (out) {
-            const long long zoff = (long long)z * HW;
-#pragma unroll
-            for (int o = 0; o < OPT; ++o) {
-                if (ou.off[o] < 0) continue;
-                lncc_fwd_output(acc[o], a1[o], vI[o], n, nf, inv_nf, inv_s, cc_eps, write_coef,
-                                coef + zoff + ou.off[o], N, qcc, bad, mA, mB, mC);
-            }
-        }
-    }
-    if (fail >= 0) {  // a tile copy never landed
-        if (tid == 0) {
-            status_set(&h->status, ST_TIMEOUT);
-            drain<NSTG>(bar, fail, np);
-        }
-        return;
-    }
-    if (!TMA) cp_wait<0>();
-    if (bad) status_set(&h->status, ST_NONFINITE);
-    block_sum_to(&h->loss_acc, qcc, redu);
-    if (write_coef) {
-        block_max_to(&h->coef_max_bits[0], mA, redf);
-        block_max_to(&h->coef_max_bits[1], mB, redf);
-        block_max_to(&h->coef_max_bits[2], mC, redf);
-    }
-}
-
-template <int R, int NW, int OPT, int NSTG, bool TMA>
-__global__ void __launch_bounds__(FX *NW) k_lncc_fwd(const __grid_constant__ Maps maps,
-                                                     const float *__restrict__ If,
-                                                     const float *__restrict__ J,
-                                                     const long long *__restrict__ SIg,
-                                                     const float *__restrict__ varIg,
-                                                     float *__restrict__ coef,
-                                                     WsHeader *__restrict__ h, int D, int H, int W,
-                                                     int P, int TZ, int bits, float cc_eps,
-                                                     int window, int write_coef) {
-    lncc_fwd_body<R, NW, OPT, NSTG, TMA>(map_ref(maps), If, J, SIg, varIg, coef, h, D, H, W, P, TZ, bits,
-                                         cc_eps, window, write_coef, blockIdx.x, blockIdx.y,
-                                         blockIdx.z);
-}
-
-// ====================================================================== K2
-// coef holds A, B and C as a float-float pair (C hi, C lo): [4][N].
-template <int R, int NW, int OPT, int NSTG>
-struct K2S {
-    static constexpr int NT = FX * NW, TY = NW * OPT, RX = FX + 2 * R, RY = TY + 2 * R;
-    static constexpr int XB = halo4(R), BXW = FX + 2 * XB, COFF = XB - R;
-    static constexpr int NR = BXW * RY, NS = 2 * R + 1, NOUT = NT * OPT;
-    static constexpr size_t st_bytes = al128((size_t)4 * NR * 4);    // A, B, C hi, C lo
-    static constexpr unsigned tx_plane = 4u * NR * 4;
-    static constexpr size_t o_st = 0;
-    static constexpr size_t o_ring = o_st + st_bytes * NSTG;
-    static constexpr size_t o_xL = o_ring + (size_t)NS * 3 * NOUT * 8;
-    static constexpr size_t o_q = o_xL + (size_t)3 * RY * FX * 8;
-    static constexpr size_t o_bar = al128(o_q + (size_t)3 * NR * 8);
-    static constexpr size_t bytes = o_bar + 8 * NSTG;
-};
-
-// The body of K2 for the CTA with tile coordinates (bx, by, bz).  WDJ: also
-// write dL/dJ itself to dJout (the adjoint's scatter into dL/dI_m needs it).
-template <int R, int NW, int OPT, int NSTG, bool TMA, bool WDJ = false>
-__device__ __forceinline__ void lncc_grad_body(MapRef maps, const float *__restrict__ If,
-                                               const float *__restrict__ gJ,
-                                               const float *__restrict__ J,
-                                               const float *__restrict__ coef,
-                                               WsHeader *__restrict__ h, float *__restrict__ g,
-                                               int D, int H, int W, int P, int TZ, int cbits,
-                                               int bx,
-                                               int by, int bz, float *__restrict__ dJout = nullptr) {
-    using S = K2S<R, NW, OPT, NSTG>;
-    constexpr int NT = S::NT, TY = S::TY, RX = S::RX, RY = S::RY, BXW = S::BXW, COFF = S::COFF,
-                  XB = S::XB, NR = S::NR, NS = S::NS, NOUT = S::NOUT;
-    using G = Region<RY, RX, NW, BXW, COFF>;
-    extern __shared__ __align__(128) unsigned char smem[];
-    long long *ring = (long long *)(smem + S::o_ring);
-    long long *xL = (long long *)(smem + S::o_xL);
-    long long *q = (long long *)(smem + S::o_q);
-    unsigned long long *bar = (unsigned long long *)(smem + S::o_bar);
-    __shared__ int flag;
-    auto stage = [&](int s) { return (float *)(smem + S::o_st + S::st_bytes * s); };
-
-    const int tx = threadIdx.x, wy = threadIdx.y, tid = wy * FX + tx;
-    const int x0 = bx * FX, y0 = by * TY, z0 = bz * TZ;
-    const int zend = min(z0 + TZ, D);
-    const long long N = (long long)D * H * P, HW = (long long)H * P;  // channel, plane strides
-    const float inv_n = 1.0f / (float)((long long)D * H * W);  // 1 / voxel count
-    G rg;
-    if (!TMA) rg.init(wy, tx, y0 - R, x0 - R, H, W, P);
-    Outs<OPT, NW> ou;
-    ou.init(wy, tx, y0, x0, H, W, P);
-    if (TMA && tid == 0) {
-        for (int k = 0; k < NSTG; ++k) mbar_init(bar + k);
-        mbar_init_fence();
-    }
-    for (int k = tid; k < NS * 3 * NOUT; k += NT) ring[k] = 0;
-    long long acc[OPT][3];
-#pragma unroll
-    for (int o = 0; o < OPT; ++o)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) acc[o][c] = 0;
-
-    const int zs = z0 - R, np = zend - z0 + 2 * R;
-    auto issue = [&](int i) {
-        const int zp = zs + i, s = i % NSTG;
-        if (TMA) {
-            if (tid == 0 && i < np) {
-                mbar_expect(bar + s, S::tx_plane);
-                tma4(stage(s), maps.a, x0 - XB, y0 - R, zp, 0, bar + s);
-            }
-        } else {
-            if (i < np)
-                rg.template load<4>(stage(s), coef, N, (long long)zp * HW, zp >= 0 && zp < D);
-            cp_commit();
-        }
-    };
-    // the outputs' operands grad I_m(phi), I_f, J, loaded one plane ahead
-    float gn[OPT][3], In[OPT][1], Jn[OPT][1];
-    auto fetch_ops = [&](int i) {
-        const int zo = zs + i - R;
-        if (i < np && zo >= z0 && zo < zend) {
-            ou.fetch(gn, gJ, N, (long long)zo * HW);
-            ou.fetch(In, If, N, (long long)zo * HW);
-            ou.fetch(Jn, J, N, (long long)zo * HW);
-        }
-    };
-    // after the previous kernel: first copies, operands and header loads in
-    // flight together, then the status check
-    pdl_wait();
-    fetch_ops(0);
-#pragma unroll
-    for (int k = 0; k < NSTG - 1; ++k) issue(k);
-    float cmax[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) cmax[c] = __uint_as_float(h->coef_max_bits[c]);
-    if (status_timed_out(h, tid, &flag)) {
-        drain_first<TMA, NSTG>(bar, np, tid);
-        return;
-    }
-    float qs[3], us[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const int e = fixed_shift(cmax[c], cbits);
-        qs[c] = pow2f(e);
-        us[c] = pow2f(-e);
-    }
-
-    int fail = -1, slot = 0;
-    for (int i = 0; i < np; ++i) {
-        const int zp = zs + i, zo = zp - R, s = i % NSTG;
-        issue(i + NSTG - 1);
-        const bool out = zo >= z0 && zo < zend;
-        float Gz[OPT], Gy[OPT], Gx[OPT], Iv[OPT], Jv[OPT];
-#pragma unroll
-        for (int k = 0; k < OPT; ++k) {
-            Gz[k] = gn[k][0];
-            Gy[k] = gn[k][1];
-            Gx[k] = gn[k][2];
-            Iv[k] = In[k][0];
-            Jv[k] = Jn[k][0];
-        }
-        fetch_ops(i + 1);
-        bool ok = true;
-        if (TMA)
-            ok = mbar_wait(bar + s, (unsigned)(i / NSTG) & 1u);
-        else
-            cp_wait<NSTG - 1>();
-        const bool zin = zp >= 0 && zp < D;
-        if (zin) {
-            const float *sp = stage(s);
-            auto quant = [&](int k) {
-                q[k] = quantize(sp[k], qs[0]);
-                q[NR + k] = quantize(sp[NR + k], qs[1]);
-                q[2 * NR + k] = quantize(sp[2 * NR + k], qs[2]) + quantize(sp[3 * NR + k], qs[2]);
-            };
-            if (TMA) {
-                for (int k = tid; k < NR; k += NT) quant(k);
-            } else {
-#pragma unroll
-                for (int j = 0; j < G::NJ; ++j)
-#pragma unroll
-                    for (int c = 0; c < G::NC; ++c) {  // own copies
-                        if (rg.off[j * G::NC + c] == -2) continue;
-                        quant(rg.sbase + G::sofs(j, c));
-                    }
-            }
-        }
-        if (__syncthreads_or(!ok)) {
-            fail = i;
-            break;
-        }
-        long long P[OPT][3];
-        if (zin) {
-            box_x4_adj<R, RY, BXW, COFF, NT>(q, xL, tid);
-            __syncthreads();
-            box_y3<R, RY, NW, OPT>(xL, wy, tx, P);
-        } else {
-#pragma unroll
-            for (int o = 0; o < OPT; ++o)
-#pragma unroll
-                for (int c = 0; c < 3; ++c) P[o][c] = 0;
-        }
-        zslide<NS, OPT, NOUT, NT>(ring, slot, tid, P, acc);
-        slot = (slot + 1 == NS) ? 0 : slot + 1;
-        if (out) {
-            const long long zoff = (long long)zo * HW;
-#pragma unroll
-            for (int o = 0; o < OPT; ++o) {
-                if (ou.off[o] < 0) continue;
-                float ah, al, bh, bl, ch, cl, rh, rl, th, tl;
-                i64_to_ff(acc[o][0], ah, al);
-                i64_to_ff(acc[o][1], bh, bl);
-                i64_to_ff(acc[o][2], ch, cl);
-                ff_mul_f(Iv[o], ah * us[0], al * us[0], rh, rl);      // I SA
-                ff_mul_f(2.0f * Jv[o], bh * us[1], bl * us[1], th, tl);  // 2 J SB
-                ff_add(rh, rl, th, tl);
-                ff_add(rh, rl, ch * us[2], cl * us[2]);               // + SC
-                const float dj = -(rh + rl) * inv_n;
-                float *gp = g + zoff + ou.off[o];
-                gp[0] = dj * Gz[o];
-                gp[N] = dj * Gy[o];
-                gp[2 * N] = dj * Gx[o];
-                if (WDJ) dJout[zoff + ou.off[o]] = dj;
-            }
-        }
-    }
-    if (fail >= 0) {
-        if (tid == 0) {
-            status_set(&h->status, ST_TIMEOUT);
-            drain<NSTG>(bar, fail, np);
-        }
-        return;
-    }
-    if (!TMA) cp_wait<0>();
-}
-
-template <int R, int NW, int OPT, int NSTG, bool TMA, bool WDJ = false>
-__global__ void __launch_bounds__(FX *NW) k_lncc_grad(const __grid_constant__ Maps maps,
-                                                      const float *__restrict__ If,
-                                                      const float *__restrict__ gJ,
-                                                      const float *__restrict__ J,
-                                                      const float *__restrict__ coef,
-                                                      WsHeader *__restrict__ h,
-                                                      float *__restrict__ g, int D, int H, int W,
-                                                      int P, int TZ, int cbits,
-                                                      float *__restrict__ dJout) {
-    lncc_grad_body<R, NW, OPT, NSTG, TMA, WDJ>(map_ref(maps), If, gJ, J, coef, h, g, D, H, W, P, TZ, cbits,
-                                               blockIdx.x, blockIdx.y, blockIdx.z, dJout);
 }
 
 // MSE: g = 2 (J - I) / N * grad I_m(phi) (pointwise, J and the gradient as
@@ -1512,62 +925,8 @@ __global__ void __launch_bounds__(FX *NW, NW >= 16 ? 2 : 1) k_compose(const __gr
 
 // ================================================================ launch helpers
 
-std::mutex g_mu;
-int g_num_sms = 0;
-
-int num_sms() {
-    std::lock_guard<std::mutex> lock(g_mu);
-    if (g_num_sms == 0) {
-        int dev = 0, n = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0)
-            g_num_sms = n;
-        else
-            g_num_sms = 152;
-    }
-    return g_num_sms;
-}
-
-// Opts the kernel into its dynamic shared memory and returns its resident
-// CTAs per SM (called once per kernel instantiation).
-template <class K>
-int prepare(K kernel, size_t smem, int threads) {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                         (int)cudaSharedmemCarveoutMaxShared);
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, smem) != cudaSuccess ||
-        n < 1)
-        n = 1;
-    return n;
-}
-
-struct LaunchGeom {
-    dim3 grid, block;
-    int tz;
-};
-
-// Launch with programmatic stream serialization (see pdl_wait).
-template <class... KArgs, class... Args>
-cudaError_t launch_pdl(void (*kern)(KArgs...), const LaunchGeom &g, size_t smem, cudaStream_t s,
-                       Args &&...args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = g.grid;
-    cfg.blockDim = g.block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
-}
-
 // tile shapes (warps per CTA, outputs per thread along y) and pipeline depths
 // of the TMA and of the cp.async variant
-constexpr int K1_NW = 8, K1_OPT = 1, K1_ST_TMA = 3, K1_ST_CP = 3;
-constexpr int K2_NW = 8, K2_OPT = 1, K2_ST_TMA = 2, K2_ST_CP = 2;
 constexpr int K3_NW = 8, K3_OPT = 1, K3_ST_TMA = 2, K3_ST_CP = 2;
 constexpr int K4_NW = 8, K4_OPT = 1, K4_ST_TMA = 2, K4_ST_CP = 2;
 

@@ -117,7 +117,8 @@ extern "C" fa_status fa_lncc_fwd_bwd_noalloc(const fa_vol *fixed, const fa_vol *
     const float *I = (const float *)fixed->data, *J = (const float *)warped->data;
     FA_CUDA_TRY(launch_header_reset(h, s));  // loss accumulator, maxima, status start at zero
     FA_CUDA_TRY(launch_absmax2(I, J, N, h, s));
-    FA_CUDA_TRY(launch_lncc_forward(I, J, d, window, cc_eps, dL_dfixed_opt != nullptr, h, b, s));
+    FA_CUDA_TRY(launch_lncc_forward(I, J, d, window, cc_eps, dL_dwarped_opt || dL_dfixed_opt,
+                                    dL_dfixed_opt != nullptr, h, b, s));
     FA_CUDA_TRY(launch_loss_finalize(h, N, -1.0f, loss_dev, s));
     if (dL_dwarped_opt || dL_dfixed_opt)
         FA_CUDA_TRY(launch_lncc_backward(

@@ -41,19 +41,56 @@ cudaError_t launch_compose_fields(const float *u, const float *delta, float *uo,
 cudaError_t launch_jac_direction(const float *gin, const float *u, float *gout, Dims d,
                                  cudaStream_t s);
 
+// ---- LNCC window sums (window.cuh has the kernels)
+// kFwdGiven: the fixed image's window sum and variance are given (constant
+//   over a level); sums of J, J^2, I J; writes A, B, C hi, C lo.
+// kFwdBoth: sums of I, J, I^2, J^2, I J; writes A, B, C and, with want_dI,
+//   B', C' (the coefficients of dL/dI).
+// kFwdStats: sums of I, I^2; writes the window sum and the variance.
+enum FwdMode { kFwdGiven, kFwdBoth, kFwdStats };
+struct FwdArgs {
+    const float *I, *J;
+    long long *SI;  // kFwdGiven: read; kFwdStats: written
+    float *varI;
+    float *coef;  // [4][N] (kFwdBoth with want_dI: [7][N])
+    WsHeader *h;
+    int D, H, W, P, TZ;
+    int bits, window;
+    float cc_eps;
+    int write_coef, want_dI;
+};
+// dL/dJ = -(1/N) [I SA + 2 J SB + SC]; the caller swaps the images for dL/dI,
+// whose coefficients A, B', C' are channels 0, 4, 5, 6.
+struct GradArgs {
+    const float *I, *J;
+    const float *gJ;    // grad I_m(phi), [3][N]; read where g is wanted
+    const float *coef;  // [4][N] or [7][N]
+    const WsHeader *h;
+    float *g, *dJ;  // dL/dJ times gJ, and dL/dJ (either may be NULL)
+    int D, H, W, P, TZ;
+    int cbits, n;
+};
+// Grid, pitch, window and slab depth (tz; 0: the cost model) are filled in.
+cudaError_t launch_window_fwd(FwdMode mode, FwdArgs g, Dims d, int window, int tz, cudaStream_t s);
+cudaError_t launch_window_grad(bool swap, GradArgs g, Dims d, int window, int tz, cudaStream_t s);
+
 // ---- plain LNCC / MSE (lncc.cu)
 // Header fields used: absmax_bits, coef_max_bits, loss_acc, status.
 struct LnccBuffers {
-    long long *p0, *p1;   // [5][N] int64 each
+    // [5][N] int64 each: part of the workspace sizes callers allocate by; the
+    // window sums stay on the chip, so only p0 is used, as scratch for a
+    // gradient that overlaps an input
+    long long *p0, *p1;
     float *coef;          // [7][N]: A, B, C hi, C lo, B', C' hi, C' lo
 };
 size_t lncc_plain_bytes(long long N);
 LnccBuffers lncc_carve(WsCarver &c, long long N);  // the plain-path scratch of an N-voxel grid
 cudaError_t launch_absmax2(const float *I, const float *J, long long N, WsHeader *h,
                            cudaStream_t s);
-// Forward: coefficients and loss accumulator.  want_dI selects B', C'.
+// Forward: loss accumulator and (want_coef) the coefficients; want_dI adds B', C'.
 cudaError_t launch_lncc_forward(const float *I, const float *J, Dims d, int window, float cc_eps,
-                                bool want_dI, WsHeader *h, LnccBuffers b, cudaStream_t s);
+                                bool want_coef, bool want_dI, WsHeader *h, LnccBuffers b,
+                                cudaStream_t s);
 // Backward: dJ = dL/dJ (may be NULL), dI = dL/dI (may be NULL),
 // g = dL/dJ * grad (3 channels, may be NULL; needs grad).
 cudaError_t launch_lncc_backward(const float *I, const float *J, const float *grad, Dims d,
@@ -90,11 +127,9 @@ cudaError_t launch_mi_range_set(const float *range4, MiBuffers b, cudaStream_t s
 cudaError_t launch_mi(const float *I, const float *J, const float *grad, Dims d, int bins,
                       WsHeader *h, MiBuffers b, float *loss_out, float *dJ, float *g,
                       cudaStream_t s);
-// Exact window sum S_I and rounded variance of the fixed image (p0, p1:
-// 2N int64 scratch each).
-cudaError_t launch_fixed_stats(const float *I, Dims d, int window, const WsHeader *h,
-                               long long *p0, long long *p1, long long *sI, float *varI,
-                               cudaStream_t s);
+// Exact window sum S_I and rounded variance of the fixed image.
+cudaError_t launch_fixed_stats(const float *I, Dims d, int window, WsHeader *h, long long *sI,
+                               float *varI, cudaStream_t s);
 // loss_out = sign * loss_acc * 2^-32 / N; also stored in h->loss.
 cudaError_t launch_loss_finalize(WsHeader *h, long long N, float sign, float *loss_out,
                                  cudaStream_t s);

@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(PT, 3) k_level_persistent(const __grid_constan
                     const long long a1 = __ldg(a.sI + vox), a2 = acc[0];
                     const float varI = __ldg(a.varI + vox);
                     const float varJ =
-                        diff_i128_to_float(n, acc[1], a2, a2) * inv_s * inv_s * inv_nf;
+                        diff_i128_to_float<true>(n, acc[1], a2, a2) * inv_s * inv_s * inv_nf;
                     const float cross =
                         diff_i128_to_float(n, acc[2], a1, a2) * inv_s * inv_s * inv_nf;
                     const float den = fmaf(varI, varJ, a.cc_eps);

@@ -238,7 +238,8 @@ static fa_status plain_iteration(Plan &P, const fa_params *p, int l, const float
     FA_CUDA_TRY(iter_reset(P.h, s));
     FA_CUDA_TRY(launch_warp(Im, u, P.J, P.grad, d, s));
     if (p->loss == FA_LOSS_LNCC) {
-        FA_CUDA_TRY(launch_lncc_forward(If, P.J, d, p->window, p->cc_eps, false, P.h, P.lb, s));
+        FA_CUDA_TRY(launch_lncc_forward(If, P.J, d, p->window, p->cc_eps, true, false, P.h, P.lb,
+                                        s));
         FA_CUDA_TRY(launch_lncc_backward(If, P.J, P.grad, d, p->window, P.h, P.lb, nullptr,
                                          nullptr, P.g, s));
     } else if (p->loss == FA_LOSS_MI) {
@@ -265,7 +266,8 @@ static fa_status final_loss(Plan &P, const fa_params *p, int l, const float *If,
         FA_CUDA_TRY(launch_warp(Im, u, P.J, nullptr, d, s));
     if (p->loss == FA_LOSS_LNCC) {
         if (p->mode == FA_MODE_PLAIN) {
-            FA_CUDA_TRY(launch_lncc_forward(If, P.J, d, p->window, p->cc_eps, false, P.h, P.lb, s));
+            FA_CUDA_TRY(launch_lncc_forward(If, P.J, d, p->window, p->cc_eps, false, false, P.h, P.lb,
+                                            s));
         } else {
             FA_CUDA_TRY(fused_lncc_forward_only(If, P.fb, d, p->window, p->cc_eps, P.h, s));
         }

@@ -32,7 +32,7 @@ fa_status fused_iteration(FusedBuffers &fb, WsHeader *h, const fa_params *p, Dim
 // (LNCC) and J = I_m o (id + u) with its gradient for the first iteration
 // (later iterations get both from the compose kernel).  Needs the level's image maxima in h.
 cudaError_t fused_level_start(const float *If, const float *Im, const float *u, Dims d,
-                              const fa_params *p, const WsHeader *h, FusedBuffers &fb,
+                              const fa_params *p, WsHeader *h, FusedBuffers &fb,
                               cudaStream_t s);
 // Measures candidate tile choices of the fused kernels on grid d (any
 // buffer contents) and records the fastest for later launches.

@@ -158,7 +158,8 @@ fa_status svf_eval(SvfWs &q, const fa_params *p, int steps, Dims d, const float 
     for (int k = 0; k < steps; ++k) FA_CUDA_TRY(launch_compose_fields(uk(k), uk(k), uk(k + 1), d, s));
     FA_CUDA_TRY(launch_warp(Im, uk(steps), q.J, grads ? q.grad : nullptr, d, s));
     if (p->loss == FA_LOSS_LNCC) {
-        FA_CUDA_TRY(launch_lncc_forward(If, q.J, d, p->window, p->cc_eps, false, q.h, q.lb, s));
+        FA_CUDA_TRY(launch_lncc_forward(If, q.J, d, p->window, p->cc_eps, grads, false, q.h, q.lb,
+                                        s));
         FA_CUDA_TRY(launch_loss_finalize(q.h, N, -1.0f, loss_dev, s));
         if (grads)
             FA_CUDA_TRY(launch_lncc_backward(If, q.J, q.grad, d, p->window, q.h, q.lb, nullptr,

@@ -113,7 +113,7 @@ fa_status sym_loss(SymWs &q, int loss, int window, float cc_eps, Dims d, const f
     FA_CUDA_TRY(launch_warp(If, uF, q.JF, grads ? q.gIF : nullptr, d, s));
     FA_CUDA_TRY(launch_warp(Im, uM, q.JM, grads ? q.gIM : nullptr, d, s));
     if (loss == FA_LOSS_LNCC) {
-        FA_CUDA_TRY(launch_lncc_forward(q.JF, q.JM, d, window, cc_eps, grads, q.h, q.lb, s));
+        FA_CUDA_TRY(launch_lncc_forward(q.JF, q.JM, d, window, cc_eps, grads, grads, q.h, q.lb, s));
         FA_CUDA_TRY(launch_loss_finalize(q.h, N, -1.0f, loss_dev, s));
         if (grads)
             FA_CUDA_TRY(launch_lncc_backward(q.JF, q.JM, q.gIM, d, window, q.h, q.lb, nullptr,

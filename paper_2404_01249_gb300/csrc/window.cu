@@ -1,0 +1,95 @@
+// Launches of the LNCC window-sum kernels (window.cuh) over one grid.
+#include "launch.cuh"
+#include "window.cuh"
+
+namespace fa {
+
+namespace {
+
+template <int R>
+LaunchGeom window_geom(Dims d, int tz, int occ) {
+    using G = WinTile<R>;
+    LaunchGeom g;
+    const int gx = (d.W + FX - 1) / FX, gy = (d.H + G::TY - 1) / G::TY;
+    g.tz = tz > 0 ? (tz < d.D ? tz : d.D) : choose_tz(d.D, gx * gy, window_slab_extra(R), occ);
+    g.grid = dim3(gx, gy, (d.D + g.tz - 1) / g.tz);
+    g.block = dim3(G::NT);
+    return g;
+}
+
+template <int R, FwdMode M>
+cudaError_t fwd(FwdArgs &a, Dims d, int tz, cudaStream_t s) {
+    using S = FwdSmem<R, M>;
+    auto kern = k_lncc_fwd<R, M>;
+    static const int occ = prepare(kern, S::bytes, WinTile<R>::NT);
+    const LaunchGeom g = window_geom<R>(d, tz, occ);
+    a.TZ = g.tz;
+    return launch_pdl(kern, g, S::bytes, s, a);
+}
+
+template <int R, bool SWAP>
+cudaError_t grad(GradArgs &a, Dims d, int tz, cudaStream_t s) {
+    using S = GradTile<R>;
+    auto kern = k_lncc_grad<R, SWAP>;
+    static const int occ = prepare(kern, S::bytes, WinTile<R>::NT);
+    const LaunchGeom g = window_geom<R>(d, tz, occ);
+    a.TZ = g.tz;
+    return launch_pdl(kern, g, S::bytes, s, a);
+}
+
+template <int R>
+cudaError_t fwd_mode(FwdMode m, FwdArgs &a, Dims d, int tz, cudaStream_t s) {
+    switch (m) {
+        case kFwdGiven: return fwd<R, kFwdGiven>(a, d, tz, s);
+        case kFwdBoth: return fwd<R, kFwdBoth>(a, d, tz, s);
+        case kFwdStats: return fwd<R, kFwdStats>(a, d, tz, s);
+    }
+    return cudaErrorInvalidValue;
+}
+
+template <class A>
+void fill_grid(A &a, Dims d) {
+    a.D = d.D;
+    a.H = d.H;
+    a.W = d.W;
+    a.P = d.pitch();
+}
+
+}  // namespace
+
+#define FA_EACH_R(call)                                \
+    switch (window / 2) {                              \
+        case 0: { constexpr int RR = 0; e = call; break; } \
+        case 1: { constexpr int RR = 1; e = call; break; } \
+        case 2: { constexpr int RR = 2; e = call; break; } \
+        case 3: { constexpr int RR = 3; e = call; break; } \
+        case 4: { constexpr int RR = 4; e = call; break; } \
+        case 5: { constexpr int RR = 5; e = call; break; } \
+        case 6: { constexpr int RR = 6; e = call; break; } \
+        case 7: { constexpr int RR = 7; e = call; break; } \
+    }
+
+cudaError_t launch_window_fwd(FwdMode mode, FwdArgs a, Dims d, int window, int tz,
+                              cudaStream_t s) {
+    fill_grid(a, d);
+    a.window = window;
+    a.bits = lncc_image_bits(window);
+    cudaError_t e = cudaErrorInvalidValue;
+    FA_EACH_R((fwd_mode<RR>(mode, a, d, tz, s)))
+    note_launch();
+    return e;
+}
+
+cudaError_t launch_window_grad(bool swap, GradArgs a, Dims d, int window, int tz,
+                               cudaStream_t s) {
+    fill_grid(a, d);
+    a.n = window * window * window;
+    a.cbits = lncc_coef_bits(window);
+    cudaError_t e = cudaErrorInvalidValue;
+    FA_EACH_R((swap ? grad<RR, true>(a, d, tz, s) : grad<RR, false>(a, d, tz, s)))
+    note_launch();
+    return e;
+}
+#undef FA_EACH_R
+
+}  // namespace fa
