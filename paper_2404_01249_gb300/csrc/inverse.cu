@@ -331,8 +331,9 @@ extern "C" fa_status fa_inverse(const fa_vol *u, const fa_params *p, fa_vol *w_o
             ++t;
             const int parity = t & 1;
             FA_CUDA_TRY(inverse_gradient(q, q.ul, q.w[cur], d, q.g, nullptr, s));
-            FA_CUDA_TRY(launch_gauss3(q.g, q.g, q.t1, q.t2, 3, d, tg, s));
-            FA_CUDA_TRY(launch_adam(q.g, q.m[cur], q.v[cur], q.dir, d.N(), adam_consts(p, t),
+            const float *g;
+            FA_CUDA_TRY(launch_gauss3_any(q.g, q.t1, q.t2, 3, d, tg, &g, s));
+            FA_CUDA_TRY(launch_adam(g, q.m[cur], q.v[cur], q.dir, d.N(), adam_consts(p, t),
                                     q.h, parity, s));
             FA_CUDA_TRY(launch_compose(q.w[cur], q.dir, q.w[cur ^ 1], d, p->lr, p->c_lp, q.h,
                                        parity, nullptr, s));

@@ -94,9 +94,7 @@ cudaError_t launch_pyramid_level(const float *img, Dims d, int s, float *out, Di
     GaussTaps t;
     if (!make_gauss_taps(0.5f * (float)s, &t)) return cudaErrorInvalidValue;
     cudaError_t e;
-    if ((e = launch_gauss_axis(img, t1, 1, d, t, 0, st)) != cudaSuccess) return e;
-    if ((e = launch_gauss_axis(t1, t2, 1, d, t, 1, st)) != cudaSuccess) return e;
-    if ((e = launch_gauss_axis(t2, t1, 1, d, t, 2, st)) != cudaSuccess) return e;
+    if ((e = launch_gauss3(img, t1, t1, t2, 1, d, t, st)) != cudaSuccess) return e;
     return launch_resample(t1, d, out, dl, 1, nullptr, st);
 }
 

@@ -138,9 +138,14 @@ cudaError_t launch_header_reset(WsHeader *h, cudaStream_t s);
 // ---- Gaussian (gauss.cu)
 cudaError_t launch_gauss_axis(const float *in, float *out, int C, Dims d, const GaussTaps &t,
                               int axis, cudaStream_t s);
-// Three passes in -> t1 -> t2 -> out (t1, t2: C*N floats each).  R == 0 copies.
+// in -> out (t1, t2: C*N floats of scratch each; out may be in or t1).  R == 0 copies.
 cudaError_t launch_gauss3(const float *in, float *out, float *t1, float *t2, int C, Dims d,
                           const GaussTaps &t, cudaStream_t s);
+
+// The smoothed field where the caller does not mind the place: in itself for
+// R == 0, else t1 (t1, t2 as above); *res points at it.
+cudaError_t launch_gauss3_any(const float *in, float *t1, float *t2, int C, Dims d,
+                              const GaussTaps &t, const float **res, cudaStream_t s);
 
 // ---- Adam, step scale, compose (adam.cu)
 // Records a kernel timer's event on s: as an external event node while s is

@@ -248,9 +248,10 @@ static fa_status plain_iteration(Plan &P, const fa_params *p, int l, const float
         FA_CUDA_TRY(launch_mse(If, P.J, P.grad, d, P.h, P.partials, nullptr, nullptr, P.g, s));
     }
     if (p->use_jac) FA_CUDA_TRY(launch_jac_direction(P.g, u, P.g, d, s));
-    FA_CUDA_TRY(launch_gauss3(P.g, P.g, P.t1, P.t2, 3, d, tg, s));
+    const float *g;
+    FA_CUDA_TRY(launch_gauss3_any(P.g, P.t1, P.t2, 3, d, tg, &g, s));
     int parity = t & 1;
-    FA_CUDA_TRY(launch_adam_state(P.g, m, v, p->state_storage, P.dir, N, adam_consts(p, t), P.h,
+    FA_CUDA_TRY(launch_adam_state(g, m, v, p->state_storage, P.dir, N, adam_consts(p, t), P.h,
                                   parity, s));
     FA_CUDA_TRY(launch_compose(u, P.dir, u_alt, d, p->lr, p->c_lp, P.h, parity, nullptr, s));
     FA_CUDA_TRY(launch_gauss3(u_alt, u, P.t1, P.t2, 3, d, tw, s));

@@ -292,8 +292,9 @@ extern "C" fa_status fa_register_svf(const fa_vol *fixed, const fa_vol *moving,
             ++t;
             const int parity = t & 1;
             FA_TRY(svf_eval(q, p, steps, d, If, Im, q.v[cur], true, nullptr, s));
-            FA_CUDA_TRY(launch_gauss3(q.g, q.g, q.t1, q.t2, 3, d, tg, s));
-            FA_CUDA_TRY(launch_adam(q.g, q.m[cur], q.nu[cur], q.dir, d.N(), adam_consts(p, t), q.h,
+            const float *g;
+            FA_CUDA_TRY(launch_gauss3_any(q.g, q.t1, q.t2, 3, d, tg, &g, s));
+            FA_CUDA_TRY(launch_adam(g, q.m[cur], q.nu[cur], q.dir, d.N(), adam_consts(p, t), q.h,
                                     parity, s));
             k_svf_step<<<blocks_for(n3), 256, 0, s>>>(q.v[cur], q.dir, q.v[cur ^ 1], n3, p->lr,
                                                       p->c_lp, q.h, parity);

@@ -143,8 +143,9 @@ fa_status sym_update(SymWs &q, const fa_params *p, Dims d, float *g, int k, int 
     // the two maps share the step-maximum slot of this parity
     FA_CUDA_TRY(cudaMemsetAsync(&q.h->step_max_bits[parity], 0, sizeof(unsigned), s));
     if (p->use_jac) FA_CUDA_TRY(launch_jac_direction(g, u, g, d, s));
-    FA_CUDA_TRY(launch_gauss3(g, g, q.t1, q.t2, 3, d, tg, s));
-    FA_CUDA_TRY(launch_adam(g, q.m[k][cur], q.v[k][cur], q.dir, d.N(), adam_consts(p, t), q.h,
+    const float *sg;
+    FA_CUDA_TRY(launch_gauss3_any(g, q.t1, q.t2, 3, d, tg, &sg, s));
+    FA_CUDA_TRY(launch_adam(sg, q.m[k][cur], q.v[k][cur], q.dir, d.N(), adam_consts(p, t), q.h,
                             parity, s));
     FA_CUDA_TRY(launch_compose(u, q.dir, alt, d, p->lr, p->c_lp, q.h, parity, nullptr, s));
     FA_CUDA_TRY(launch_gauss3(alt, u, q.t1, q.t2, 3, d, tw, s));
