@@ -56,8 +56,8 @@ __device__ __forceinline__ float bias_recip(float b, int t) {
 }
 
 // The same step with the step number taken from the device counter:
-// t = *t_dev + 1 (the counter itself is advanced by k_count_step after the
-// compose, so that every block here reads the same value).
+// t = *t_dev + 1 (the counter itself is advanced by the compose kernel, so
+// that every block here reads the same value).
 template <class TS>
 __global__ void __launch_bounds__(256) k_adam_tdev(const float *__restrict__ g,
                                                    TS *__restrict__ m, TS *__restrict__ v,
@@ -78,13 +78,11 @@ __global__ void __launch_bounds__(256) k_adam_tdev(const float *__restrict__ g,
     adam_body<TS>(g, m, v, d, N, c, h, 0);
 }
 
-__global__ void k_count_step(int *t_dev) { *t_dev += 1; }
-
 __global__ void __launch_bounds__(256) k_compose(const float *__restrict__ u,
                                                  const float *__restrict__ d,
                                                  float *__restrict__ uo, int D, int H, int W,
                                                  float lr, float c_lp, WsHeader *h, int parity,
-                                                 float *eps_out) {
+                                                 float *eps_out, int *t_dev) {
     int x = blockIdx.x * 32 + threadIdx.x;
     int y = blockIdx.y * 8 + threadIdx.y;
     int z = blockIdx.z;
@@ -95,17 +93,18 @@ __global__ void __launch_bounds__(256) k_compose(const float *__restrict__ u,
         h->step_max_bits[parity ^ 1] = 0u;  // slot of the next iteration
         h->eps_t = e;
         if (eps_out) *eps_out = e;
+        if (t_dev) *t_dev += 1;  // the Adam kernel before this one read it
     }
     if (x >= W || y >= H) return;
     long long N = (long long)D * H * W;
     long long i = ((long long)z * H + y) * W + x;
     float dz = -e * d[i], dy = -e * d[N + i], dx = -e * d[2 * N + i];
     float gz, gy, gx;
+    TriPending q[3];  // the compose's cell (the same as the fused schedule's)
+    tri_issue_step3(q, u, N, D, H, W, z, y, x, dz, dy, dx);
 #pragma unroll
     for (int ch = 0; ch < 3; ++ch) {
-        TriPending q;  // the compose's cell (the same as the fused schedule's)
-        tri_issue_step(q, u + ch * N, D, H, W, W, z, y, x, dz, dy, dx);
-        float s = tri_finish<false>(q, gz, gy, gx);
+        float s = tri_finish<false>(q[ch], gz, gy, gx);
         float dc = ch == 0 ? dz : (ch == 1 ? dy : dx);
         uo[ch * N + i] = dc + s;
     }
@@ -125,9 +124,10 @@ __global__ void __launch_bounds__(256) k_compose_fields(const float *__restrict_
     long long i = ((long long)z * H + y) * W + x;
     const float dz = delta[i], dy = delta[N + i], dx = delta[2 * N + i];
     float gz, gy, gx, r[3];
+    TriPending q[3];
+    tri_issue3(q, u, N, D, H, W, z, y, x, dz, dy, dx);
 #pragma unroll
-    for (int ch = 0; ch < 3; ++ch)
-        r[ch] = tri_sample<false>(u + ch * N, D, H, W, z, y, x, dz, dy, dx, gz, gy, gx);
+    for (int ch = 0; ch < 3; ++ch) r[ch] = tri_finish<false>(q[ch], gz, gy, gx);
     uo[i] = dz + r[0];
     uo[N + i] = dy + r[1];
     uo[2 * N + i] = dx + r[2];
@@ -187,10 +187,11 @@ cudaError_t launch_adam_tdev(const float *g, void *m, void *v, int state, float 
 }
 
 cudaError_t launch_compose(const float *u_in, const float *d, float *u_out, Dims dm, float lr,
-                           float c_lp, WsHeader *h, int parity, float *eps_out, cudaStream_t s) {
+                           float c_lp, WsHeader *h, int parity, float *eps_out, cudaStream_t s,
+                           int *t_dev) {
     VoxGrid g(dm.D, dm.H, dm.W);
     k_compose<<<g.grid, g.block, 0, s>>>(u_in, d, u_out, dm.D, dm.H, dm.W, lr, c_lp, h, parity,
-                                         eps_out); note_launch();
+                                         eps_out, t_dev); note_launch();
     return cudaGetLastError();
 }
 
@@ -274,10 +275,7 @@ extern "C" fa_status fa_radam_step(const fa_vol *u_in, fa_vol *u_out, fa_vol *m,
     FA_CUDA_TRY(launch_adam_tdev((const float *)g->data, m->data, v->data, m->dtype, dir, d.N(), p,
                                  t_dev, h, s));
     FA_CUDA_TRY(launch_compose((const float *)u_in->data, dir, (float *)u_out->data, d, p->lr,
-                               p->c_lp, h, 0, eps_t_dev, s));
-    k_count_step<<<1, 1, 0, s>>>(t_dev);
-    note_launch();
-    FA_CUDA_TRY(cudaGetLastError());
+                               p->c_lp, h, 0, eps_t_dev, s, t_dev));
     return FA_OK;
 }
 

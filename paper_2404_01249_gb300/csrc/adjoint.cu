@@ -19,13 +19,13 @@
 // in which threads add (the same fixed-point scheme as the window sums).
 #include "ops.h"
 #include "register.h"
+#include "scatter.cuh"
 #include "validate.h"
 
 namespace fa {
 
 namespace {
 
-constexpr int kScatterBits = 40;  // |term| <= 2^40: sums of 2^23 terms fit int64
 constexpr int kSlotDJ = 7;        // header slot of max |dL/dJ|
 
 struct AdjointBuffers {
@@ -87,47 +87,30 @@ __global__ void __launch_bounds__(256) k_warp_adjoint_scatter(const float *__res
     const int x = blockIdx.x * 32 + threadIdx.x;
     const int y = blockIdx.y * 8 + threadIdx.y;
     const int z = blockIdx.z;
-    if (x >= W || y >= H) return;
+    if (y >= H) return;  // whole warps; lanes beyond a row's end stay for the shuffles
     const long long N = (long long)D * H * W;
     const long long i = ((long long)z * H + y) * W + x;
-    const float g = dJ[i];
-    const float uz = u[i], uy = u[N + i], ux = u[2 * N + i];
+    float g = 0.0f, uz = 0.0f, uy = 0.0f, ux = 0.0f;
+    if (x < W) {
+        g = dJ[i];
+        uz = u[i];
+        uy = u[N + i];
+        ux = u[2 * N + i];
+    }
     const float LIM = 1048576.0f;
     // zero, non-finite (reported by the loss) or far-outside samples add nothing
-    if (!(fabsf(g) > 0.0f && fabsf(g) < 3.4e38f) ||
-        !(fabsf(uz) < LIM && fabsf(uy) < LIM && fabsf(ux) < LIM))
-        return;
-    const int sh = fixed_shift(__uint_as_float(h->coef_max_bits[kSlotDJ]), kScatterBits);
-    const float scale = pow2f(sh);
+    const bool on = fabsf(g) > 0.0f && fabsf(g) < 3.4e38f && fabsf(uz) < LIM &&
+                    fabsf(uy) < LIM && fabsf(ux) < LIM;
+    const int sh = fixed_shift(__uint_as_float(h->coef_max_bits[kSlotDJ]), kFieldScatterBits);
     const float fz = floorf(uz), fy = floorf(uy), fx = floorf(ux);
-    const int iz = z + (int)fz, iy = y + (int)fy, ix = x + (int)fx;
-    const float tz = uz - fz, ty = uy - fy, tx = ux - fx;
-    const float wz[2] = {1.0f - tz, tz}, wy[2] = {1.0f - ty, ty}, wx[2] = {1.0f - tx, tx};
-#pragma unroll
-    for (int a = 0; a < 2; ++a) {
-        const int zz = iz + a;
-        if (zz < 0 || zz >= D) continue;
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-            const int yy = iy + b;
-            if (yy < 0 || yy >= H) continue;
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                const int xx = ix + c;
-                if (xx < 0 || xx >= W) continue;
-                const float w = wz[a] * wy[b] * wx[c];
-                const long long q = quantize(g * w, scale);
-                if (q != 0)
-                    atomicAdd(acc + ((long long)zz * H + yy) * W + xx, (unsigned long long)q);
-            }
-        }
-    }
+    scatter_cell1(acc, D, H, W, z + (on ? (int)fz : 0), y + (on ? (int)fy : 0),
+                  x + (on ? (int)fx : 0), uz - fz, uy - fy, ux - fx, on ? g : 0.0f, pow2f(sh), on);
 }
 
 __global__ void __launch_bounds__(256) k_scatter_finalize(const long long *__restrict__ acc,
                                                           const WsHeader *h, float *out,
                                                           long long n) {
-    const int sh = fixed_shift(__uint_as_float(h->coef_max_bits[kSlotDJ]), kScatterBits);
+    const int sh = fixed_shift(__uint_as_float(h->coef_max_bits[kSlotDJ]), kFieldScatterBits);
     const float inv = pow2f(-sh);
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)

@@ -224,6 +224,112 @@ __device__ __forceinline__ void tri_issue_step(TriPending &p, const T *__restric
     p.c111 = zo && yo && xo ? ld_field(q1 + oy + sx) : 0.0f;
 }
 
+// The same cells for three channels of a field, N elements apart: the cell,
+// its place and the choice of path are worked out once for all three.
+template <class T>
+__device__ __forceinline__ void tri_issue3(TriPending (&p)[3], const T *__restrict__ v,
+                                           long long N, int D, int H, int W, int z, int y, int x,
+                                           float uz, float uy, float ux) {
+    const float LIM = 1048576.0f;
+    if (!(fabsf(uz) < LIM && fabsf(uy) < LIM && fabsf(ux) < LIM)) {
+        tri_issue_p(p[0], v, D, H, W, W, z, y, x, uz, uy, ux);
+        p[1] = p[2] = p[0];
+        return;
+    }
+    const float fz = floorf(uz), fy = floorf(uy), fx = floorf(ux);
+    const int iz = z + (int)fz, iy = y + (int)fy, ix = x + (int)fx;
+    const bool z0 = iz >= 0 && iz < D, z1 = iz + 1 >= 0 && iz + 1 < D;
+    const bool y0 = iy >= 0 && iy < H, y1 = iy + 1 >= 0 && iy + 1 < H;
+    const bool x0 = ix >= 0 && ix < W, x1 = ix + 1 >= 0 && ix + 1 < W;
+    // corners outside the grid read as zero
+    const T *q0 = v + ((long long)iz * H + iy) * W + ix, *q1 = q0 + (long long)H * W;
+    if (z0 && z1 && y0 && y1 && x0 && x1) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            p[c].c000 = ld_field(q0);
+            p[c].c001 = ld_field(q0 + 1);
+            p[c].c010 = ld_field(q0 + W);
+            p[c].c011 = ld_field(q0 + W + 1);
+            p[c].c100 = ld_field(q1);
+            p[c].c101 = ld_field(q1 + 1);
+            p[c].c110 = ld_field(q1 + W);
+            p[c].c111 = ld_field(q1 + W + 1);
+            q0 += N;
+            q1 += N;
+        }
+    } else {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            p[c].c000 = z0 && y0 && x0 ? ld_field(q0) : 0.0f;
+            p[c].c001 = z0 && y0 && x1 ? ld_field(q0 + 1) : 0.0f;
+            p[c].c010 = z0 && y1 && x0 ? ld_field(q0 + W) : 0.0f;
+            p[c].c011 = z0 && y1 && x1 ? ld_field(q0 + W + 1) : 0.0f;
+            p[c].c100 = z1 && y0 && x0 ? ld_field(q1) : 0.0f;
+            p[c].c101 = z1 && y0 && x1 ? ld_field(q1 + 1) : 0.0f;
+            p[c].c110 = z1 && y1 && x0 ? ld_field(q1 + W) : 0.0f;
+            p[c].c111 = z1 && y1 && x1 ? ld_field(q1 + W + 1) : 0.0f;
+            q0 += N;
+            q1 += N;
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        p[c].tz = uz - fz;
+        p[c].ty = uy - fy;
+        p[c].tx = ux - fx;
+    }
+}
+
+template <class T>
+__device__ __forceinline__ void tri_issue_step3(TriPending (&p)[3], const T *__restrict__ v,
+                                                long long N, int D, int H, int W, int z, int y,
+                                                int x, float uz, float uy, float ux) {
+    if (!(fabsf(uz) < 1.0f && fabsf(uy) < 1.0f && fabsf(ux) < 1.0f)) {
+        tri_issue3(p, v, N, D, H, W, z, y, x, uz, uy, ux);
+        return;
+    }
+    const int sz = uz < 0.0f ? -1 : 1, sy = uy < 0.0f ? -1 : 1, sx = ux < 0.0f ? -1 : 1;
+    const bool zo = z + sz >= 0 && z + sz < D, yo = y + sy >= 0 && y + sy < H,
+               xo = x + sx >= 0 && x + sx < W;
+    const T *q0 = v + ((long long)z * H + y) * W + x, *q1 = q0 + (long long)sz * H * W;
+    const int oy = sy * W;
+    if (zo && yo && xo) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            p[c].c000 = ld_field(q0);
+            p[c].c001 = ld_field(q0 + sx);
+            p[c].c010 = ld_field(q0 + oy);
+            p[c].c011 = ld_field(q0 + oy + sx);
+            p[c].c100 = ld_field(q1);
+            p[c].c101 = ld_field(q1 + sx);
+            p[c].c110 = ld_field(q1 + oy);
+            p[c].c111 = ld_field(q1 + oy + sx);
+            q0 += N;
+            q1 += N;
+        }
+    } else {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            p[c].c000 = ld_field(q0);
+            p[c].c001 = xo ? ld_field(q0 + sx) : 0.0f;
+            p[c].c010 = yo ? ld_field(q0 + oy) : 0.0f;
+            p[c].c011 = yo && xo ? ld_field(q0 + oy + sx) : 0.0f;
+            p[c].c100 = zo ? ld_field(q1) : 0.0f;
+            p[c].c101 = zo && xo ? ld_field(q1 + sx) : 0.0f;
+            p[c].c110 = zo && yo ? ld_field(q1 + oy) : 0.0f;
+            p[c].c111 = zo && yo && xo ? ld_field(q1 + oy + sx) : 0.0f;
+            q0 += N;
+            q1 += N;
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        p[c].tz = fabsf(uz);
+        p[c].ty = fabsf(uy);
+        p[c].tx = fabsf(ux);
+    }
+}
+
 __device__ __forceinline__ void tri_issue(TriPending &p, const float *__restrict__ v, int D,
                                           int H, int W, int z, int y, int x, float uz, float uy,
                                           float ux) {

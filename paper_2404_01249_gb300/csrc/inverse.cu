@@ -12,13 +12,13 @@
 // The descent is Algorithm 1's: Gaussian(sigma_grad), Adam, step scaling,
 // compose, Gaussian(sigma_warp), with the per-op kernels.
 #include "ops.h"
+#include "scatter.cuh"
 #include "validate.h"
 
 namespace fa {
 
 namespace {
 
-constexpr int kInvBits = 40;
 constexpr int kSlotA = 7;  // header slot of max |A|
 constexpr int kEnergyBlocks = 152 * 4;
 
@@ -71,14 +71,16 @@ __global__ void __launch_bounds__(256) k_inverse_terms(const float *__restrict__
         const float uz = u[i], uy = u[N + i], ux = u[2 * N + i];
         const float wz = w[i], wy = w[N + i], wx = w[2 * N + i];
         float A[3], B[3], G[3][3], gz, gy, gx;
-        A[0] = uz + tri_sample<false>(w, D, H, W, z, y, x, uz, uy, ux, gz, gy, gx);
-        A[1] = uy + tri_sample<false>(w + N, D, H, W, z, y, x, uz, uy, ux, gz, gy, gx);
-        A[2] = ux + tri_sample<false>(w + 2 * N, D, H, W, z, y, x, uz, uy, ux, gz, gy, gx);
+        TriPending q[3];
+        tri_issue3(q, w, N, D, H, W, z, y, x, uz, uy, ux);
+        A[0] = uz + tri_finish<false>(q[0], gz, gy, gx);
+        A[1] = uy + tri_finish<false>(q[1], gz, gy, gx);
+        A[2] = ux + tri_finish<false>(q[2], gz, gy, gx);
+        tri_issue3(q, u, N, D, H, W, z, y, x, wz, wy, wx);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const float wc = c == 0 ? wz : (c == 1 ? wy : wx);
-            B[c] = wc + tri_sample<true>(u + c * N, D, H, W, z, y, x, wz, wy, wx, G[c][0], G[c][1],
-                                         G[c][2]);
+            B[c] = wc + tri_finish<true>(q[c], G[c][0], G[c][1], G[c][2]);
         }
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
@@ -120,52 +122,55 @@ __global__ void __launch_bounds__(256) k_field_scatter(const float *__restrict__
                                                        unsigned long long *acc, const WsHeader *h,
                                                        int slot, int D, int H, int W) {
     const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y, z = blockIdx.z;
-    if (x >= W || y >= H) return;
+    if (y >= H) return;  // whole warps; lanes beyond a row's end stay for the shuffles
     const long long N = (long long)D * H * W, i = ((long long)z * H + y) * W + x;
-    const float uz = u[i], uy = u[N + i], ux = u[2 * N + i];
-    const float LIM = 1048576.0f;
-    if (!(fabsf(uz) < LIM && fabsf(uy) < LIM && fabsf(ux) < LIM)) return;
-    const int sh = fixed_shift(__uint_as_float(h->coef_max_bits[slot]), kInvBits);
-    const float scale = pow2f(sh);
-    const float a[3] = {A[i], A[N + i], A[2 * N + i]};
-    if (!(fabsf(a[0]) < 3.4e38f && fabsf(a[1]) < 3.4e38f && fabsf(a[2]) < 3.4e38f)) return;
-    const float fz = floorf(uz), fy = floorf(uy), fx = floorf(ux);
-    const int iz = z + (int)fz, iy = y + (int)fy, ix = x + (int)fx;
-    const float tz = uz - fz, ty = uy - fy, tx = ux - fx;
-    const float wz[2] = {1.0f - tz, tz}, wy[2] = {1.0f - ty, ty}, wx[2] = {1.0f - tx, tx};
-#pragma unroll
-    for (int p = 0; p < 2; ++p) {
-        const int zz = iz + p;
-        if (zz < 0 || zz >= D) continue;
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int yy = iy + q;
-            if (yy < 0 || yy >= H) continue;
-#pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                const int xx = ix + r;
-                if (xx < 0 || xx >= W) continue;
-                const float wt = wz[p] * wy[q] * wx[r];
-                const long long j = ((long long)zz * H + yy) * W + xx;
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    const long long qv = quantize(a[c] * wt, scale);
-                    if (qv != 0) atomicAdd(acc + c * N + j, (unsigned long long)qv);
-                }
-            }
-        }
+    float uz = 0.0f, uy = 0.0f, ux = 0.0f, a[3] = {0.0f, 0.0f, 0.0f};
+    bool on = x < W;
+    if (on) {
+        uz = u[i];
+        uy = u[N + i];
+        ux = u[2 * N + i];
+        a[0] = A[i];
+        a[1] = A[N + i];
+        a[2] = A[2 * N + i];
     }
+    on = on && scatter_takes(uz, uy, ux, a);
+    const int sh = fixed_shift(__uint_as_float(h->coef_max_bits[slot]), kFieldScatterBits);
+    const float fz = floorf(uz), fy = floorf(uy), fx = floorf(ux);
+    scatter_cell3(acc, N, D, H, W, z + (on ? (int)fz : 0), y + (on ? (int)fy : 0),
+                  x + (on ? (int)fx : 0), uz - fz, uy - fy, ux - fx, a, pow2f(sh), on);
 }
 
-// g += factor * (scattered a)
+// See launch_field_scatter_add.  Bound: HBM, 16 bytes per value (two values
+// per thread and step).  Storing the next scatter's zeros here, instead of a
+// memset before it, took 435 us per 20.6 M values against 84: the stores wait
+// for lines that the reductions left on the other half of L2.
 __global__ void __launch_bounds__(256) k_field_scatter_add(const long long *__restrict__ acc,
-                                                           const WsHeader *h, int slot, float *g,
-                                                           long long n3, float factor) {
-    const int sh = fixed_shift(__uint_as_float(h->coef_max_bits[slot]), kInvBits);
+                                                           WsHeader *h, int slot,
+                                                           const float *src, float *dst,
+                                                           long long n3, float factor, float post,
+                                                           int max_slot) {
+    __shared__ float red[32];
+    const int sh = fixed_shift(__uint_as_float(h->coef_max_bits[slot]), kFieldScatterBits);
     const float f = factor * pow2f(-sh);
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n3;
-         i += (long long)gridDim.x * blockDim.x)
-        g[i] = fmaf(i64_to_float_rn(acc[i]), f, g[i]);
+    float amax = 0.0f;
+    auto one = [&](long long a, float g) {
+        const float v = fmaf(i64_to_float_rn(a), f, g) * post;
+        const float av = fabsf(v);
+        if (av < 3.4e38f) amax = fmaxf(amax, av);
+        return v;
+    };
+    const long long stride = 2ll * gridDim.x * blockDim.x;
+    for (long long i = 2 * ((long long)blockIdx.x * blockDim.x + threadIdx.x); i < n3; i += stride) {
+        if (i + 1 < n3) {
+            const longlong2 a = *(const longlong2 *)(acc + i);
+            const float2 g = *(const float2 *)(src + i);
+            *(float2 *)(dst + i) = make_float2(one(a.x, g.x), one(a.y, g.y));
+        } else {
+            dst[i] = one(acc[i], src[i]);
+        }
+    }
+    if (max_slot >= 0) block_max_to(&h->coef_max_bits[max_slot], amax, red);
 }
 
 __global__ void k_energy_finalize(const float *__restrict__ partials, int nb, long long N,
@@ -195,9 +200,8 @@ cudaError_t inverse_gradient(InverseWs &q, const float *u, const float *w, Dims 
         note_launch();
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    if ((e = cudaMemsetAsync(q.acc, 0, sizeof(long long) * 3 * N, s)) != cudaSuccess) return e;
     if ((e = launch_field_scatter(u, q.A, q.acc, q.h, kSlotA, d, s)) != cudaSuccess) return e;
-    return launch_field_scatter_add(q.acc, q.h, kSlotA, 2.0f / (float)N, g, 3 * N, s);
+    return launch_field_scatter_add(q.acc, q.h, kSlotA, 2.0f / (float)N, g, g, 1.0f, -1, 3 * N, s);
 }
 
 fa_status check_inverse_params(const fa_params *p) {
@@ -230,6 +234,8 @@ size_t inverse_ws_bytes(Dims full, const fa_params *p) {
 
 cudaError_t launch_field_scatter(const float *u, const float *a, long long *acc,
                                  const WsHeader *h, int slot, Dims d, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(acc, 0, sizeof(long long) * 3 * d.N(), s);
+    if (e != cudaSuccess) return e;
     VoxGrid vg(d.D, d.H, d.W);
     k_field_scatter<<<vg.grid, vg.block, 0, s>>>(u, a, (unsigned long long *)acc, h, slot, d.D,
                                                  d.H, d.W);
@@ -237,9 +243,13 @@ cudaError_t launch_field_scatter(const float *u, const float *a, long long *acc,
     return cudaGetLastError();
 }
 
-cudaError_t launch_field_scatter_add(const long long *acc, const WsHeader *h, int slot,
-                                     float factor, float *g, long long n3, cudaStream_t s) {
-    k_field_scatter_add<<<kEnergyBlocks, 256, 0, s>>>(acc, h, slot, g, n3, factor);
+cudaError_t launch_field_scatter_add(const long long *acc, WsHeader *h, int slot, float factor,
+                                     const float *src, float *dst, float post, int max_slot,
+                                     long long n3, cudaStream_t s) {
+    long long blocks = (n3 + 511) / 512;
+    blocks = blocks > 152 * 16 ? 152 * 16 : blocks;
+    k_field_scatter_add<<<(unsigned)blocks, 256, 0, s>>>(acc, h, slot, src, dst, n3, factor, post,
+                                                         max_slot);
     note_launch();
     return cudaGetLastError();
 }

@@ -100,15 +100,18 @@ long long mse_partials_count(Dims d);  // floats of `partials` launch_mse needs
 cudaError_t launch_mse(const float *I, const float *J, const float *grad, Dims d, WsHeader *h,
                        float *partials, float *dJ, float *dI, float *g, cudaStream_t s);
 // ---- field adjoints (inverse.cu)
-// acc (3 channels, int64, zeroed by the caller) += a scattered through the
+// acc (3 channels, int64) = a scattered through the
 // trilinear weights of the corners of x + u(x) (zero outside), each term
 // quantised to 2^-40 of max |a|, whose float bits the caller has put in
 // h->coef_max_bits[slot]: the sums do not depend on the order of the adds.
 cudaError_t launch_field_scatter(const float *u, const float *a, long long *acc,
                                  const WsHeader *h, int slot, Dims d, cudaStream_t s);
-// g += factor * acc, converted back with the same scale.
-cudaError_t launch_field_scatter_add(const long long *acc, const WsHeader *h, int slot,
-                                     float factor, float *g, long long n3, cudaStream_t s);
+// dst = (src + factor * acc) * post with acc converted back with the same
+// scale; max_slot >= 0: max |dst| of the finite values into that header slot
+// (another one than `slot`).  dst may be src.
+cudaError_t launch_field_scatter_add(const long long *acc, WsHeader *h, int slot, float factor,
+                                     const float *src, float *dst, float post, int max_slot,
+                                     long long n3, cudaStream_t s);
 
 // ---- mutual information (mi.cu)
 struct MiBuffers {
@@ -176,9 +179,11 @@ cudaError_t launch_adam_state(const float *g, void *m, void *v, int state, float
 // Bytes of one element of the Adam moments stored as `state`.
 inline size_t state_bytes(int state) { return state == FA_F32 ? 4 : 2; }
 // u_out = delta + u_in o (id + delta), delta = -lr / (c_lp max) d; resets the
-// other parity's max slot; eps_t to h->eps_t and eps_out (if not NULL).
+// other parity's max slot; eps_t to h->eps_t and eps_out (if not NULL);
+// advances the step counter t_dev (if not NULL) by one.
 cudaError_t launch_compose(const float *u_in, const float *d, float *u_out, Dims dm, float lr,
-                           float c_lp, WsHeader *h, int parity, float *eps_out, cudaStream_t s);
+                           float c_lp, WsHeader *h, int parity, float *eps_out, cudaStream_t s,
+                           int *t_dev = nullptr);
 
 // ---- pyramid and hand-off (levels.cu)
 // dst channel c = scale[c] * trilinear align-corners resample of src channel c
