@@ -34,20 +34,27 @@ std::mutex g_tune_mu;
 std::map<TuneKey, TileChoice> g_tune;
 thread_local const TileChoice *g_force = nullptr;  // a candidate under measurement
 
-constexpr int kDefaultWide[4] = {0, 0, 0, 1};
+// 32 x 16 tiles for K3 and K4 unless even slabs of one plane leave SMs without
+// a CTA: there the shorter march of 32 x 8 tiles counts (a 32^3 pair: 1.80 ms
+// with 32 x 16 tiles on both levels, 1.70 with 32 x 8; K4 on 16 x 32 x 32
+// voxels 14.4 against 12.3 us, but on 32 x 64 x 64 voxels 22.6 against 24.3).
+int default_wide(int kernel, Dims d) {
+    const long long tiles = (long long)((d.W + FX - 1) / FX) * ((d.H + 15) / 16);
+    return kernel >= 2 && tiles * d.D >= num_sms();
+}
 
 TileChoice tile_choice(int kernel, int radius, int su, Dims d) {
     if (g_force) return *g_force;
     std::lock_guard<std::mutex> lock(g_tune_mu);
     auto it = g_tune.find(TuneKey{kernel, radius, su, d.D, d.H, d.W});
     if (it != g_tune.end()) return it->second;
-    return TileChoice{kDefaultWide[kernel], 0};
+    return TileChoice{default_wide(kernel, d), 0};
 }
 
-inline LaunchGeom geometry(int occ, int nw, int ty, int halo, Dims d, int tz = 0) {
+inline LaunchGeom geometry(int occ, int nw, int ty, float extra, Dims d, int tz) {
     LaunchGeom g;
     const int gx = (d.W + FX - 1) / FX, gy = (d.H + ty - 1) / ty;
-    g.tz = tz > 0 ? (tz < d.D ? tz : d.D) : choose_tz(d.D, gx * gy, 2.0f * halo, occ);
+    g.tz = tz > 0 ? (tz < d.D ? tz : d.D) : choose_tz(d.D, gx * gy, extra, occ);
     g.grid = dim3(gx, gy, (d.D + g.tz - 1) / g.tz);
     g.block = dim3(FX, nw);
     return g;
@@ -163,20 +170,19 @@ cudaError_t launch_k2(const float *If, const float *gJ, const float *J, const fl
     return launch_window_grad(false, a, d, window, tile_choice(1, window / 2, 0, d).tz, s);
 }
 
-template <int RG, int NW, class TS>
+template <int RG, int NW, int OPT, class TS>
 cudaError_t launch_k3_tma(const Maps &mp, const float *g, TS *m, TS *v, float *dir, WsHeader *h,
                           Dims d, const GaussTaps &t, AdamConsts ac, int parity, int tz,
                           cudaStream_t s) {
-    using ST = K3S<RG, NW, K3_OPT, K3_ST_TMA, sizeof(TS) == 4>;
-    auto kern = k_smooth_adam<RG, NW, K3_OPT, K3_ST_TMA, true, TS>;
+    using ST = K3S<RG, NW, OPT, K3_ST, sizeof(TS) == 4>;
+    auto kern = k_smooth_adam<RG, NW, OPT, K3_ST, true, TS>;
     static const int occ = prepare(kern, ST::bytes, ST::NT);
-    LaunchGeom gg = geometry(occ, NW, ST::TY, RG, d, tz);
+    LaunchGeom gg = geometry(occ, NW, ST::TY, 2.0f * RG, d, tz);
     return launch_pdl(kern, gg, ST::bytes, s, mp, g, m, v, dir, h, d.D, d.H, d.W, d.pitch(), gg.tz, t, ac,
                       parity);
 }
 
-// TS: storage of the moments (float, __nv_bfloat16 or __half); 16-bit moments
-// take the 32 x 8 tiles only.
+// TS: storage of the moments (float, __nv_bfloat16 or __half).
 template <int RG, class TS>
 cudaError_t launch_k3(const float *g, TS *m, TS *v, float *dir, WsHeader *h, Dims d,
                       const GaussTaps &t, AdamConsts ac, int parity, cudaStream_t s) {
@@ -184,22 +190,21 @@ cudaError_t launch_k3(const float *g, TS *m, TS *v, float *dir, WsHeader *h, Dim
     Maps mp{};
     cudaError_t le;
     const TileChoice tc = tile_choice(2, RG, 0, d);
-    const bool wide = S32 && tc.wide;
-    const int nw = wide ? 16 : 8;
-    const bool tma = tmap(&mp.a, g, 4, d, 3, FX + 2 * halo4(RG), nw + 2 * RG, 3) &&
-                     (!S32 || (tmap(&mp.b, m, 4, d, 3, FX, nw, 3) &&
-                               tmap(&mp.c, v, 4, d, 3, FX, nw, 3)));
+    const bool wide = tc.wide;
+    const int ty = wide ? 16 : 8;
+    const bool tma = tmap(&mp.a, g, 4, d, 3, FX + 2 * halo4(RG), ty + 2 * RG, 3) &&
+                     (!S32 || (tmap(&mp.b, m, 4, d, 3, FX, ty, 3) &&
+                               tmap(&mp.c, v, 4, d, 3, FX, ty, 3)));
     if (tma) {
-        if constexpr (S32)
-            le = wide ? launch_k3_tma<RG, 16, TS>(mp, g, m, v, dir, h, d, t, ac, parity, tc.tz, s)
-                      : launch_k3_tma<RG, 8, TS>(mp, g, m, v, dir, h, d, t, ac, parity, tc.tz, s);
-        else
-            le = launch_k3_tma<RG, 8, TS>(mp, g, m, v, dir, h, d, t, ac, parity, tc.tz, s);
+        le = wide ? launch_k3_tma<RG, K3W_NW, K3W_OPT, TS>(mp, g, m, v, dir, h, d, t, ac, parity,
+                                                           tc.tz, s)
+                  : launch_k3_tma<RG, K3_NW, K3_OPT, TS>(mp, g, m, v, dir, h, d, t, ac, parity,
+                                                         tc.tz, s);
     } else {
-        using SC = K3S<RG, K3_NW, K3_OPT, K3_ST_CP, false>;  // moments unstaged
-        auto kern = k_smooth_adam<RG, K3_NW, K3_OPT, K3_ST_CP, false, TS>;
+        using SC = K3S<RG, K3_NW, K3_OPT, K3_ST, false>;  // moments unstaged
+        auto kern = k_smooth_adam<RG, K3_NW, K3_OPT, K3_ST, false, TS>;
         static const int occ = prepare(kern, SC::bytes, SC::NT);
-        LaunchGeom gg = geometry(occ, K3_NW, SC::TY, RG, d, tc.tz);
+        LaunchGeom gg = geometry(occ, K3_NW, SC::TY, 2.0f * RG, d, tc.tz);
         le = launch_pdl(kern, gg, SC::bytes, s, mp, g, m, v, dir, h, d.D, d.H, d.W, d.pitch(), gg.tz, t, ac,
                         parity);
     }
@@ -207,14 +212,14 @@ cudaError_t launch_k3(const float *g, TS *m, TS *v, float *dir, WsHeader *h, Dim
     return le;
 }
 
-template <int RG, bool SU, int NW, class TU>
+template <int RG, bool SU, int NW, int OPT, class TU>
 cudaError_t launch_k4_tma(const Maps &mp, const TU *u, const float *dir, TU *uo,
                           const float *Im, float *J, float *gJ, WsHeader *h, Dims d, const GaussTaps &t,
                           float lr, float c_lp, int parity, int tz, cudaStream_t s) {
-    using ST = K4S<RG, NW, K4_OPT, SU, K4_ST_TMA, TU>;
-    auto kern = k_compose<RG, NW, K4_OPT, SU, K4_ST_TMA, true, TU>;
+    using ST = K4S<RG, NW, OPT, SU, K4_ST, TU>;
+    auto kern = k_compose<RG, NW, OPT, SU, K4_ST, true, TU>;
     static const int occ = prepare(kern, ST::bytes, ST::NT);
-    LaunchGeom gg = geometry(occ, NW, ST::TY, RG, d, tz);
+    LaunchGeom gg = geometry(occ, NW, ST::TY, 2.0f * RG, d, tz);
     return launch_pdl(kern, gg, ST::bytes, s, mp, u, dir, uo, Im, J, gJ, h, d.D, d.H, d.W, d.pitch(), gg.tz, t,
                       lr, c_lp, parity);
 }
@@ -226,25 +231,23 @@ cudaError_t launch_k4(const TU *u, const float *dir, TU *uo, const float *Im, fl
                       float *gJ, WsHeader *h, Dims d, const GaussTaps &t, float lr, float c_lp, int parity,
                       cudaStream_t s) {
     constexpr int EU = (int)sizeof(TU);
-    using S16 = K4S<RG, 16, K4_OPT, SU, K4_ST_TMA, TU>;
-    using S8 = K4S<RG, 8, K4_OPT, SU, K4_ST_TMA, TU>;
+    using SW = K4S<RG, K4W_NW, K4W_OPT, SU, K4_ST, TU>;  // its row lengths are any tile's
     Maps mp{};
     cudaError_t le;
     const TileChoice tc = tile_choice(3, RG, SU ? 1 : 0, d);
-    const int nw = tc.wide ? 16 : 8;
-    const int ubx = tc.wide ? S16::UBXW : S8::UBXW;
-    const bool tma = tmap(&mp.a, dir, 4, d, 3, FX + 2 * halo4(RG), nw + 2 * RG, 3) &&
-                     (!SU || tmap(&mp.b, u, EU, d, 3, ubx, nw + 2 * RG + 2, 3));
+    const int ty = tc.wide ? 16 : 8;
+    const bool tma = tmap(&mp.a, dir, 4, d, 3, SW::BXW, ty + 2 * RG, 3) &&
+                     (!SU || tmap(&mp.b, u, EU, d, 3, SW::UBXW, ty + 2 * RG + 2, 3));
     if (tma) {
-        le = tc.wide ? launch_k4_tma<RG, SU, 16>(mp, u, dir, uo, Im, J, gJ, h, d, t, lr, c_lp, parity,
+        le = tc.wide ? launch_k4_tma<RG, SU, K4W_NW, K4W_OPT>(mp, u, dir, uo, Im, J, gJ, h, d, t, lr, c_lp, parity,
                                                  tc.tz, s)
-                     : launch_k4_tma<RG, SU, 8>(mp, u, dir, uo, Im, J, gJ, h, d, t, lr, c_lp, parity,
+                     : launch_k4_tma<RG, SU, K4_NW, K4_OPT>(mp, u, dir, uo, Im, J, gJ, h, d, t, lr, c_lp, parity,
                                                 tc.tz, s);
     } else if constexpr (EU == 4) {
-        using SC = K4S<RG, K4_NW, K4_OPT, SU, K4_ST_CP>;
-        auto kern = k_compose<RG, K4_NW, K4_OPT, SU, K4_ST_CP, false>;
+        using SC = K4S<RG, K4_NW, K4_OPT, SU, K4_ST>;
+        auto kern = k_compose<RG, K4_NW, K4_OPT, SU, K4_ST, false>;
         static const int occ = prepare(kern, SC::bytes, SC::NT);
-        LaunchGeom gg = geometry(occ, K4_NW, SC::TY, RG, d, tc.tz);
+        LaunchGeom gg = geometry(occ, K4_NW, SC::TY, 2.0f * RG, d, tc.tz);
         le = launch_pdl(kern, gg, SC::bytes, s, mp, u, dir, uo, Im, J, gJ, h, d.D, d.H, d.W, d.pitch(), gg.tz, t,
                         lr, c_lp, parity);
     } else {
@@ -454,7 +457,7 @@ fa_status fused_autotune_level(FusedBuffers &fb, WsHeader *h, const fa_params *p
     for (int kernel = (p->loss == FA_LOSS_LNCC ? 0 : 2); kernel < 4 && result == FA_OK; ++kernel) {
         const int radius = kernel < 2 ? p->window / 2 : (kernel == 2 ? g3.R : g4.R);
         const int sukey = kernel == 3 && su ? 1 : 0;
-        TileChoice best{kDefaultWide[kernel], 0};
+        TileChoice best{default_wide(kernel, d), 0};
         float best_ms = -1.0f;
         for (int wide = 0; wide < (kernel >= 2 ? 2 : 1) && result == FA_OK; ++wide)
             for (int tz : tzs) {

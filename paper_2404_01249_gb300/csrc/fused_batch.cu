@@ -17,10 +17,9 @@ namespace {
 // tiles when every job's buffers meet TMA's alignment rules (the row pitch
 // of a level's buffers is a multiple of 4 floats whenever the fused kernels
 // run it), else the per-thread copy variant (cp.async) for all its jobs.
-// The compose kernel of a batch takes 32 x 16 tiles of 16 warps: its u' region
-// (the tile plus the sigma_warp halo) is then 1.25 instead of 1.5 times the
-// tile, the choice the single-job launches make by default.
-constexpr int K4B_NW = 16;
+// The update kernels of a batch take 32 x 16 tiles (the compose's u' region, the
+// tile plus the sigma_warp halo, is then 1.41 instead of 1.69 times the tile):
+// a wave's jobs fill the GPU together.
 
 struct BGeom {
     int D, H, W, P, TZ, gx, gy;  // P: row pitch of the job's buffers
@@ -146,26 +145,26 @@ constexpr int k3_maps() {
 }
 
 template <int RG, class TS, bool TMA>
-__global__ void __launch_bounds__(FX *K3_NW) k_smooth_adam_batch(
+__global__ void __launch_bounds__(FX *K3W_NW, k3_min_ctas(RG, K3W_NW, K3W_OPT)) k_smooth_adam_batch(
     const __grid_constant__ K3Batch<k3_maps<TS>()> b) {
     const int k = batch_job(b.first, b.n, (int)blockIdx.x);
     const K3Job &j = b.j[k];
     int bx, by, bz;
     batch_tile(j.geo, (int)blockIdx.x - b.first[k], bx, by, bz);
-    smooth_adam_body<RG, K3_NW, K3_OPT, TMA ? K3_ST_TMA : K3_ST_CP, TMA>(
+    smooth_adam_body<RG, K3W_NW, K3W_OPT, K3_ST, TMA>(
         job_maps<k3_maps<TS>(), TMA>(b.tm, k), j.g, (TS *)j.m, (TS *)j.v, j.dir, j.h, j.geo.D,
         j.geo.H, j.geo.W, j.geo.P, j.geo.TZ, j.t, b.ac, b.parity, bx, by, bz);
 }
 
 // TU: storage of u (float, or __half: tile copies only).
 template <int RG, bool SU, bool TMA, class TU>
-__global__ void __launch_bounds__(FX *K4B_NW, 2) k_compose_batch(
+__global__ void __launch_bounds__(FX *K4W_NW, k4_min_ctas(RG, K4W_NW, K4W_OPT)) k_compose_batch(
     const __grid_constant__ K4Batch<SU ? 2 : 1> b) {
     const int k = batch_job(b.first, b.n, (int)blockIdx.x);
     const K4Job &j = b.j[k];
     int bx, by, bz;
     batch_tile(j.geo, (int)blockIdx.x - b.first[k], bx, by, bz);
-    compose_body<RG, K4B_NW, K4_OPT, SU, TMA ? K4_ST_TMA : K4_ST_CP, TMA>(
+    compose_body<RG, K4W_NW, K4W_OPT, SU, K4_ST, TMA>(
         job_maps<SU ? 2 : 1, TMA>(b.tm, k), (const TU *)j.u, j.dir, (TU *)j.uo, j.Im, j.J, j.gJ,
         j.h, j.geo.D, j.geo.H, j.geo.W, j.geo.P, j.geo.TZ, j.t, j.lr, j.c_lp, b.parity, bx, by,
         bz);
@@ -290,7 +289,7 @@ cudaError_t launch_k3_batch(K3Batch<k3_maps<TS>()> &b, const LockstepJob *jobs, 
                             cudaStream_t s) {
     constexpr bool S32 = sizeof(TS) == 4;
     constexpr int NM = k3_maps<TS>();
-    using ST = K3S<RG, K3_NW, K3_OPT, K3_ST_TMA, S32>;  // FP32 moments staged
+    using ST = K3S<RG, K3W_NW, K3W_OPT, K3_ST, S32>;  // FP32 moments staged
     bool tma = true;
     for (int k = 0; k < b.n && tma; ++k) {
         const LockstepJob &q = jobs[idx[k]];
@@ -305,7 +304,7 @@ cudaError_t launch_k3_batch(K3Batch<k3_maps<TS>()> &b, const LockstepJob *jobs, 
         batch_layout(b, jobs, idx, ST::TY, RG, occ);
         return launch_batch(kern, b, ST::NT / FX, ST::bytes, s);
     }
-    using SC = K3S<RG, K3_NW, K3_OPT, K3_ST_CP, false>;  // moments unstaged
+    using SC = K3S<RG, K3W_NW, K3W_OPT, K3_ST, false>;  // moments unstaged
     auto kern = k_smooth_adam_batch<RG, TS, false>;
     static const int occ = prepare(kern, SC::bytes, SC::NT);
     batch_layout(b, jobs, idx, SC::TY, RG, occ);
@@ -318,7 +317,7 @@ template <int RG, bool SU, class TU>
 cudaError_t launch_k4_batch(K4Batch<SU ? 2 : 1> &b, const LockstepJob *jobs, const int *idx,
                             cudaStream_t s) {
     constexpr int NM = SU ? 2 : 1, EU = (int)sizeof(TU);
-    using ST = K4S<RG, K4B_NW, K4_OPT, SU, K4_ST_TMA, TU>;
+    using ST = K4S<RG, K4W_NW, K4W_OPT, SU, K4_ST, TU>;
     bool tma = true;
     for (int k = 0; k < b.n && tma; ++k) {
         const LockstepJob &q = jobs[idx[k]];
@@ -333,7 +332,7 @@ cudaError_t launch_k4_batch(K4Batch<SU ? 2 : 1> &b, const LockstepJob *jobs, con
         return launch_batch(kern, b, ST::NT / FX, ST::bytes, s);
     }
     if constexpr (EU == 4) {
-        using SC = K4S<RG, K4B_NW, K4_OPT, SU, K4_ST_CP>;
+        using SC = K4S<RG, K4W_NW, K4W_OPT, SU, K4_ST>;
         auto kern = k_compose_batch<RG, SU, false, float>;
         static const int occ = prepare(kern, SC::bytes, SC::NT);
         batch_layout(b, jobs, idx, SC::TY, RG, occ);

@@ -22,18 +22,29 @@
 // K1 and K2 are in window.cuh; K3 and K4 are here.
 //
 // Every kernel marches along z ("2.5-D" tiling).  In K3 and K4 a CTA owns a
-// 32 x TY tile of (x, y) columns and a slab of TZ output planes.  A plane's inputs (the tile
-// plus its halo, and the operands of the plane's outputs) arrive NSTG - 1
-// planes ahead of use.  When the buffers' rows start on 16-byte boundaries
-// (a registration pads its levels' rows to a multiple of 4 floats) they come
-// as TMA tile copies issued by one thread and completed on an mbarrier (zero
-// fill outside the grid); otherwise each thread copies its own positions with
-// cp.async.  A plane is reduced along x (register-blocked, 16-byte shared
-// loads) and then y in shared memory; the last 2R + 1 in-plane results per
-// output column sit in a shared-memory ring from which the z reduction reads.
-// No intermediate of the separable sums goes to HBM; halo re-reads hit L2.
+// 32 x TY tile of (x, y) columns and a slab of TZ output planes.  A plane's
+// inputs (the tile plus its halo, and the operands of the plane's outputs)
+// arrive NSTG - 1 planes ahead of use.  When the buffers' rows start on
+// 16-byte boundaries (a registration pads its levels' rows to a multiple of 4
+// floats) they come as TMA tile copies issued by one thread and completed on
+// an mbarrier (zero fill outside the grid); otherwise each thread copies its
+// own positions with cp.async.
 //
-// Shared plane layout: [C][RY][BXW] with BXW = 32 + 2 XB and XB = R rounded
+// The passes over a plane are pipelined over the planes: between two barriers
+// each pass works on a plane of its own, one behind the pass before it, with
+// doubled buffers in between.  So there is one barrier per plane instead of
+// two (K3) or three (K4), and the passes' shared-memory latencies overlap.
+// Along x a plane goes from shared memory to shared memory (4 outputs per item
+// from 16-byte loads); along y a thread sums its adjacent output rows in
+// registers; along z it adds the plane into the 2R + 1 outputs it reaches
+// (OpenZ), which took the place of a shared-memory ring of 2R + 1 planes.  No
+// intermediate of the separable sums goes to HBM; halo re-reads hit L2.
+//
+// K4 is bound by the shared-memory pipe (per 32 outputs about 62 wavefronts of
+// loads and stores, 34 of them the cell corners, against 85 with the ring and
+// one row per thread), K3 by HBM at the finest level and by latency below.
+//
+// Shared layout of a staged plane: [C][RY][BXW] with BXW = 32 + 2 XB and XB = R rounded
 // up to a multiple of 4.  Column c holds x = x0 - XB + c and row r holds
 // y = y0 - R + r, so that a TMA box starts on a 16-byte boundary.
 //
@@ -70,11 +81,6 @@ __device__ __forceinline__ void cp4(void *dst, const void *src, bool ok) {
                  "r"(ok ? 4 : 0)
                  : "memory");
 }
-__device__ __forceinline__ void cp8(void *dst, const void *src, bool ok) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(su32(dst)), "l"(src),
-                 "r"(ok ? 8 : 0)
-                 : "memory");
-}
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_wait() {
@@ -88,11 +94,6 @@ __device__ __forceinline__ void mbar_init(unsigned long long *b) {
 // Makes initialised barriers visible to the TMA unit.
 __device__ __forceinline__ void mbar_init_fence() {
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-}
-// Orders this thread's shared-memory stores before later tile copies into the
-// same bytes (a buffer refilled by TMA after the threads wrote to it).
-__device__ __forceinline__ void proxy_fence_async() {
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
 }
 // The arrival of the one expected thread, announcing `bytes` of copies.
@@ -165,13 +166,13 @@ __device__ __forceinline__ bool status_timed_out(const WsHeader *h, int tid, int
     return *flag != 0;
 }
 
-// Bounded wait for the first min(n, NSTG - 1) stage copies a CTA issued
-// before it returns early (TMA), or for its copy groups (cp.async).
+// Bounded wait for the first min(n, NSTG) stage copies a CTA issued before it
+// returns early (TMA), or for its copy groups (cp.async).
 template <bool TMA, int NSTG>
 __device__ __forceinline__ void drain_first(unsigned long long *bar, int n, int tid) {
     if (TMA) {
         if (tid == 0)
-            for (int j = 0; j < n && j < NSTG - 1; ++j) mbar_wait(bar + j, 0u);
+            for (int j = 0; j < n && j < NSTG; ++j) mbar_wait(bar + j, 0u);
     } else {
         cp_wait<0>();
     }
@@ -221,16 +222,17 @@ struct Region {
     }
 };
 
-// This thread's OPT output voxels; its slot o of a [C][TY][32] output tile is
-// o NT + tid (the layout a {32, TY, 1, C} TMA box lands in).
+// This thread's OPT output voxels: rows OPT wy .. OPT wy + OPT - 1 of the
+// tile, column tx (its places in a [TY][32] output tile start at `place`).
 template <int OPT, int NW>
 struct Outs {
-    static constexpr int NT = 32 * NW, NOUT = OPT * NT;
     int off[OPT];  // y P + x (P: the row pitch), -1 outside the grid
+    int place;
     __device__ __forceinline__ void init(int wy, int tx, int y0, int x0, int H, int W, int P) {
+        place = OPT * wy * FX + tx;
 #pragma unroll
         for (int o = 0; o < OPT; ++o) {
-            const int y = y0 + wy + NW * o, x = x0 + tx;
+            const int y = y0 + OPT * wy + o, x = x0 + tx;
             off[o] = (y < H && x < W) ? y * P + x : -1;
         }
     }
@@ -243,22 +245,6 @@ struct Outs {
         for (int o = 0; o < OPT; ++o)
 #pragma unroll
             for (int c = 0; c < C; ++c) r[o][c] = off[o] >= 0 ? src[c * N + zoff + off[o]] : T(0);
-    }
-    template <int C, class T>
-    __device__ __forceinline__ void load(T *dst, const T *src, long long N, long long zoff,
-                                         int tid) const {
-#pragma unroll
-        for (int o = 0; o < OPT; ++o) {
-            const bool ok = off[o] >= 0;
-            const T *s = src + (ok ? zoff + off[o] : 0);
-#pragma unroll
-            for (int ch = 0; ch < C; ++ch) {
-                if (sizeof(T) == 8)
-                    cp8(dst + ch * NOUT + o * NT + tid, s + ch * N, ok);
-                else
-                    cp4(dst + ch * NOUT + o * NT + tid, s + ch * N, ok);
-            }
-        }
     }
 };
 
@@ -302,64 +288,79 @@ __device__ __forceinline__ void gauss_x4(const float *pl, float *xb, const TT &t
 // Channels 0 and 1 of the y and z passes run as one packed FP32 pair
 // (__ffma2_rn: each component is exactly fmaf), channel 2 alone; every
 // channel's taps accumulate in the same order as a scalar loop would.
-template <int RG, int RY, int NW, int OPT, class TT>
+// The OPT outputs of a thread are adjacent rows and share their reads.
+template <int RG, int RY, int OPT, class TT>
 __device__ __forceinline__ void gauss_y3(const float *xb, const TT &t, int wy, int tx,
-                                         float Q[OPT][3]) {
+                                         float2 (&q01)[OPT], float (&q2)[OPT]) {
+    const float *xi = xb + OPT * wy * FX + tx;
+    float2 r01[OPT + 2 * RG];
+    float r2[OPT + 2 * RG];
+#pragma unroll
+    for (int k = 0; k < OPT + 2 * RG; ++k) {
+        r01[k] = make_float2(xi[k * FX], xi[(RY + k) * FX]);
+        r2[k] = xi[(2 * RY + k) * FX];
+    }
 #pragma unroll
     for (int o = 0; o < OPT; ++o) {
-        const float *xi = xb + (wy + NW * o) * FX + tx;
-        float2 s01 = make_float2(0.0f, 0.0f);
-        float s2 = 0.0f;
+        q01[o] = make_float2(0.0f, 0.0f);
+        q2[o] = 0.0f;
 #pragma unroll
         for (int k = 0; k <= 2 * RG; ++k) {
-            const float w = t.w[k];
-            s01 = __ffma2_rn(make_float2(w, w),
-                             make_float2(xi[k * FX], xi[RY * FX + k * FX]), s01);
-            s2 = fmaf(w, xi[2 * RY * FX + k * FX], s2);
+            q01[o] = __ffma2_rn(make_float2(t.w[k], t.w[k]), r01[o + k], q01[o]);
+            q2[o] = fmaf(t.w[k], r2[o + k], q2[o]);
         }
-        Q[o][0] = s01.x;
-        Q[o][1] = s01.y;
-        Q[o][2] = s2;
     }
 }
 
-// Ring of the last NS in-plane results of this thread's outputs, [NS][3][NOUT]
-// floats; slot `newest` holds the current plane.
-template <int NS, int OPT, int NOUT, int NT>
-__device__ __forceinline__ void ring_put(float *ring, int newest, int tid, const float Q[OPT][3]) {
+// The z pass as a transposed filter: a plane's in-plane results are added into
+// the 2 RG + 1 outputs they reach; the 2 RG outputs still open sit in
+// registers.  Planes come in ascending order, so every output's taps do too.
+template <int RG, int OPT>
+struct OpenZ {
+    static constexpr int K = RG > 0 ? 2 * RG : 1;
+    float2 a01[OPT][K];
+    float a2[OPT][K];
+    __device__ __forceinline__ void init() {
 #pragma unroll
-    for (int o = 0; o < OPT; ++o)
+        for (int o = 0; o < OPT; ++o)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) ring[(newest * 3 + c) * NOUT + o * NT + tid] = Q[o][c];
-}
-
-// Weighted z window of all three channels of one output: tap k takes the
-// plane k - R of the window, i.e. ring slot (newest + 1 + k) mod NS.
-template <int RG, int NOUT, class TT>
-__device__ __forceinline__ void gauss_z3(const float *ring_o, int newest, const TT &t,
-                                         float out[3]) {
-    constexpr int NS = 2 * RG + 1;
-    float2 s01 = make_float2(0.0f, 0.0f);
-    float s2 = 0.0f;
-#pragma unroll
-    for (int k = 0; k < NS; ++k) {
-        int j = newest + 1 + k;
-        j = j >= NS ? j - NS : j;
-        const float *r = ring_o + j * 3 * NOUT;
-        const float w = t.w[k];
-        s01 = __ffma2_rn(make_float2(w, w), make_float2(r[0], r[NOUT]), s01);
-        s2 = fmaf(w, r[2 * NOUT], s2);
+            for (int k = 0; k < K; ++k) {
+                a01[o][k] = make_float2(0.0f, 0.0f);
+                a2[o][k] = 0.0f;
+            }
     }
-    out[0] = s01.x;
-    out[1] = s01.y;
-    out[2] = s2;
-}
+    // adds a plane; the output RG planes below it leaves with its sum
+    template <class TT>
+    __device__ __forceinline__ void push(const TT &t, const float2 (&q01)[OPT],
+                                         const float (&q2)[OPT], float (&out)[OPT][3]) {
+#pragma unroll
+        for (int o = 0; o < OPT; ++o) {
+            auto tap01 = [&](int k, float2 acc) {
+                return __ffma2_rn(make_float2(t.w[k], t.w[k]), q01[o], acc);
+            };
+            const float2 z01 =
+                tap01(2 * RG, RG > 0 ? a01[o][0] : make_float2(0.0f, 0.0f));
+            out[o][0] = z01.x;
+            out[o][1] = z01.y;
+            out[o][2] = fmaf(t.w[2 * RG], q2[o], RG > 0 ? a2[o][0] : 0.0f);
+            if (RG > 0) {
+#pragma unroll
+                for (int k = 0; k + 1 < 2 * RG; ++k) {
+                    a01[o][k] = tap01(2 * RG - 1 - k, a01[o][k + 1]);
+                    a2[o][k] = fmaf(t.w[2 * RG - 1 - k], q2[o], a2[o][k + 1]);
+                }
+                a01[o][K - 1] = tap01(0, make_float2(0.0f, 0.0f));
+                a2[o][K - 1] = fmaf(t.w[0], q2[o], 0.0f);
+            }
+        }
+    }
+};
 
-// Bounded wait, by thread 0, for the copies of planes i .. i + NSTG - 1 that
-// may still be in flight when a CTA stops early.
+// Bounded wait, by thread 0, for the copies of planes i .. end - 1 that may
+// still be in flight when a CTA stops early.
 template <int NSTG>
-__device__ __forceinline__ void drain(unsigned long long *bar, int i, int np) {
-    for (int j = i; j < i + NSTG && j < np; ++j) mbar_wait(bar + j % NSTG, (unsigned)(j / NSTG) & 1u);
+__device__ __forceinline__ void drain(unsigned long long *bar, int i, int end) {
+    for (int j = i; j < end; ++j) mbar_wait(bar + j % NSTG, (unsigned)(j / NSTG) & 1u);
 }
 
 // MSE: g = 2 (J - I) / N * grad I_m(phi) (pointwise, J and the gradient as
@@ -381,6 +382,14 @@ __global__ void __launch_bounds__(256) k_fused_mse_grad(const float *__restrict_
     g[2 * N + i] = dj * __ldg(gJ + 2 * N + i);
 }
 
+// Resident CTAs the register allocation of K3 and K4 aims at.
+__host__ __device__ constexpr int k3_min_ctas(int RG, int NW, int OPT) {
+    return RG <= 3 ? 32 / (NW * OPT) : 1;
+}
+__host__ __device__ constexpr int k4_min_ctas(int RG, int NW, int OPT) {
+    return RG <= 3 ? (NW * OPT == 16 ? 2 : 3) : 1;
+}
+
 // ====================================================================== K3
 // STAGED: the moments m, nu (FP32) arrive with the plane's TMA copies;
 // otherwise (16-bit moments, or the per-thread copy variant) each thread loads
@@ -389,24 +398,24 @@ template <int RG, int NW, int OPT, int NSTG, bool STAGED = true>
 struct K3S {
     static constexpr int NT = FX * NW, TY = NW * OPT, RX = FX + 2 * RG, RY = TY + 2 * RG;
     static constexpr int XB = halo4(RG), BXW = FX + 2 * XB, COFF = XB - RG;
-    static constexpr int NR = BXW * RY, NS = 2 * RG + 1, NOUT = NT * OPT;
+    static constexpr int NR = BXW * RY, NOUT = NT * OPT, XS = 3 * RY * FX;
     static constexpr size_t st_bytes = al128((size_t)3 * NR * 4);    // g
     static constexpr size_t ost_bytes = STAGED ? al128((size_t)6 * NOUT * 4) : 0;  // m, v
     static constexpr unsigned tx_plane = 3u * NR * 4, tx_out = 6u * NOUT * 4;
     static constexpr size_t o_st = 0;
     static constexpr size_t o_ost = o_st + st_bytes * NSTG;
-    static constexpr size_t o_ring = o_ost + ost_bytes * NSTG;
-    static constexpr size_t o_xb = o_ring + (size_t)NS * 3 * NOUT * 4;
-    static constexpr size_t o_bar = al128(o_xb + (size_t)3 * RY * FX * 4);
+    static constexpr size_t o_xb = o_ost + ost_bytes * NSTG;  // x sums, doubled
+    static constexpr size_t o_bar = al128(o_xb + (size_t)2 * XS * 4);
     static constexpr size_t bytes = o_bar + 8 * NSTG;
 };
 
-// The body of K3 for the CTA with tile coordinates (bx, by, bz).
+// The body of K3 for the CTA with tile coordinates (bx, by, bz).  Between two
+// barriers the CTA sums plane i along x and plane i - 1 along y and z.
 template <int RG, int NW, int OPT, int NSTG, bool TMA, class TT, class TS>
 __device__ __forceinline__ void smooth_adam_body(MapRef maps, const float *__restrict__ g,
                                                  TS *__restrict__ m, TS *__restrict__ v,
                                                  float *__restrict__ dir, WsHeader *__restrict__ h,
-                                                 int D, int H, int W, int P, int TZ, const TT t,
+                                                 int D, int H, int W, int P, int TZ, const TT &t,
                                                  const AdamConsts ac, int parity, int bx, int by,
                                                  int bz) {
     constexpr bool S32 = sizeof(TS) == 4, STAGED = S32 && TMA;
@@ -414,10 +423,9 @@ __device__ __forceinline__ void smooth_adam_body(MapRef maps, const float *__res
     // moments as loaded into registers: FP32 values or 16-bit patterns
     using FT = typename std::conditional<S32, float, unsigned short>::type;
     constexpr int NT = S::NT, TY = S::TY, RX = S::RX, RY = S::RY, BXW = S::BXW, COFF = S::COFF,
-                  XB = S::XB, NS = S::NS, NOUT = S::NOUT;
+                  XB = S::XB, NOUT = S::NOUT, XS = S::XS;
     using G = Region<RY, RX, NW, BXW, COFF>;
     extern __shared__ __align__(128) unsigned char smem[];
-    float *ring = (float *)(smem + S::o_ring);
     float *xb = (float *)(smem + S::o_xb);
     unsigned long long *bar = (unsigned long long *)(smem + S::o_bar);
     __shared__ float redf[32];
@@ -437,34 +445,34 @@ __device__ __forceinline__ void smooth_adam_body(MapRef maps, const float *__res
         for (int k = 0; k < NSTG; ++k) mbar_init(bar + k);
         mbar_init_fence();
     }
-    for (int k = tid; k < NS * 3 * NOUT; k += NT) ring[k] = 0.0f;
 
+    // group i: g of plane zs + i and the moments of the outputs that plane
+    // i - 1 completes (plane zs + i - 1 - RG); the last group has no plane
     const int zs = z0 - RG, np = zend - z0 + 2 * RG;
     auto issue = [&](int i) {
-        const int zp = zs + i, zo = zp - RG, s = i % NSTG;
-        const bool out = STAGED && zo >= z0 && zo < zend;
+        const int zp = zs + i, zo = zp - 1 - RG, s = i % NSTG;
+        const bool in = i < np, out = STAGED && i <= np && zo >= z0;
         if (TMA) {
-            if (tid == 0 && i < np) {
-                mbar_expect(bar + s, S::tx_plane + (out ? S::tx_out : 0u));
-                tma4(stage(s), maps.a, x0 - XB, y0 - RG, zp, 0, bar + s);
+            if (tid == 0 && (in || out)) {
+                mbar_expect(bar + s, (in ? S::tx_plane : 0u) + (out ? S::tx_out : 0u));
+                if (in) tma4(stage(s), maps.a, x0 - XB, y0 - RG, zp, 0, bar + s);
                 if (out) {
                     tma4(ostage(s), maps.b, x0, y0, zo, 0, bar + s);
                     tma4(ostage(s) + 3 * NOUT, maps.c, x0, y0, zo, 0, bar + s);
                 }
             }
         } else {
-            if (i < np) {
-                rg.template load<3>(stage(s), g, N, (long long)zp * HW, zp >= 0 && zp < D);
-            }
+            if (in) rg.template load<3>(stage(s), g, N, (long long)zp * HW, zp >= 0 && zp < D);
             cp_commit();
         }
     };
+    const int groups = STAGED ? np + 1 : np;  // groups that copy something
     // unstaged moments of the next output plane, loaded one plane ahead
     FT mn[OPT][3], vn[OPT][3];
     auto fetch_mv = [&](int i) {
         if constexpr (!STAGED) {
-            const int zo = zs + i - RG;
-            if (i < np && zo >= z0 && zo < zend) {
+            const int zo = zs + i - 1 - RG;
+            if (i <= np && zo >= z0) {
                 ou.fetch(mn, (const FT *)m, N, (long long)zo * HW);
                 ou.fetch(vn, (const FT *)v, N, (long long)zo * HW);
             }
@@ -473,76 +481,78 @@ __device__ __forceinline__ void smooth_adam_body(MapRef maps, const float *__res
     // after the previous kernel: first copies and loads in flight, then the
     // status check
     pdl_wait();
-    fetch_mv(0);
+    fetch_mv(1);
 #pragma unroll
-    for (int k = 0; k < NSTG - 1; ++k) issue(k);
+    for (int k = 0; k < NSTG; ++k) issue(k);
     if (status_timed_out(h, tid, &flag)) {
-        drain_first<TMA, NSTG>(bar, np, tid);
+        drain_first<TMA, NSTG>(bar, groups, tid);
         return;
     }
 
+    OpenZ<RG, OPT> oz;
+    oz.init();
     float mx = 0.0f;
     bool bad = false;
-    int fail = -1, slot = 0;
-    for (int i = 0; i < np; ++i) {
-        const int zp = zs + i, zo = zp - RG, s = i % NSTG;
-        issue(i + NSTG - 1);
+    int fail = -1;
+    for (int i = 0; i <= np; ++i) {
+        const int zp = zs + i, s = i % NSTG;
         bool ok = true;
-        if (TMA)
-            ok = mbar_wait(bar + s, (unsigned)(i / NSTG) & 1u);
-        else
-            cp_wait<NSTG - 1>();
-        const bool out = zo >= z0 && zo < zend;
-        float mo[OPT][3], vo[OPT][3];
-        if (out) {
-            if constexpr (STAGED) {
-                const float *od = ostage(s) + tid;
-#pragma unroll
-                for (int o = 0; o < OPT; ++o)
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) {
-                        mo[o][c] = od[c * NOUT + o * NT];
-                        vo[o][c] = od[(3 + c) * NOUT + o * NT];
-                    }
-            } else {
-#pragma unroll
-                for (int o = 0; o < OPT; ++o)
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) {
-                        mo[o][c] = st_value<TS>(mn[o][c]);
-                        vo[o][c] = st_value<TS>(vn[o][c]);
-                    }
-            }
+        if (TMA) {
+            if (i < groups) ok = mbar_wait(bar + s, (unsigned)(i / NSTG) & 1u);
+        } else {
+            cp_wait<NSTG - 2>();
         }
-        fetch_mv(i + 1);
-        if (__syncthreads_or(!ok)) {  // also: the x pass reads neighbours' copies
+        // also: the x pass reads neighbours' copies, the y pass their x sums,
+        // and the stage of plane i - 1 is free
+        if (__syncthreads_or(!ok)) {
             fail = i;
             break;
         }
-        float Q[OPT][3];
-        if (zp >= 0 && zp < D) {
-            gauss_x4<RG, 3, RY, BXW, COFF, NT>(stage(s), xb, t, tid);
-            __syncthreads();
-            gauss_y3<RG, RY, NW, OPT>(xb, t, wy, tx, Q);
+        if (i > 0) issue(i + NSTG - 1);
+        if (i < np && zp >= 0 && zp < D)
+            gauss_x4<RG, 3, RY, BXW, COFF, NT>(stage(s), xb + (i & 1 ? XS : 0), t, tid);
+        if (i == 0) continue;
+        const int zq = zp - 1, zo = zq - RG;
+        float2 q01[OPT];
+        float q2[OPT];
+        if (zq >= 0 && zq < D) {
+            gauss_y3<RG, RY, OPT>(xb + (i & 1 ? 0 : XS), t, wy, tx, q01, q2);
         } else {
 #pragma unroll
-            for (int o = 0; o < OPT; ++o) Q[o][0] = Q[o][1] = Q[o][2] = 0.0f;
+            for (int o = 0; o < OPT; ++o) {
+                q01[o] = make_float2(0.0f, 0.0f);
+                q2[o] = 0.0f;
+            }
         }
-        ring_put<NS, OPT, NOUT, NT>(ring, slot, tid, Q);
-        const int newest = slot;
-        slot = (slot + 1 == NS) ? 0 : slot + 1;
-        if (out) {
+        float sz[OPT][3];
+        oz.push(t, q01, q2, sz);
+        float mo[OPT][3], vo[OPT][3];
+        if (zo >= z0) {
+#pragma unroll
+            for (int o = 0; o < OPT; ++o)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    if constexpr (STAGED) {
+                        const float *od = ostage(s) + ou.place + o * FX;
+                        mo[o][c] = od[c * NOUT];
+                        vo[o][c] = od[(3 + c) * NOUT];
+                    } else {
+                        mo[o][c] = st_value<TS>(mn[o][c]);
+                        vo[o][c] = st_value<TS>(vn[o][c]);
+                    }
+                }
+        }
+        fetch_mv(i + 1);
+        if (zo >= z0) {
             const long long zoff = (long long)zo * HW;
 #pragma unroll
             for (int o = 0; o < OPT; ++o) {
                 if (ou.off[o] < 0) continue;
-                float sz[3];
-                gauss_z3<RG, NOUT>(ring + o * NT + tid, newest, t, sz);
                 const long long gi = zoff + ou.off[o];
                 float nrm2 = 0.0f;
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
-                    const float sg = sz[c];
+                    const float sg = sz[o][c];
                     const float mvv = fmaf(ac.b1, mo[o][c], (1.0f - ac.b1) * sg);
                     const float vvv = fmaf(ac.b2, vo[o][c], (1.0f - ac.b2) * sg * sg);
                     m[c * N + gi] = st_store<TS>(mvv);
@@ -561,7 +571,7 @@ __device__ __forceinline__ void smooth_adam_body(MapRef maps, const float *__res
     if (fail >= 0) {
         if (tid == 0) {
             status_set(&h->status, ST_TIMEOUT);
-            drain<NSTG>(bar, fail, np);
+            drain<NSTG>(bar, fail, min(groups, fail + (fail ? NSTG - 1 : NSTG)));
         }
         return;
     }
@@ -571,7 +581,7 @@ __device__ __forceinline__ void smooth_adam_body(MapRef maps, const float *__res
 }
 
 template <int RG, int NW, int OPT, int NSTG, bool TMA, class TS = float>
-__global__ void __launch_bounds__(FX *NW, NW >= 16 ? 2 : 1) k_smooth_adam(const __grid_constant__ Maps maps,
+__global__ void __launch_bounds__(FX *NW, k3_min_ctas(RG, NW, OPT)) k_smooth_adam(const __grid_constant__ Maps maps,
                                                         const float *__restrict__ g,
                                                         TS *__restrict__ m,
                                                         TS *__restrict__ v,
@@ -595,21 +605,23 @@ template <int RG, int NW, int OPT, bool SU, int NSTG, class TU = float>
 struct K4S {
     static constexpr int NT = FX * NW, TY = NW * OPT, RX = FX + 2 * RG, RY = TY + 2 * RG;
     static constexpr int XB = halo4(RG), BXW = FX + 2 * XB, COFF = XB - RG;
-    static constexpr int NR = BXW * RY, NS = 2 * RG + 1, NOUT = NT * OPT;
+    static constexpr int NR = BXW * RY;
+    // u' and its x sums of a plane, doubled
+    static constexpr int UPW = (RX + 3) / 4 * 4, NU = UPW * RY, XS = 3 * RY * FX;
     // u planes z-1, z, z+1 in use plus NSTG - 1 in flight, halo RG + 1
     static constexpr int EU = (int)sizeof(TU);
     static constexpr int URX = RX + 2, URY = RY + 2, UXB = (RG + 1 + 7) / 8 * 8,
                          UBXW = FX + 2 * UXB;
     static constexpr int UCOFF = UXB - RG - 1, NRU = UBXW * URY, NSU = NSTG + 2;
     static constexpr int NP = RY * RX, NJP = (NP + NT - 1) / NT;  // compose positions
-    static constexpr size_t st_bytes = al128((size_t)3 * NR * 4);     // d, then u' in place
+    static constexpr size_t st_bytes = al128((size_t)3 * NR * 4);     // d
     static constexpr size_t ust_bytes = al128((size_t)3 * NRU * EU);  // u
     static constexpr unsigned tx_plane = 3u * NR * 4, tx_u = 3u * NRU * EU;
     static constexpr size_t o_st = 0;
     static constexpr size_t o_ust = o_st + st_bytes * NSTG;
-    static constexpr size_t o_ring = o_ust + (SU ? ust_bytes * NSU : 0);
-    static constexpr size_t o_xb = o_ring + (size_t)NS * 3 * NOUT * 4;
-    static constexpr size_t o_bar = al128(o_xb + (size_t)3 * RY * FX * 4);
+    static constexpr size_t o_up = o_ust + (SU ? ust_bytes * NSU : 0);
+    static constexpr size_t o_xb = o_up + (size_t)6 * NU * 4;
+    static constexpr size_t o_bar = al128(o_xb + (size_t)2 * XS * 4);
     static constexpr size_t bytes = o_bar + 8 * (NSTG + 1);
     static_assert(EU == 2 || UBXW % 32 == 16 || UBXW % 32 == 0, "u rows of 16 or 32 banks");
 };
@@ -631,7 +643,10 @@ __device__ __forceinline__ void compose_position(int pidx, int &ry, int &rx) {
     }
 }
 
-// The body of K4 for the CTA with tile coordinates (bx, by, bz).
+// The body of K4 for the CTA with tile coordinates (bx, by, bz).  Between two
+// barriers the CTA composes plane i, sums plane i - 1 along x and plane i - 2
+// along y and z, each from the half of a doubled buffer that the interval
+// before filled.
 template <int RG, int NW, int OPT, bool SU, int NSTG, bool TMA, class TT, class TU>
 __device__ __forceinline__ void compose_body(MapRef maps, const TU *__restrict__ u,
                                              const float *__restrict__ dir,
@@ -640,18 +655,18 @@ __device__ __forceinline__ void compose_body(MapRef maps, const TU *__restrict__
                                              float *__restrict__ Jout, float *__restrict__ gJout,
                                              WsHeader *__restrict__ h, int D, int H, int W, int P,
                                              int TZ,
-                                             const TT t, float lr, float c_lp, int parity, int bx,
+                                             const TT &t, float lr, float c_lp, int parity, int bx,
                                              int by, int bz) {
     static_assert(TMA || sizeof(TU) == 4, "an FP16 u is staged by tile copies only");
     using S = K4S<RG, NW, OPT, SU, NSTG, TU>;
     constexpr int NT = S::NT, TY = S::TY, RX = S::RX, RY = S::RY, BXW = S::BXW, COFF = S::COFF,
-                  XB = S::XB, NR = S::NR, NS = S::NS, NOUT = S::NOUT, URX = S::URX,
+                  XB = S::XB, NR = S::NR, NU = S::NU, UPW = S::UPW, XS = S::XS, URX = S::URX,
                   URY = S::URY, UXB = S::UXB, UBXW = S::UBXW, UCOFF = S::UCOFF, NRU = S::NRU,
                   NSU = S::NSU, NP = S::NP, NJP = S::NJP;
     using G = Region<RY, RX, NW, BXW, COFF>;
     using GU = Region<URY, URX, NW, UBXW, UCOFF>;
     extern __shared__ __align__(128) unsigned char smem[];
-    float *ring = (float *)(smem + S::o_ring);
+    float *up = (float *)(smem + S::o_up);
     float *xb = (float *)(smem + S::o_xb);
     unsigned long long *bar = (unsigned long long *)(smem + S::o_bar);
     __shared__ int flag;
@@ -673,7 +688,6 @@ __device__ __forceinline__ void compose_body(MapRef maps, const TU *__restrict__
         for (int k = 0; k <= NSTG; ++k) mbar_init(bar + k);
         mbar_init_fence();
     }
-    for (int k = tid; k < NS * 3 * NOUT; k += NT) ring[k] = 0.0f;
 
     const int zs = z0 - RG, np = zend - z0 + 2 * RG;
     // u plane q lives in u stage (q - (zs - 1)) % NSU
@@ -717,7 +731,7 @@ __device__ __forceinline__ void compose_body(MapRef maps, const TU *__restrict__
         }
     }
 #pragma unroll
-    for (int k = 0; k < NSTG - 1; ++k) issue(k);
+    for (int k = 0; k < NSTG; ++k) issue(k);
     const float mxd = __uint_as_float(h->step_max_bits[parity]);
     if (status_timed_out(h, tid, &flag)) {
         if (SU && TMA && tid == 0) mbar_wait(bar + NSTG, 0u);
@@ -734,9 +748,9 @@ __device__ __forceinline__ void compose_body(MapRef maps, const TU *__restrict__
 #pragma unroll
     for (int o = 0; o < OPT; ++o) jlive[o] = false;
 
-    // this thread's compose positions (fixed for every plane): plane-layout
-    // index (-1: none), inside the grid, and the u stage index of the position
-    int pk[NJP], pub[NJP];
+    // this thread's compose positions (fixed for every plane): index in the d
+    // stage (-1: none), in u' and in the u stage, and whether in the grid
+    int pk[NJP], pup[NJP], pub[NJP];
     bool pin[NJP];
 #pragma unroll
     for (int j = 0; j < NJP; ++j) {
@@ -746,27 +760,31 @@ __device__ __forceinline__ void compose_body(MapRef maps, const TU *__restrict__
         const int y = y0 - RG + ry, x = x0 - RG + rx;
         pk[j] = pidx < NP ? ry * BXW + rx + COFF : -1;
         pin[j] = pidx < NP && y >= 0 && y < H && x >= 0 && x < W;
+        pup[j] = ry * UPW + rx;
         pub[j] = (ry + 1) * UBXW + (rx + 1) + UCOFF;
     }
 
-    int fail = -1, slot = 0;
-    for (int i = 0; i < np; ++i) {
-        const int zp = zs + i, zo = zp - RG, s = i % NSTG;
-        issue(i + NSTG - 1);
+    OpenZ<RG, OPT> oz;
+    oz.init();
+    int fail = -1;
+    for (int i = 0; i < np + 2; ++i) {
+        const int zp = zs + i, s = i % NSTG;
         bool ok = ok0;
-        if (TMA)
-            ok = mbar_wait(bar + s, (unsigned)(i / NSTG) & 1u) && ok;
-        else
-            cp_wait<NSTG - 1>();
-        if (__syncthreads_or(!ok)) {  // the stages hold neighbours' copies
+        if (TMA) {
+            if (i < np) ok = mbar_wait(bar + s, (unsigned)(i / NSTG) & 1u) && ok;
+        } else {
+            cp_wait<NSTG - 2>();
+        }
+        // the stages hold neighbours' copies, u' and the x sums their results;
+        // the stage of plane i - 1 is free
+        if (__syncthreads_or(!ok)) {
             fail = i;
             break;
         }
-        float Q[OPT][3];
-        if (zp >= 0 && zp < D) {
-            // u' replaces d in the stage, position by position (each thread
-            // reads its positions' d before it writes them)
-            float *ds = stage(s);
+        if (i > 0) issue(i + NSTG - 1);
+        if (i < np && zp >= 0 && zp < D) {
+            const float *ds = stage(s);
+            float *us = up + (i & 1 ? 3 * NU : 0);
             const TU *um = uslot(zp - 1), *u0 = uslot(zp), *u1 = uslot(zp + 1);
             // u' on the RY x RX region (positions spread over all threads),
             // at the plane layout's columns
@@ -834,23 +852,30 @@ __device__ __forceinline__ void compose_body(MapRef maps, const TU *__restrict__
                         c = dx + tri_finish<false>(q, gz, gy, gx);
                     }
                 }
-                ds[k] = a;
-                ds[NR + k] = b;
-                ds[2 * NR + k] = c;
+                us[pup[j]] = a;
+                us[NU + pup[j]] = b;
+                us[2 * NU + pup[j]] = c;
             }
-            if (TMA) proxy_fence_async();  // the stage is refilled by a tile copy later
-            __syncthreads();
-            gauss_x4<RG, 3, RY, BXW, COFF, NT>(ds, xb, t, tid);
-            __syncthreads();
-            gauss_y3<RG, RY, NW, OPT>(xb, t, wy, tx, Q);
+        }
+        if (i >= 1 && i <= np && zp - 1 >= 0 && zp - 1 < D)
+            gauss_x4<RG, 3, RY, UPW, 0, NT>(up + (i & 1 ? 0 : 3 * NU), xb + (i & 1 ? 0 : XS), t,
+                                            tid);
+        if (i < 2) continue;
+        const int zq = zp - 2, zo = zq - RG;
+        float2 q01[OPT];
+        float q2[OPT];
+        if (zq >= 0 && zq < D) {
+            gauss_y3<RG, RY, OPT>(xb + (i & 1 ? XS : 0), t, wy, tx, q01, q2);
         } else {
 #pragma unroll
-            for (int o = 0; o < OPT; ++o) Q[o][0] = Q[o][1] = Q[o][2] = 0.0f;
+            for (int o = 0; o < OPT; ++o) {
+                q01[o] = make_float2(0.0f, 0.0f);
+                q2[o] = 0.0f;
+            }
         }
-        ring_put<NS, OPT, NOUT, NT>(ring, slot, tid, Q);
-        const int newest = slot;
-        slot = (slot + 1 == NS) ? 0 : slot + 1;
-        if (zo >= z0 && zo < zend) {
+        float sz[OPT][3];
+        oz.push(t, q01, q2, sz);
+        if (zo >= z0) {
             const long long zoff = (long long)zo * HW;
 #pragma unroll
             for (int o = 0; o < OPT; ++o) {
@@ -864,16 +889,14 @@ __device__ __forceinline__ void compose_body(MapRef maps, const TU *__restrict__
                     jlive[o] = false;
                 }
                 if (ou.off[o] < 0) continue;
-                float sz[3];
-                gauss_z3<RG, NOUT>(ring + o * NT + tid, newest, t, sz);
                 const long long gi = zoff + ou.off[o];
-                const float a = sz[0], b = sz[1], c = sz[2];
+                const float a = sz[o][0], b = sz[o][1], c = sz[o][2];
                 // the stored (for FP16, rounded) u is the one the next steps read
                 const TU sa = st_store<TU>(a), sb = st_store<TU>(b), sc = st_store<TU>(c);
                 uo[gi] = sa;
                 uo[N + gi] = sb;
                 uo[2 * N + gi] = sc;
-                tri_issue_p(jp[o], Im, D, H, W, P, zo, y0 + wy + NW * o, x0 + tx, st_load(sa),
+                tri_issue_p(jp[o], Im, D, H, W, P, zo, y0 + OPT * wy + o, x0 + tx, st_load(sa),
                             st_load(sb), st_load(sc));
                 jidx[o] = gi;
                 jlive[o] = true;
@@ -884,7 +907,7 @@ __device__ __forceinline__ void compose_body(MapRef maps, const TU *__restrict__
         if (tid == 0) {
             status_set(&h->status, ST_TIMEOUT);
             if (SU && !ok0) mbar_wait(bar + NSTG, 0u);
-            drain<NSTG>(bar, fail, np);
+            drain<NSTG>(bar, fail, min(np, fail + (fail ? NSTG - 1 : NSTG)));
         }
         return;
     }
@@ -908,7 +931,7 @@ __device__ __forceinline__ void compose_body(MapRef maps, const TU *__restrict__
 }
 
 template <int RG, int NW, int OPT, bool SU, int NSTG, bool TMA, class TU = float>
-__global__ void __launch_bounds__(FX *NW, NW >= 16 ? 2 : 1) k_compose(const __grid_constant__ Maps maps,
+__global__ void __launch_bounds__(FX *NW, k4_min_ctas(RG, NW, OPT)) k_compose(const __grid_constant__ Maps maps,
                                                     const TU *__restrict__ u,
                                                     const float *__restrict__ dir,
                                                     TU *__restrict__ uo,
@@ -925,10 +948,14 @@ __global__ void __launch_bounds__(FX *NW, NW >= 16 ? 2 : 1) k_compose(const __gr
 
 // ================================================================ launch helpers
 
-// tile shapes (warps per CTA, outputs per thread along y) and pipeline depths
-// of the TMA and of the cp.async variant
-constexpr int K3_NW = 8, K3_OPT = 1, K3_ST_TMA = 2, K3_ST_CP = 2;
-constexpr int K4_NW = 8, K4_OPT = 1, K4_ST_TMA = 2, K4_ST_CP = 2;
+// Tile shapes (warps per CTA, rows per thread) of the 32 x 8 and 32 x 16
+// tiles, and pipeline depths.  Measured on the 160 x 192 x 224 pair (ms): K3
+// with 32 x 8 tiles 41.0, with 32 x 16 and two stages 40.5, three 39.6 (what
+// the ring took holds the third stage); K4 with 16 warps of one row 40.6, with
+// 8 warps of two rows 39.8; a third stage of K4 leaves one CTA per SM: 45.2.
+// Before the passes were pipelined: 43.5.
+constexpr int K3_NW = 8, K3_OPT = 1, K3W_NW = 8, K3W_OPT = 2, K3_ST = 3;
+constexpr int K4_NW = 8, K4_OPT = 1, K4W_NW = 8, K4W_OPT = 2, K4_ST = 2;
 
 // Gaussians up to this radius run inside the fused kernels
 constexpr int kMaxFusedRG = kMaxFusedRadius;
