@@ -423,6 +423,20 @@ fa_status fused_iteration(FusedBuffers &fb, WsHeader *h, const fa_params *p, Dim
     return FA_OK;
 }
 
+bool fused_update_takes(const fa_params *p, const GaussTaps &tg, const GaussTaps &tw) {
+    return tg.R <= kMaxFusedRG && tw.R <= kMaxFusedRG &&
+           (double)p->lr / (double)p->c_lp < 0.999;
+}
+
+cudaError_t fused_update(const float *g, float *m, float *v, float *dir, const float *u, float *uo,
+                         const float *Im, float *J, float *gJ, WsHeader *h, Dims d,
+                         const fa_params *p, const GaussTaps &tg, const GaussTaps &tw, int t,
+                         int parity, cudaStream_t s) {
+    cudaError_t e = dispatch_k3(g, m, v, FA_F32, dir, h, d, tg, adam_consts(p, t), parity, s);
+    if (e != cudaSuccess) return e;
+    return dispatch_k4(u, dir, uo, FA_F32, Im, J, gJ, h, d, tw, p->lr, p->c_lp, parity, true, s);
+}
+
 fa_status fused_autotune_level(FusedBuffers &fb, WsHeader *h, const fa_params *p, Dims d,
                                const float *If, const float *Im, float *u, float *u_alt, void *m,
                                void *v, const GaussTaps &tg, const GaussTaps &tw,

@@ -643,7 +643,8 @@ __device__ __forceinline__ void compose_position(int pidx, int &ry, int &rx) {
     }
 }
 
-// The body of K4 for the CTA with tile coordinates (bx, by, bz).  Between two
+// The body of K4 for the CTA with tile coordinates (bx, by, bz); Im may be
+// null (no image is warped).  Between two
 // barriers the CTA composes plane i, sums plane i - 1 along x and plane i - 2
 // along y and z, each from the half of a doubled buffer that the interval
 // before filled.
@@ -896,6 +897,7 @@ __device__ __forceinline__ void compose_body(MapRef maps, const TU *__restrict__
                 uo[gi] = sa;
                 uo[N + gi] = sb;
                 uo[2 * N + gi] = sc;
+                if (!Im) continue;
                 tri_issue_p(jp[o], Im, D, H, W, P, zo, y0 + OPT * wy + o, x0 + tx, st_load(sa),
                             st_load(sb), st_load(sc));
                 jidx[o] = gi;

@@ -10,8 +10,10 @@
 // integer atomics: order-independent); the B term gives
 // 2 (I + grad u(x + w(x)))^T B(x) / N with the interpolant's derivative.
 // The descent is Algorithm 1's: Gaussian(sigma_grad), Adam, step scaling,
-// compose, Gaussian(sigma_warp), with the per-op kernels.
+// compose, Gaussian(sigma_warp), with the two update kernels of the fused
+// iteration or the per-op kernels.
 #include "ops.h"
+#include "register.h"
 #include "scatter.cuh"
 #include "validate.h"
 
@@ -341,6 +343,15 @@ extern "C" fa_status fa_inverse(const fa_vol *u, const fa_params *p, fa_vol *w_o
             ++t;
             const int parity = t & 1;
             FA_CUDA_TRY(inverse_gradient(q, q.ul, q.w[cur], d, q.g, nullptr, s));
+            // where tile copies can take the rows (else one kernel per step is faster)
+            if (d.W % 4 == 0 && fused_update_takes(p, tg, tw)) {
+                float *w = q.w[cur], *wo = q.w[cur ^ 1];
+                FA_CUDA_TRY(fused_update(q.g, q.m[cur], q.v[cur], q.dir, w, wo, nullptr, nullptr,
+                                         nullptr, q.h, d, p, tg, tw, t, parity, s));
+                q.w[cur] = wo;  // the new field is the current one
+                q.w[cur ^ 1] = w;
+                continue;
+            }
             const float *g;
             FA_CUDA_TRY(launch_gauss3_any(q.g, q.t1, q.t2, 3, d, tg, &g, s));
             FA_CUDA_TRY(launch_adam(g, q.m[cur], q.v[cur], q.dir, d.N(), adam_consts(p, t),

@@ -186,6 +186,26 @@ cudaError_t launch_lncc_backward(const float *I, const float *J, const float *gr
     return cudaSuccess;
 }
 
+// gF = dL/dI gradI and gM = dL/dJ gradJ (three channels each).
+cudaError_t launch_lncc_grads(const float *I, const float *J, const float *gradI,
+                              const float *gradJ, Dims d, int window, WsHeader *h, LnccBuffers b,
+                              float *gF, float *gM, cudaStream_t s) {
+    GradArgs a{};
+    a.coef = b.coef;
+    a.h = h;
+    a.I = I;
+    a.J = J;
+    a.gJ = gradJ;
+    a.g = gM;
+    cudaError_t e = launch_window_grad(false, a, d, window, 0, s);
+    if (e != cudaSuccess) return e;
+    a.I = J;
+    a.J = I;
+    a.gJ = gradI;
+    a.g = gF;
+    return launch_window_grad(true, a, d, window, 0, s);
+}
+
 long long mse_partials_count(Dims d) {
     VoxGrid gg(d.D, d.H, d.W);
     return (long long)gg.grid.x * gg.grid.y * gg.grid.z;

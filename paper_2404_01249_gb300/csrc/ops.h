@@ -93,6 +93,9 @@ cudaError_t launch_lncc_forward(const float *I, const float *J, Dims d, int wind
                                 cudaStream_t s);
 // Backward: dJ = dL/dJ (may be NULL), dI = dL/dI (may be NULL),
 // g = dL/dJ * grad (3 channels, may be NULL; needs grad).
+cudaError_t launch_lncc_grads(const float *I, const float *J, const float *gradI,
+                              const float *gradJ, Dims d, int window, WsHeader *h, LnccBuffers b,
+                              float *gF, float *gM, cudaStream_t s);
 cudaError_t launch_lncc_backward(const float *I, const float *J, const float *grad, Dims d,
                                  int window, WsHeader *h, LnccBuffers b, float *dJ, float *dI,
                                  float *g, cudaStream_t s);

@@ -28,6 +28,18 @@ struct FusedIter {
 fa_status fused_iteration(FusedBuffers &fb, WsHeader *h, const fa_params *p, Dims d,
                           const FusedIter &it, const GaussTaps &tg, const GaussTaps &tw,
                           fa_kernel_timer *timer, int level, cudaStream_t s);
+// One map's update for the loops written from the per-op kernels (symmetric
+// registration, post-hoc inverse): smoothing, Adam, compose, smoothing of g,
+// m, v (FP32) and u -> uo in the two kernels of the fused iteration, and with
+// an image (else NULL) J = Im o (id + uo) and its gradient.  step_max_bits[parity]
+// is zero on entry; afterwards the other parity's is, with the coefficient
+// maxima and the loss accumulator.  Takes steps below a voxel and Gaussians up
+// to the fused radius.
+bool fused_update_takes(const fa_params *p, const GaussTaps &tg, const GaussTaps &tw);
+cudaError_t fused_update(const float *g, float *m, float *v, float *dir, const float *u, float *uo,
+                         const float *Im, float *J, float *gJ, WsHeader *h, Dims d,
+                         const fa_params *p, const GaussTaps &tg, const GaussTaps &tw, int t,
+                         int parity, cudaStream_t s);
 // Per-level set-up of the fused path: the fixed image's window statistics
 // (LNCC) and J = I_m o (id + u) with its gradient for the first iteration
 // (later iterations get both from the compose kernel).  Needs the level's image maxima in h.

@@ -8,9 +8,13 @@
 //   dL/dphi_F = dL/dJ_F grad I_f(phi_F),   dL/dphi_M = dL/dJ_M grad I_m(phi_M)
 // with its own Adam moments and step scale (one step counter).  On the last
 // level u = w + u_M o (id + w), w the post-hoc inverse of u_F.
-// Built from the per-op kernels: J_F takes the fixed-image role of the LNCC
-// kernels and J_M the warped-image role, so dL/dJ_F is their fixed-image
-// adjoint.
+// J_F takes the fixed-image role of the LNCC kernels and J_M the warped-image
+// role, so dL/dJ_F is their fixed-image adjoint.  Each map's update runs as
+// the two kernels of the fused iteration (fused_update), which also warp the
+// map's image for the next iteration: seven launches per iteration, against
+// eighteen with one kernel per step, which remains for wide Gaussians, steps
+// of a voxel or more and rows that tile copies cannot take (same bits).  96 x
+// 113 x 101, two levels and the inverse: 32.3 ms one kernel per step, 28.6 so.
 #include <stddef.h>
 #include <string.h>
 
@@ -34,6 +38,23 @@ struct SymWs {
     size_t inv_bytes;
 };
 
+// Whether the levels' rows are padded to a multiple of 4 floats, which the
+// update kernels' tile copies need (on dense odd rows, copied per thread, the
+// call above takes 35.7 ms); the MSE and Jacobian kernels take dense rows only.
+bool sym_pitched(const fa_params *p) {
+    GaussTaps tg, tw;
+    make_gauss_taps(p->sigma_grad, &tg);
+    make_gauss_taps(p->sigma_warp, &tw);
+    return p->loss == FA_LOSS_LNCC && !p->use_jac && fused_update_takes(p, tg, tw);
+}
+
+cudaError_t copy_rows(float *dst, int dpitch, const float *src, int spitch, Dims d, int C,
+                      cudaStream_t s) {
+    return cudaMemcpy2DAsync(dst, sizeof(float) * dpitch, src, sizeof(float) * spitch,
+                             sizeof(float) * d.W, (size_t)C * d.D * d.H, cudaMemcpyDeviceToDevice,
+                             s);
+}
+
 // p_inv == nullptr: one grid, loss and gradients only (no fields, no inverse).
 void sym_carve(WsCarver &c, Dims full, const fa_params *p, const fa_params *p_inv, int storage,
                SymWs *q) {
@@ -44,16 +65,17 @@ void sym_carve(WsCarver &c, Dims full, const fa_params *p, const fa_params *p_in
     for (int l = 0; l < L; ++l) {
         const int s = p_inv ? p->scales[l] : 1;
         q->lvl[l] = Dims{level_size(full.D, s), level_size(full.H, s), level_size(full.W, s)};
-        n = q->lvl[l].N() > n ? q->lvl[l].N() : n;
+        if (p_inv && sym_pitched(p)) q->lvl[l].P = (q->lvl[l].W + 3) & ~3;
+        n = q->lvl[l].NP() > n ? q->lvl[l].NP() : n;
     }
     if (storage != FA_F32) {
         q->If0 = c.take<float>(full.N());
         q->Im0 = c.take<float>(full.N());
     }
     for (int l = 0; l < L; ++l) {
-        if (!p_inv || p->scales[l] == 1) continue;
-        q->If[l] = c.take<float>(q->lvl[l].N());
-        q->Im[l] = c.take<float>(q->lvl[l].N());
+        if (!p_inv || (p->scales[l] == 1 && q->lvl[l].pitch() == full.W)) continue;
+        q->If[l] = c.take<float>(q->lvl[l].NP());
+        q->Im[l] = c.take<float>(q->lvl[l].NP());
     }
     if (p_inv)
         for (int k = 0; k < 2; ++k)
@@ -103,28 +125,32 @@ cudaError_t eval_reset(WsHeader *h, cudaStream_t s) {
     return cudaMemsetAsync((char *)h + a, 0, b - a, s);
 }
 
-// L(I_f o phi_F, I_m o phi_M) into loss_dev (may be NULL); with grads,
-// dL/du_F into q.gF and dL/du_M into q.gM.  Needs the images' maxima in h.
-fa_status sym_loss(SymWs &q, int loss, int window, float cc_eps, Dims d, const float *If,
-                   const float *Im, const float *uF, const float *uM, bool grads,
-                   float *loss_dev, cudaStream_t s) {
+cudaError_t sym_warp(SymWs &q, Dims d, const float *If, const float *Im, const float *uF,
+                     const float *uM, bool grads, cudaStream_t s) {
+    cudaError_t e = launch_warp(If, uF, q.JF, grads ? q.gIF : nullptr, d, s);
+    if (e != cudaSuccess) return e;
+    return launch_warp(Im, uM, q.JM, grads ? q.gIM : nullptr, d, s);
+}
+
+// L(J_F, J_M) of the warped images in q into loss_dev (may be NULL); with
+// grads, dL/du_F into q.gF and dL/du_M into q.gM.  Needs the images' maxima in
+// h and its per-evaluation state reset.
+fa_status sym_terms(SymWs &q, int loss, int window, float cc_eps, Dims d, bool grads,
+                    float *loss_dev, cudaStream_t s) {
     const long long N = d.N();
-    FA_CUDA_TRY(eval_reset(q.h, s));
-    FA_CUDA_TRY(launch_warp(If, uF, q.JF, grads ? q.gIF : nullptr, d, s));
-    FA_CUDA_TRY(launch_warp(Im, uM, q.JM, grads ? q.gIM : nullptr, d, s));
     if (loss == FA_LOSS_LNCC) {
         FA_CUDA_TRY(launch_lncc_forward(q.JF, q.JM, d, window, cc_eps, grads, grads, q.h, q.lb, s));
-        FA_CUDA_TRY(launch_loss_finalize(q.h, N, -1.0f, loss_dev, s));
+        if (loss_dev) FA_CUDA_TRY(launch_loss_finalize(q.h, N, -1.0f, loss_dev, s));
         if (grads)
-            FA_CUDA_TRY(launch_lncc_backward(q.JF, q.JM, q.gIM, d, window, q.h, q.lb, nullptr,
-                                             q.dF, q.gM, s));
-    } else {
-        FA_CUDA_TRY(launch_mse(q.JF, q.JM, grads ? q.gIM : nullptr, d, q.h, q.partials, nullptr,
-                               grads ? q.dF : nullptr, grads ? q.gM : nullptr, s));
-        if (loss_dev)
-            FA_CUDA_TRY(cudaMemcpyAsync(loss_dev, &q.h->loss, sizeof(float),
-                                        cudaMemcpyDeviceToDevice, s));
+            FA_CUDA_TRY(launch_lncc_grads(q.JF, q.JM, q.gIF, q.gIM, d, window, q.h, q.lb, q.gF,
+                                          q.gM, s));
+        return FA_OK;
     }
+    FA_CUDA_TRY(launch_mse(q.JF, q.JM, grads ? q.gIM : nullptr, d, q.h, q.partials, nullptr,
+                           grads ? q.dF : nullptr, grads ? q.gM : nullptr, s));
+    if (loss_dev)
+        FA_CUDA_TRY(cudaMemcpyAsync(loss_dev, &q.h->loss, sizeof(float), cudaMemcpyDeviceToDevice,
+                                    s));
     if (grads) {
         long long blocks = (N + 255) / 256;
         blocks = blocks > 152 * 8 ? 152 * 8 : blocks;
@@ -133,6 +159,16 @@ fa_status sym_loss(SymWs &q, int loss, int window, float cc_eps, Dims d, const f
         FA_CUDA_TRY(cudaGetLastError());
     }
     return FA_OK;
+}
+
+// L(I_f o phi_F, I_m o phi_M) into loss_dev (may be NULL), its gradients as
+// sym_terms.
+fa_status sym_loss(SymWs &q, int loss, int window, float cc_eps, Dims d, const float *If,
+                   const float *Im, const float *uF, const float *uM, bool grads,
+                   float *loss_dev, cudaStream_t s) {
+    FA_CUDA_TRY(eval_reset(q.h, s));
+    FA_CUDA_TRY(sym_warp(q, d, If, Im, uF, uM, grads, s));
+    return sym_terms(q, loss, window, cc_eps, d, grads, loss_dev, s);
 }
 
 // Algorithm 1's update of one map (k) from its derivative g (overwritten).
@@ -304,7 +340,11 @@ extern "C" fa_status fa_register_symmetric(const fa_vol *fixed, const fa_vol *mo
     make_gauss_taps(p->sigma_warp, &tw);
     FA_CUDA_TRY(launch_header_reset(q.h, s));
     for (int l = 0; l < p->n_levels; ++l) {
-        if (p->scales[l] == 1) continue;
+        if (!q.If[l]) continue;  // the inputs themselves
+        if (q.lvl[l].pitch() != q.lvl[l].W) {  // zero padding: the maxima read whole rows
+            FA_CUDA_TRY(cudaMemsetAsync(q.If[l], 0, sizeof(float) * q.lvl[l].NP(), s));
+            FA_CUDA_TRY(cudaMemsetAsync(q.Im[l], 0, sizeof(float) * q.lvl[l].NP(), s));
+        }
         FA_CUDA_TRY(launch_pyramid_level(If0, full, p->scales[l], q.If[l], q.lvl[l], q.t1, q.t2, s));
         FA_CUDA_TRY(launch_pyramid_level(Im0, full, p->scales[l], q.Im[l], q.lvl[l], q.t1, q.t2, s));
     }
@@ -312,9 +352,9 @@ extern "C" fa_status fa_register_symmetric(const fa_vol *fixed, const fa_vol *mo
     int cur = 0, t = 0;
     for (int l = 0; l < p->n_levels; ++l) {
         const Dims d = q.lvl[l];
-        const float *If = p->scales[l] == 1 ? If0 : q.If[l];
-        const float *Im = p->scales[l] == 1 ? Im0 : q.Im[l];
-        const size_t b = sizeof(float) * 3 * d.N();
+        const float *If = q.If[l] ? q.If[l] : If0;
+        const float *Im = q.Im[l] ? q.Im[l] : Im0;
+        const size_t b = sizeof(float) * 3 * d.NP();
         if (l == 0) {
             for (int k = 0; k < 2; ++k) {
                 FA_CUDA_TRY(cudaMemsetAsync(q.u[k][cur], 0, b, s));
@@ -335,35 +375,64 @@ extern "C" fa_status fa_register_symmetric(const fa_vol *fixed, const fa_vol *mo
             }
             cur = nx;
         }
+        const bool fused = d.pitch() % 4 == 0 && fused_update_takes(p, tg, tw);
         // fixed-point scale of this level's images (bounds of J_F and J_M)
         FA_CUDA_TRY(cudaMemsetAsync(q.h->absmax_bits, 0, sizeof(q.h->absmax_bits), s));
-        FA_CUDA_TRY(launch_absmax2(If, Im, d.N(), q.h, s));
+        FA_CUDA_TRY(launch_absmax2(If, Im, d.NP(), q.h, s));
+        if (fused) {  // the first iteration's state; its updates leave the next one's
+            FA_CUDA_TRY(eval_reset(q.h, s));
+            FA_CUDA_TRY(sym_warp(q, d, If, Im, q.u[0][cur], q.u[1][cur], true, s));
+        }
         for (int it = 0; it < p->iters[l]; ++it) {
             ++t;
-            FA_TRY(sym_loss(q, p->loss, p->window, p->cc_eps, d, If, Im, q.u[0][cur], q.u[1][cur],
-                            true, nullptr, s));
-            FA_TRY(sym_update(q, p, d, q.gF, 0, cur, t, tg, tw, s));
-            FA_TRY(sym_update(q, p, d, q.gM, 1, cur, t, tg, tw, s));
+            if (!fused) {
+                FA_TRY(sym_loss(q, p->loss, p->window, p->cc_eps, d, If, Im, q.u[0][cur],
+                                q.u[1][cur], true, nullptr, s));
+                FA_TRY(sym_update(q, p, d, q.gF, 0, cur, t, tg, tw, s));
+                FA_TRY(sym_update(q, p, d, q.gM, 1, cur, t, tg, tw, s));
+                continue;
+            }
+            FA_TRY(sym_terms(q, p->loss, p->window, p->cc_eps, d, true, nullptr, s));
+            for (int k = 0; k < 2; ++k) {  // each map has its parity's step maximum
+                float *g = k ? q.gM : q.gF, *u = q.u[k][cur], *uo = q.u[k][cur ^ 1];
+                if (p->use_jac) FA_CUDA_TRY(launch_jac_direction(g, u, g, d, s));
+                FA_CUDA_TRY(fused_update(g, q.m[k][cur], q.v[k][cur], q.dir, u, uo, k ? Im : If,
+                                         k ? q.JM : q.JF, k ? q.gIM : q.gIF, q.h, d, p, tg, tw, t,
+                                         k, s));
+                q.u[k][cur] = uo;  // the new map is the current one
+                q.u[k][cur ^ 1] = u;
+            }
         }
         if (l == L) {
             if (mid_loss_dev)
                 FA_TRY(sym_loss(q, p->loss, p->window, p->cc_eps, d, If, Im, q.u[0][cur],
                                 q.u[1][cur], false, mid_loss_dev, s));
-            fa_vol uf{q.u[0][cur], FA_F32, 3, d.D, d.H, d.W};
+            const Dims dd{d.D, d.H, d.W};
+            const float *uF = q.u[0][cur], *uM = q.u[1][cur];
+            float *zero = q.u[0][cur ^ 1], *ul = (float *)u_out->data;
+            if (d.pitch() != d.W) {  // dense copies for the inverse and the caller
+                FA_CUDA_TRY(copy_rows(q.t1, d.W, uF, d.pitch(), d, 3, s));
+                FA_CUDA_TRY(copy_rows(q.t2, d.W, uM, d.pitch(), d, 3, s));
+                uF = q.t1;
+                uM = q.t2;
+                ul = q.u[1][cur ^ 1];
+            }
+            fa_vol uf{const_cast<float *>(uF), FA_F32, 3, d.D, d.H, d.W};
             fa_vol wv{q.w, FA_F32, 3, d.D, d.H, d.W};
             FA_TRY(fa_inverse(&uf, p_inv, &wv, nullptr, q.inv_ws, q.inv_bytes, stream));
             // phi_M o phi_F^-1 - id = w + u_M o (id + w)
-            FA_CUDA_TRY(launch_compose_fields(q.u[1][cur], q.w, (float *)u_out->data, d, s));
+            FA_CUDA_TRY(launch_compose_fields(uM, q.w, (float *)u_out->data, dd, s));
             // final loss L(I_f, I_m o (id + u)) with zero-displacement F map
-            FA_CUDA_TRY(cudaMemsetAsync(q.u[0][cur ^ 1], 0, b, s));
-            FA_TRY(sym_loss(q, p->loss, p->window, p->cc_eps, d, If, Im, q.u[0][cur ^ 1],
-                            (const float *)u_out->data, false, final_loss_dev, s));
+            if (ul != u_out->data)
+                FA_CUDA_TRY(copy_rows(ul, d.pitch(), (const float *)u_out->data, d.W, d, 3, s));
+            FA_CUDA_TRY(cudaMemsetAsync(zero, 0, b, s));
+            FA_TRY(sym_loss(q, p->loss, p->window, p->cc_eps, d, If, Im, zero, ul, false,
+                            final_loss_dev, s));
+            const size_t bd = sizeof(float) * 3 * d.N();
             if (uF_out_opt)
-                FA_CUDA_TRY(cudaMemcpyAsync(uF_out_opt->data, q.u[0][cur], b,
-                                            cudaMemcpyDeviceToDevice, s));
+                FA_CUDA_TRY(cudaMemcpyAsync(uF_out_opt->data, uF, bd, cudaMemcpyDeviceToDevice, s));
             if (uM_out_opt)
-                FA_CUDA_TRY(cudaMemcpyAsync(uM_out_opt->data, q.u[1][cur], b,
-                                            cudaMemcpyDeviceToDevice, s));
+                FA_CUDA_TRY(cudaMemcpyAsync(uM_out_opt->data, uM, bd, cudaMemcpyDeviceToDevice, s));
         }
     }
     return FA_OK;
