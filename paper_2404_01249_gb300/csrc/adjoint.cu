@@ -9,10 +9,10 @@
 //   dL/dI_m(p) = sum_x dL/dJ(x) w_p(x)            (the adjoint of the warp:
 //                w_p(x) is the trilinear weight of corner p at x + u(x))
 //
-// Without dL/dI_f the call runs on the fused kernels of the registration
-// loop: the warp (J and grad I_m at x + u), the fixed image's window
-// statistics, K1 (exact window sums, cc, the adjoint coefficients, the loss)
-// and K2 (the adjoint window sums, dL/du, and dL/dJ for the scatter).  With
+// Without dL/dI_f the call runs on the window kernels: the warp (J and grad
+// I_m at x + u), the forward sums of both images (cc, the adjoint
+// coefficients, the loss) and K2 (the adjoint window sums, dL/du, and dL/dJ
+// for the scatter).  With
 // dL/dI_f it runs the per-op LNCC kernels, which also form the fixed image's
 // coefficients.  The scatter of dL/dI_m accumulates quantised contributions
 // in int64 with integer atomics, so the result does not depend on the order
