@@ -7,6 +7,8 @@
 #include <string.h>
 
 #include "common.cuh"
+#include "context_table.h"
+#include "launch.cuh"
 #include "validate.h"
 
 namespace fa {
@@ -32,37 +34,92 @@ fa_status cuda_fail(cudaError_t e, const char *where) {
     return FA_ERR_CUDA;
 }
 
+namespace {
+struct CtxEntries {  // the driver's calls about contexts (null: not provided)
+    CUresult (*get_current)(CUcontext *);
+    CUresult (*get_id)(CUcontext, unsigned long long *);
+};
+const CtxEntries &ctx_entries() {
+    static const CtxEntries c = [] {
+        auto entry = [](const char *name) {
+            void *p = nullptr;
+            cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+            if (cudaGetDriverEntryPointByVersion(name, &p, 12000, cudaEnableDefault, &q) !=
+                    cudaSuccess ||
+                q != cudaDriverEntryPointSuccess)
+                p = nullptr;
+            return p;
+        };
+        CtxEntries r;
+        r.get_current = (decltype(r.get_current))entry("cuCtxGetCurrent");
+        r.get_id = (decltype(r.get_id))entry("cuCtxGetId");
+        return r;
+    }();
+    return c;
+}
+}  // namespace
+
 cudaError_t current_context_id(unsigned long long *id) {
-    using GetCurrent = CUresult (*)(CUcontext *);
-    using GetId = CUresult (*)(CUcontext, unsigned long long *);
-    static const GetCurrent get_current = [] {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &p, 12000, cudaEnableDefault,
-                                             &q) != cudaSuccess ||
-            q != cudaDriverEntryPointSuccess)
-            p = nullptr;
-        return (GetCurrent)p;
-    }();
-    static const GetId get_id = [] {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q) !=
-                cudaSuccess ||
-            q != cudaDriverEntryPointSuccess)
-            p = nullptr;
-        return (GetId)p;
-    }();
+    const CtxEntries &c = ctx_entries();
     *id = 0;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if ((e = cudaSetDevice(dev)) != cudaSuccess) return e;  // makes the primary context current
-    if (!get_current || !get_id) return cudaSuccess;
+    if (!c.get_current || !c.get_id) return cudaSuccess;
     CUcontext ctx = nullptr;
     unsigned long long v = 0;
-    if (get_current(&ctx) == CUDA_SUCCESS && ctx && get_id(ctx, &v) == CUDA_SUCCESS) *id = v;
+    if (c.get_current(&ctx) == CUDA_SUCCESS && ctx && c.get_id(ctx, &v) == CUDA_SUCCESS) *id = v;
     return cudaSuccess;
+}
+
+// The device and the context (see current_context_id) that a launch from this
+// thread goes to.  Asked before every launch, so it makes no context current
+// unless the thread has none.
+static cudaError_t launch_context(int *dev, unsigned long long *id) {
+    const CtxEntries &c = ctx_entries();
+    cudaError_t e = cudaGetDevice(dev);
+    if (e != cudaSuccess) return e;
+    CUcontext ctx = nullptr;
+    if (c.get_current && c.get_id && c.get_current(&ctx) == CUDA_SUCCESS && ctx &&
+        c.get_id(ctx, id) == CUDA_SUCCESS)
+        return cudaSuccess;
+    return current_context_id(id);
+}
+
+int prepare_kernel(const void *kernel, size_t smem, int threads) {
+    static ContextTable<int> table;
+    int dev = 0;
+    unsigned long long ctx = 0;
+    if (launch_context(&dev, &ctx) != cudaSuccess) return 1;  // the launch reports it
+    return table.get(dev, ctx, kernel, [&](int *n) {
+        *n = 1;
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+                cudaSuccess ||
+            cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 (int)cudaSharedmemCarveoutMaxShared) != cudaSuccess)
+            return false;
+        int c = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c, kernel, threads, smem) ==
+                cudaSuccess &&
+            c > 1)
+            *n = c;
+        return true;
+    });
+}
+
+int num_sms() {
+    static ContextTable<int> table;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 152;
+    return table.get(dev, 0, nullptr, [&](int *n) {
+        *n = 152;
+        int c = 0;
+        if (cudaDeviceGetAttribute(&c, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || c < 1)
+            return false;
+        *n = c;
+        return true;
+    });
 }
 
 fa_status check_vol(const fa_vol *v, const char *name, int C) {

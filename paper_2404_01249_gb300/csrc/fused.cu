@@ -176,7 +176,7 @@ cudaError_t launch_k3_tma(const Maps &mp, const float *g, TS *m, TS *v, float *d
                           cudaStream_t s) {
     using ST = K3S<RG, NW, OPT, K3_ST, sizeof(TS) == 4>;
     auto kern = k_smooth_adam<RG, NW, OPT, K3_ST, true, TS>;
-    static const int occ = prepare(kern, ST::bytes, ST::NT);
+    const int occ = prepare(kern, ST::bytes, ST::NT);
     LaunchGeom gg = geometry(occ, NW, ST::TY, 2.0f * RG, d, tz);
     return launch_pdl(kern, gg, ST::bytes, s, mp, g, m, v, dir, h, d.D, d.H, d.W, d.pitch(), gg.tz, t, ac,
                       parity);
@@ -203,7 +203,7 @@ cudaError_t launch_k3(const float *g, TS *m, TS *v, float *dir, WsHeader *h, Dim
     } else {
         using SC = K3S<RG, K3_NW, K3_OPT, K3_ST, false>;  // moments unstaged
         auto kern = k_smooth_adam<RG, K3_NW, K3_OPT, K3_ST, false, TS>;
-        static const int occ = prepare(kern, SC::bytes, SC::NT);
+        const int occ = prepare(kern, SC::bytes, SC::NT);
         LaunchGeom gg = geometry(occ, K3_NW, SC::TY, 2.0f * RG, d, tc.tz);
         le = launch_pdl(kern, gg, SC::bytes, s, mp, g, m, v, dir, h, d.D, d.H, d.W, d.pitch(), gg.tz, t, ac,
                         parity);
@@ -218,7 +218,7 @@ cudaError_t launch_k4_tma(const Maps &mp, const TU *u, const float *dir, TU *uo,
                           float lr, float c_lp, int parity, int tz, cudaStream_t s) {
     using ST = K4S<RG, NW, OPT, SU, K4_ST, TU>;
     auto kern = k_compose<RG, NW, OPT, SU, K4_ST, true, TU>;
-    static const int occ = prepare(kern, ST::bytes, ST::NT);
+    const int occ = prepare(kern, ST::bytes, ST::NT);
     LaunchGeom gg = geometry(occ, NW, ST::TY, 2.0f * RG, d, tz);
     return launch_pdl(kern, gg, ST::bytes, s, mp, u, dir, uo, Im, J, gJ, h, d.D, d.H, d.W, d.pitch(), gg.tz, t,
                       lr, c_lp, parity);
@@ -246,7 +246,7 @@ cudaError_t launch_k4(const TU *u, const float *dir, TU *uo, const float *Im, fl
     } else if constexpr (EU == 4) {
         using SC = K4S<RG, K4_NW, K4_OPT, SU, K4_ST>;
         auto kern = k_compose<RG, K4_NW, K4_OPT, SU, K4_ST, false>;
-        static const int occ = prepare(kern, SC::bytes, SC::NT);
+        const int occ = prepare(kern, SC::bytes, SC::NT);
         LaunchGeom gg = geometry(occ, K4_NW, SC::TY, 2.0f * RG, d, tc.tz);
         le = launch_pdl(kern, gg, SC::bytes, s, mp, u, dir, uo, Im, J, gJ, h, d.D, d.H, d.W, d.pitch(), gg.tz, t,
                         lr, c_lp, parity);

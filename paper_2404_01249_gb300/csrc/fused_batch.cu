@@ -270,7 +270,7 @@ template <int R>
 cudaError_t launch_k1_batch(K1Batch &b, const LockstepJob *jobs, cudaStream_t s) {
     constexpr size_t smem = FwdSmem<R, kFwdGiven>::bytes;
     auto kern = k_lncc_fwd_batch<R>;
-    static const int occ = prepare(kern, smem, WinTile<R>::NT);
+    const int occ = prepare(kern, smem, WinTile<R>::NT);
     window_layout<R>(b, jobs, occ);
     return launch_window_batch(kern, b, WinTile<R>::NT, smem, s);
 }
@@ -279,7 +279,7 @@ template <int R>
 cudaError_t launch_k2_batch(K2Batch &b, const LockstepJob *jobs, cudaStream_t s) {
     constexpr size_t smem = GradTile<R>::bytes;
     auto kern = k_lncc_grad_batch<R>;
-    static const int occ = prepare(kern, smem, WinTile<R>::NT);
+    const int occ = prepare(kern, smem, WinTile<R>::NT);
     window_layout<R>(b, jobs, occ);
     return launch_window_batch(kern, b, WinTile<R>::NT, smem, s);
 }
@@ -300,13 +300,13 @@ cudaError_t launch_k3_batch(K3Batch<k3_maps<TS>()> &b, const LockstepJob *jobs, 
     }
     if (tma) {
         auto kern = k_smooth_adam_batch<RG, TS, true>;
-        static const int occ = prepare(kern, ST::bytes, ST::NT);
+        const int occ = prepare(kern, ST::bytes, ST::NT);
         batch_layout(b, jobs, idx, ST::TY, RG, occ);
         return launch_batch(kern, b, ST::NT / FX, ST::bytes, s);
     }
     using SC = K3S<RG, K3W_NW, K3W_OPT, K3_ST, false>;  // moments unstaged
     auto kern = k_smooth_adam_batch<RG, TS, false>;
-    static const int occ = prepare(kern, SC::bytes, SC::NT);
+    const int occ = prepare(kern, SC::bytes, SC::NT);
     batch_layout(b, jobs, idx, SC::TY, RG, occ);
     return launch_batch(kern, b, SC::NT / FX, SC::bytes, s);
 }
@@ -327,14 +327,14 @@ cudaError_t launch_k4_batch(K4Batch<SU ? 2 : 1> &b, const LockstepJob *jobs, con
     }
     if (tma) {
         auto kern = k_compose_batch<RG, SU, true, TU>;
-        static const int occ = prepare(kern, ST::bytes, ST::NT);
+        const int occ = prepare(kern, ST::bytes, ST::NT);
         batch_layout(b, jobs, idx, ST::TY, RG, occ);
         return launch_batch(kern, b, ST::NT / FX, ST::bytes, s);
     }
     if constexpr (EU == 4) {
         using SC = K4S<RG, K4W_NW, K4W_OPT, SU, K4_ST>;
         auto kern = k_compose_batch<RG, SU, false, float>;
-        static const int occ = prepare(kern, SC::bytes, SC::NT);
+        const int occ = prepare(kern, SC::bytes, SC::NT);
         batch_layout(b, jobs, idx, SC::TY, RG, occ);
         return launch_batch(kern, b, SC::NT / FX, SC::bytes, s);
     } else {

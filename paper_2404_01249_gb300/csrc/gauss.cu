@@ -248,7 +248,7 @@ static cudaError_t onepass(const float *in, float *out, int C, Dims d, const Gau
                            cudaStream_t s) {
     using G = GaussTile<R>;
     auto kern = k_gauss_onepass<R>;
-    static const int occ = prepare(kern, G::bytes, G::NT);
+    const int occ = prepare(kern, G::bytes, G::NT);
     const int gx = (d.W + 31) / 32, gy = (d.H + 31) / 32;
     LaunchGeom g;
     g.tz = choose_tz(d.D, gx * gy * C, 2.0f * R + 1.0f, occ);

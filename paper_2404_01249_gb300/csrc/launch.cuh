@@ -2,43 +2,27 @@
 // memory, programmatic dependent launch.
 #pragma once
 
-#include <mutex>
 #include <utility>
 
 #include "ops.h"
 
 namespace fa {
 
+// SMs of the current device.
+int num_sms();
+// Opts a kernel into `smem` bytes of dynamic shared memory in the current
+// context and returns its resident CTAs per SM with blocks of `threads` (1
+// when the driver cannot say).  The limit belongs to the kernel in one
+// context, so it is raised, and the count kept, once per context: on another
+// device, or after a device reset, the next launch raises it there.  A kernel
+// always comes with the same smem and threads.
+int prepare_kernel(const void *kernel, size_t smem, int threads);
+
 namespace {
 
-std::mutex g_mu;
-int g_num_sms = 0;
-
-int num_sms() {
-    std::lock_guard<std::mutex> lock(g_mu);
-    if (g_num_sms == 0) {
-        int dev = 0, n = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0)
-            g_num_sms = n;
-        else
-            g_num_sms = 152;
-    }
-    return g_num_sms;
-}
-
-// Opts the kernel into its dynamic shared memory and returns its resident
-// CTAs per SM (called once per kernel instantiation).
 template <class K>
 int prepare(K kernel, size_t smem, int threads) {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                         (int)cudaSharedmemCarveoutMaxShared);
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, smem) != cudaSuccess ||
-        n < 1)
-        n = 1;
-    return n;
+    return prepare_kernel((const void *)kernel, smem, threads);
 }
 
 struct LaunchGeom {

@@ -369,8 +369,7 @@ cudaError_t launch_mi(const float *I, const float *J, const float *grad, Dims d,
     cudaError_t e = cudaMemsetAsync(b.hist, 0, sizeof(unsigned long long) * nb, s);
     if (e != cudaSuccess) return e;
     const int lc = hist_log_copies(nb);
-    static const int occ = prepare(k_mi_hist, kHistSmem, kHistThreads);
-    (void)occ;
+    prepare(k_mi_hist, kHistSmem, kHistThreads);
     const long long most = (N + kHistThreads - 1) / kHistThreads;
     long long hb = (most + kHistIters - 1) / kHistIters;
     hb = hb < num_sms() ? num_sms() : hb;

@@ -47,8 +47,7 @@
 
 #include <string.h>
 
-#include <mutex>
-
+#include "launch.cuh"
 #include "register.h"
 #include "validate.h"
 
@@ -687,19 +686,10 @@ __global__ void k_grid_barrier_selftest(WsHeader *h, long long limit) {
     grid_barrier(h, k, &flag, limit);
 }
 
-std::mutex g_pmu;
-
 template <class TS, int R>
 int persistent_occupancy(size_t smem) {
     auto kern = k_level_persistent<TS, R>;
-    static const bool attr = [&] {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)playout(PWMAX, PRMAX, PGMAX, PGMAX).bytes);
-        cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             (int)cudaSharedmemCarveoutMaxShared);
-        return true;
-    }();
-    (void)attr;
+    prepare(kern, playout(PWMAX, PRMAX, PGMAX, PGMAX).bytes, PT);
     int occ = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, PT, smem) != cudaSuccess)
         occ = 0;
@@ -709,11 +699,7 @@ int persistent_occupancy(size_t smem) {
 template <class TS, int R>
 fa_status launch_persistent(PersistArgs &a, cudaStream_t s) {
     const PLayout L = playout(a.W, a.R, a.RG, a.RW);
-    int occ;
-    {
-        std::lock_guard<std::mutex> lock(g_pmu);
-        occ = persistent_occupancy<TS, R>(L.bytes);
-    }
+    const int occ = persistent_occupancy<TS, R>(L.bytes);
     if (occ < 1) {
         set_error("persistent level: the kernel does not fit an SM");
         return FA_ERR_UNSUPPORTED;

@@ -21,7 +21,7 @@ template <int R, FwdMode M>
 cudaError_t fwd(FwdArgs &a, Dims d, int tz, cudaStream_t s) {
     using S = FwdSmem<R, M>;
     auto kern = k_lncc_fwd<R, M>;
-    static const int occ = prepare(kern, S::bytes, WinTile<R>::NT);
+    const int occ = prepare(kern, S::bytes, WinTile<R>::NT);
     const LaunchGeom g = window_geom<R>(d, tz, occ);
     a.TZ = g.tz;
     return launch_pdl(kern, g, S::bytes, s, a);
@@ -31,7 +31,7 @@ template <int R, bool SWAP>
 cudaError_t grad(GradArgs &a, Dims d, int tz, cudaStream_t s) {
     using S = GradTile<R>;
     auto kern = k_lncc_grad<R, SWAP>;
-    static const int occ = prepare(kern, S::bytes, WinTile<R>::NT);
+    const int occ = prepare(kern, S::bytes, WinTile<R>::NT);
     const LaunchGeom g = window_geom<R>(d, tz, occ);
     a.TZ = g.tz;
     return launch_pdl(kern, g, S::bytes, s, a);
