@@ -617,8 +617,9 @@ fa_status fa_symmetric_loss_grad(const fa_vol *fixed, const fa_vol *moving, cons
                                  size_t ws_bytes, void *stream);
 
 /* Waits for `stream` and returns the status word that kernels recorded in a
- * workspace used by fa_register, fa_radam_step or fa_lncc_fwd_bwd
- * (FA_OK, FA_ERR_NONFINITE or FA_ERR_TIMEOUT). */
+ * workspace used by fa_register, fa_radam_step, fa_lncc_fwd_bwd, fa_inverse or
+ * fa_register_symmetric (which includes its post-hoc inverse's): FA_OK,
+ * FA_ERR_NONFINITE or FA_ERR_TIMEOUT. */
 fa_status fa_ws_status(const void *ws, void *stream);
 
 /* Failure-detection self-test (no counterpart in the paper): one kernel

@@ -119,6 +119,12 @@ __global__ void __launch_bounds__(256) k_scale_channels(const float *__restrict_
     }
 }
 
+// The nested inverse records what its kernels find (a wait that gave up, a
+// non-finite step) in its own workspace; the caller reads this call's.
+__global__ void k_status_merge(WsHeader *h, const WsHeader *nested) {
+    if (nested->status) status_set(&h->status, nested->status);
+}
+
 // Bytes [offsetof(coef_max_bits), offsetof(loss)) are per-evaluation state.
 cudaError_t eval_reset(WsHeader *h, cudaStream_t s) {
     const size_t a = offsetof(WsHeader, coef_max_bits), b = offsetof(WsHeader, loss);
@@ -420,6 +426,9 @@ extern "C" fa_status fa_register_symmetric(const fa_vol *fixed, const fa_vol *mo
             fa_vol uf{const_cast<float *>(uF), FA_F32, 3, d.D, d.H, d.W};
             fa_vol wv{q.w, FA_F32, 3, d.D, d.H, d.W};
             FA_TRY(fa_inverse(&uf, p_inv, &wv, nullptr, q.inv_ws, q.inv_bytes, stream));
+            k_status_merge<<<1, 1, 0, s>>>(q.h, (const WsHeader *)q.inv_ws);
+            note_launch();
+            FA_CUDA_TRY(cudaGetLastError());
             // phi_M o phi_F^-1 - id = w + u_M o (id + w)
             FA_CUDA_TRY(launch_compose_fields(uM, q.w, (float *)u_out->data, dd, s));
             // final loss L(I_f, I_m o (id + u)) with zero-displacement F map

@@ -598,16 +598,26 @@ def fa_affine_field(theta: torch.Tensor, shape, out: Optional[torch.Tensor] = No
     return out
 
 
-def fa_inverse(u: torch.Tensor, params: RegParams, sync: bool = True):
+def _check_waits(ws: torch.Tensor):
+    """Raises FAError(FA_ERR_TIMEOUT) when a bounded device wait of the finished
+    call that used ws gave up (bit 1 of its status word)."""
+    if int(ws[:4].view(torch.int32)) & 2:
+        raise FAError(FA_ERR_TIMEOUT, "a bounded device wait gave up")
+
+
+def fa_inverse(u: torch.Tensor, params: RegParams, sync: bool = True,
+               ws: Optional[torch.Tensor] = None):
     """Post-hoc inverse w of the displacement u (see fa.h).  Returns
-    dict(w=[3, d, h, w] of the last level, energy, final_energy)."""
+    dict(w=[3, d, h, w] of the last level, energy, final_energy).  With
+    sync=False pass ws (fa_inverse_workspace_size bytes) to read the call's
+    status later (fa_ws_status)."""
     D, H, W = u.shape[-3:]
     p = params.to_c()
     lib = load()
     need = lib.fa_inverse_workspace_size(D, H, W, ctypes.byref(p))
     if need == 0:
         raise FAError(FA_ERR_INVALID, lib.fa_last_error().decode())
-    ws = workspace(need, u.device)
+    ws = ws if ws is not None else workspace(need, u.device)
     s = params.scales[-1]
     w = torch.empty((3, level_size(D, s), level_size(H, s), level_size(W, s)), device=u.device)
     energy = torch.empty((), device=u.device)
@@ -616,6 +626,7 @@ def fa_inverse(u: torch.Tensor, params: RegParams, sync: bool = True):
     out = dict(w=w, energy=energy)
     if sync:
         torch.cuda.current_stream().synchronize()
+        _check_waits(ws)
         out["final_energy"] = float(energy)
     return out
 
@@ -634,9 +645,11 @@ def fa_inverse_energy_grad(u: torch.Tensor, w: torch.Tensor):
 
 
 def fa_register_symmetric(fixed, moving, params: RegParams, inv_params: RegParams,
-                          sync: bool = True):
+                          sync: bool = True, ws: Optional[torch.Tensor] = None):
     """Symmetric registration (see fa.h).  Returns dict(u, uF, uM on the last
-    level's grid, loss, mid_loss, final_loss, final_mid_loss)."""
+    level's grid, loss, mid_loss, final_loss, final_mid_loss).  With sync=False
+    pass ws (fa_register_symmetric_workspace_size bytes) to read the call's
+    status later (fa_ws_status)."""
     D, H, W = fixed.shape[-3:]
     p, pi = params.to_c(), inv_params.to_c()
     p.storage = _DTYPES.get(fixed.dtype, FA_F32)  # 16-bit images are widened in the workspace
@@ -644,7 +657,7 @@ def fa_register_symmetric(fixed, moving, params: RegParams, inv_params: RegParam
     need = lib.fa_register_symmetric_workspace_size(D, H, W, ctypes.byref(p), ctypes.byref(pi))
     if need == 0:
         raise FAError(FA_ERR_INVALID, lib.fa_last_error().decode())
-    ws = workspace(need, fixed.device)
+    ws = ws if ws is not None else workspace(need, fixed.device)
     s = params.scales[-1]
     shape = (3, level_size(D, s), level_size(H, s), level_size(W, s))
     u, uF, uM = (torch.empty(shape, device=fixed.device) for _ in range(3))
@@ -656,6 +669,7 @@ def fa_register_symmetric(fixed, moving, params: RegParams, inv_params: RegParam
     out = dict(u=u, uF=uF, uM=uM, loss=loss, mid_loss=mid)
     if sync:
         torch.cuda.current_stream().synchronize()
+        _check_waits(ws)
         out["final_loss"], out["final_mid_loss"] = float(loss), float(mid)
     return out
 
