@@ -150,10 +150,6 @@ cudaError_t launch_lncc_forward(const float *I, const float *J, Dims d, int wind
     return launch_window_fwd(kFwdBoth, a, d, window, 0, s);
 }
 
-static bool overlap(const float *a, const float *b, long long n) {
-    return a && b && a < b + n && b < a + n;
-}
-
 cudaError_t launch_lncc_backward(const float *I, const float *J, const float *grad, Dims d,
                                  int window, WsHeader *h, LnccBuffers b, float *dJ, float *dI,
                                  float *g, cudaStream_t s) {
@@ -161,15 +157,19 @@ cudaError_t launch_lncc_backward(const float *I, const float *J, const float *gr
     GradArgs a{};
     a.coef = b.coef;
     a.h = h;
-    // dL/dI reads the images after dL/dJ is written: a dL/dJ that overlaps
-    // one of them waits in the scratch
-    float *dJ1 = dI && (overlap(dJ, I, N) || overlap(dJ, J, N)) ? (float *)b.p0 : dJ;
+    // dL/dI reads the images after dL/dJ and g are written: one that overlaps
+    // an image waits in the scratch
+    auto waits = [&](const float *out, long long n) {
+        auto over = [&](const float *in) { return out < in + N && in < out + n; };
+        return dI && out && (over(I) || over(J));
+    };
+    float *dJ1 = waits(dJ, N) ? (float *)b.p0 : dJ, *g1 = waits(g, 3 * N) ? (float *)b.p0 + N : g;
     cudaError_t e;
     if (dJ || g) {
         a.I = I;
         a.J = J;
         a.gJ = grad;
-        a.g = g;
+        a.g = g1;
         a.dJ = dJ1;
         if ((e = launch_window_grad(false, a, d, window, 0, s)) != cudaSuccess) return e;
     }
@@ -181,8 +181,11 @@ cudaError_t launch_lncc_backward(const float *I, const float *J, const float *gr
         a.dJ = dI;
         if ((e = launch_window_grad(true, a, d, window, 0, s)) != cudaSuccess) return e;
     }
-    if (dJ1 != dJ)
-        return cudaMemcpyAsync(dJ, dJ1, sizeof(float) * N, cudaMemcpyDeviceToDevice, s);
+    const size_t bytes = sizeof(float) * N;
+    if (dJ1 != dJ &&
+        (e = cudaMemcpyAsync(dJ, dJ1, bytes, cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
+        return e;
+    if (g1 != g) return cudaMemcpyAsync(g, g1, 3 * bytes, cudaMemcpyDeviceToDevice, s);
     return cudaSuccess;
 }
 

@@ -1,0 +1,47 @@
+"""Outputs that share memory with inputs: a result laid over an image or a
+field that the call still reads is the same as one kept apart."""
+import ctypes
+
+import pytest
+import torch
+
+from paper_2404_01249_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def fa():
+    from paper_2404_01249_gb300 import build, fa
+    build.build()
+    assert torch.cuda.is_available()
+    fa.load()
+    return fa
+
+
+@pytest.mark.parametrize("shape", [(12, 16, 40), (9, 17, 33)])
+@pytest.mark.parametrize("channel", [0, 1, 2])
+def test_adjoint_field_gradient_over_the_fixed_image(fa, shape, channel):
+    f, m, _ = synth.voronoi_pair(shape=shape, seed=321)
+    f, m = torch.from_numpy(f).cuda(), torch.from_numpy(m).cuda()
+    u = torch.from_numpy(synth.random_field(shape, 3.0, 2.5, seed=9)).float().cuda()
+    ref = fa.fa_warp_lncc_adjoint(f, m, u, 5)
+    lib = fa.load()
+    ws = fa.workspace(lib.fa_warp_lncc_adjoint_workspace_size(*shape))
+    # the image's 16-byte aligned place inside the gradient's buffer
+    n = f.numel()
+    du = torch.empty((3,) + shape, device="cuda")
+    fixed = du.view(-1)[channel * n:(channel + 1) * n].view(shape)
+    assert fixed.data_ptr() % 16 == 0 or channel  # odd grids: channel 0 only
+    if fixed.data_ptr() % 16:
+        pytest.skip("an image must start on 16 bytes")
+    fixed.copy_(f)
+    dI, dM, loss = torch.empty_like(f), torch.empty_like(f), torch.empty((), device="cuda")
+    fa._check(lib.fa_warp_lncc_adjoint(fa._vol(fixed, 1), fa._vol(m, 1), fa._vol(u, 3), 5,
+                                       ctypes.c_float(1e-5), fa._ptr(loss), fa._vol(du, 3),
+                                       fa._vol(dI, 1), fa._vol(dM, 1), fa._ptr(ws), ws.numel(),
+                                       fa._stream()))
+    assert float(loss) == float(ref["loss"])
+    assert torch.equal(du, ref["dL_du"])
+    assert torch.equal(dI, ref["dL_dfixed"])
+    assert torch.equal(dM, ref["dL_dmoving"])
