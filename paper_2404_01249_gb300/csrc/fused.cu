@@ -390,7 +390,8 @@ fa_status fused_iteration(FusedBuffers &fb, WsHeader *h, const fa_params *p, Dim
     } else {
         VoxGrid gg(d.D, d.H, d.W);
         FA_CUDA_TRY(start(FA_K_FUSED_LNCC_GRAD));
-        k_fused_mse_grad<<<gg.grid, gg.block, 0, s>>>(it.If, fb.J, fb.gJ, fb.g, d.D, d.H, d.W);
+        k_fused_mse_grad<<<gg.grid, gg.block, 0, s>>>(it.If, fb.J, fb.gJ, fb.g, d.D, d.H, d.W,
+                                                    d.pitch());
         note_launch();
         FA_CUDA_TRY(cudaGetLastError());
         FA_CUDA_TRY(stop(FA_K_FUSED_LNCC_GRAD));

@@ -369,14 +369,14 @@ __global__ void __launch_bounds__(256) k_fused_mse_grad(const float *__restrict_
                                                         const float *__restrict__ J,
                                                         const float *__restrict__ gJ,
                                                         float *__restrict__ g, int D, int H,
-                                                        int W) {
+                                                        int W, int P) {
     int x = blockIdx.x * 32 + threadIdx.x;
     int y = blockIdx.y * 8 + threadIdx.y;
     int z = blockIdx.z;
     if (x >= W || y >= H) return;
-    long long N = (long long)D * H * W;
-    long long i = ((long long)z * H + y) * W + x;
-    float dj = 2.0f * (__ldg(J + i) - __ldg(If + i)) / (float)N;
+    const long long N = (long long)D * H * P;  // rows of P elements
+    const long long i = ((long long)z * H + y) * P + x;
+    float dj = 2.0f * (__ldg(J + i) - __ldg(If + i)) / (float)((long long)D * H * W);
     g[i] = dj * __ldg(gJ + i);
     g[N + i] = dj * __ldg(gJ + N + i);
     g[2 * N + i] = dj * __ldg(gJ + 2 * N + i);

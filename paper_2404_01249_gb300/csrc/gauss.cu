@@ -37,16 +37,16 @@ bool make_gauss_taps(float sigma, GaussTaps *t) {
 template <int AXIS>
 __global__ void __launch_bounds__(256) k_gauss_axis(const float *__restrict__ in,
                                                     float *__restrict__ out, int C, int D, int H,
-                                                    int W, GaussTaps t) {
+                                                    int W, int P, GaussTaps t) {
     int x = blockIdx.x * 32 + threadIdx.x;
     int y = blockIdx.y * 8 + threadIdx.y;
     int z = blockIdx.z;
     if (x >= W || y >= H) return;
-    long long N = (long long)D * H * W;
-    long long i = ((long long)z * H + y) * W + x;
+    long long N = (long long)D * H * P;  // rows of P elements
+    long long i = ((long long)z * H + y) * P + x;
     const int c0 = AXIS == 0 ? x : (AXIS == 1 ? y : z);
     const int n = AXIS == 0 ? W : (AXIS == 1 ? H : D);
-    const long long stride = AXIS == 0 ? 1ll : (AXIS == 1 ? (long long)W : (long long)H * W);
+    const long long stride = AXIS == 0 ? 1ll : (AXIS == 1 ? (long long)P : (long long)H * P);
     const int R = t.R;
     int lo = max(-R, -c0), hi = min(R, n - 1 - c0);
     for (int c = 0; c < C; ++c) {
@@ -60,15 +60,13 @@ __global__ void __launch_bounds__(256) k_gauss_axis(const float *__restrict__ in
 cudaError_t launch_gauss_axis(const float *in, float *out, int C, Dims d, const GaussTaps &t,
                               int axis, cudaStream_t s) {
     VoxGrid g(d.D, d.H, d.W);
-    if (axis == 0) {
-        k_gauss_axis<0><<<g.grid, g.block, 0, s>>>(in, out, C, d.D, d.H, d.W, t); note_launch();
-    }
-    else if (axis == 1) {
-        k_gauss_axis<1><<<g.grid, g.block, 0, s>>>(in, out, C, d.D, d.H, d.W, t); note_launch();
-    }
-    else {
-        k_gauss_axis<2><<<g.grid, g.block, 0, s>>>(in, out, C, d.D, d.H, d.W, t); note_launch();
-    }
+    if (axis == 0)
+        k_gauss_axis<0><<<g.grid, g.block, 0, s>>>(in, out, C, d.D, d.H, d.W, d.pitch(), t);
+    else if (axis == 1)
+        k_gauss_axis<1><<<g.grid, g.block, 0, s>>>(in, out, C, d.D, d.H, d.W, d.pitch(), t);
+    else
+        k_gauss_axis<2><<<g.grid, g.block, 0, s>>>(in, out, C, d.D, d.H, d.W, d.pitch(), t);
+    note_launch();
     return cudaGetLastError();
 }
 
@@ -262,16 +260,16 @@ static cudaError_t onepass(const float *in, float *out, int C, Dims d, const Gau
     return cudaGetLastError();
 }
 
-// The one-pass kernel takes grids its launch limits allow (65,535 layers of
-// tiles along y and of slabs); anything else goes axis by axis.
+// The one-pass kernel takes unpadded grids that its launch limits allow (65,535
+// layers of tiles along y and of slabs); anything else goes axis by axis.
 static bool onepass_takes(int C, Dims d, const GaussTaps &t) {
-    return t.R >= 1 && t.R <= kOnePassRadius && (d.H + 31) / 32 <= 65535 &&
+    return t.R >= 1 && t.R <= kOnePassRadius && d.pitch() == d.W && (d.H + 31) / 32 <= 65535 &&
            (long long)C * d.D <= 65535;
 }
 
 cudaError_t launch_gauss3(const float *in, float *out, float *t1, float *t2, int C, Dims d,
                           const GaussTaps &t, cudaStream_t s) {
-    const long long n = C * d.N();
+    const long long n = C * d.NP();
     if (t.R == 0) {
         if (in == out) return cudaSuccess;
         return cudaMemcpyAsync(out, in, sizeof(float) * n, cudaMemcpyDeviceToDevice, s);

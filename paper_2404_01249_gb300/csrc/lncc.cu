@@ -55,18 +55,19 @@ __global__ void k_loss_finalize(WsHeader *h, long long N, float sign, float *out
 __global__ void __launch_bounds__(256) k_mse(const float *__restrict__ I,
                                              const float *__restrict__ J,
                                              const float *__restrict__ grad, float *dJ, float *dI,
-                                             float *g, float *partials, int D, int H, int W) {
+                                             float *g, float *partials, int D, int H, int W,
+                                             int P) {
     __shared__ float red[8];
     int x = blockIdx.x * 32 + threadIdx.x;
     int y = blockIdx.y * 8 + threadIdx.y;
     int z = blockIdx.z;
-    long long N = (long long)D * H * W;
+    const long long N = (long long)D * H * P;  // rows of P elements
     float e2 = 0.0f;
     if (x < W && y < H) {
-        long long i = ((long long)z * H + y) * W + x;
+        const long long i = ((long long)z * H + y) * P + x;
         float e = J[i] - I[i];
         e2 = e * e;
-        float dj = 2.0f * e / (float)N;
+        float dj = 2.0f * e / (float)((long long)D * H * W);
         if (dJ) dJ[i] = dj;
         if (dI) dI[i] = -dj;
         if (g) {
@@ -218,7 +219,9 @@ cudaError_t launch_mse(const float *I, const float *J, const float *grad, Dims d
                        float *partials, float *dJ, float *dI, float *g, cudaStream_t s) {
     VoxGrid gg(d.D, d.H, d.W);
     long long nb = mse_partials_count(d);
-    k_mse<<<gg.grid, gg.block, 0, s>>>(I, J, grad, dJ, dI, g, partials, d.D, d.H, d.W); note_launch();
+    k_mse<<<gg.grid, gg.block, 0, s>>>(I, J, grad, dJ, dI, g, partials, d.D, d.H, d.W,
+                                         d.pitch());
+    note_launch();
     k_partials_finalize<<<1, 256, 0, s>>>(partials, nb, d.N(), h, nullptr); note_launch();
     return cudaGetLastError();
 }

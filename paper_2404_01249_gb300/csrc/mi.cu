@@ -80,6 +80,14 @@ __device__ __forceinline__ void load4(float (&v)[4], const float *__restrict__ p
     }
 }
 
+// Which of the values i .. i + 3 (i a multiple of 4) of a volume of N elements
+// are voxels: the first so many.  Rows hold W voxels and P elements, P == W or
+// a multiple of 4 (volumes with such rows hold fewer than 2^32 elements).
+__device__ __forceinline__ int voxels4(long long i, long long N, int W, int P) {
+    if (P == W) return i + 4 <= N ? 4 : (int)(N - i);
+    return min(4, max(0, W - (int)((unsigned)i % (unsigned)P)));
+}
+
 __global__ void k_mi_range_init(unsigned *keys) {
     keys[0] = 0xffffffffu;   // lo_f: min over the fixed image
     keys[1] = 0u;            // hi_f
@@ -93,16 +101,17 @@ __global__ void k_mi_range_set(const float *range, unsigned *keys) {
 
 __global__ void __launch_bounds__(256) k_mi_range(const float *__restrict__ If,
                                                   const float *__restrict__ Im, long long N,
-                                                  unsigned *keys) {
+                                                  int W, int P, unsigned *keys) {
     unsigned k[4] = {0xffffffffu, 0u, 0xffffffffu, 0u};
     for (long long i = 4 * ((long long)blockIdx.x * blockDim.x + threadIdx.x); i < N;
          i += 4ll * gridDim.x * blockDim.x) {
         float a[4], b[4];
         load4(a, If, i, N);
         load4(b, Im, i, N);
+        const int n = voxels4(i, N, W, P);
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            if (i + e >= N) break;
+            if (e >= n) break;
             if (fabsf(a[e]) <= 3.4e38f) {
                 k[0] = min(k[0], fkey(a[e]));
                 k[1] = max(k[1], fkey(a[e]));
@@ -160,7 +169,7 @@ int hist_log_copies(int nb) {
 
 __global__ void __launch_bounds__(kHistThreads) k_mi_hist(const float *__restrict__ I,
                                                           const float *__restrict__ J, long long N,
-                                                          int B, int lc,
+                                                          int W, int P, int B, int lc,
                                                           const unsigned *__restrict__ keys,
                                                           unsigned long long *ghist, WsHeader *h) {
     extern __shared__ unsigned shu[];  // [2][B*B][2^lc]: low and high halves
@@ -172,6 +181,7 @@ __global__ void __launch_bounds__(kHistThreads) k_mi_hist(const float *__restric
     bool bad = false;
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += stride) {
+        if (P != W && (int)((unsigned)i % (unsigned)P) >= W) continue;  // a row's padding
         const float a = I[i], b = J[i];
         if (!(fabsf(a) <= 3.4e38f && fabsf(b) <= 3.4e38f)) {
             bad = true;
@@ -267,14 +277,14 @@ __global__ void __launch_bounds__(1024) k_mi_table(const unsigned long long *__r
 __global__ void __launch_bounds__(256) k_mi_grad(const float *__restrict__ I,
                                                  const float *__restrict__ J,
                                                  const float *__restrict__ grad, long long N,
-                                                 int B, const unsigned *__restrict__ keys,
+                                                 float count, int B, const unsigned *__restrict__ keys,
                                                  const float *__restrict__ Tg, float *dJ,
                                                  float *g) {
     extern __shared__ float T[];
     for (int k = threadIdx.x; k < B * B; k += blockDim.x) T[k] = Tg[k];
     __syncthreads();
     const MiMap mf = mi_map(keys, 0, B), mm = mi_map(keys, 1, B);
-    const float c = -mm.s / (float)N;
+    const float c = -mm.s / count;
     // four adjacent voxels per thread and step: their loads and table reads
     // overlap (one voxel: 48 us on 6.9 M voxels; four: 40 us, bound by the table's shared-memory reads)
     for (long long i = 4 * ((long long)blockIdx.x * blockDim.x + threadIdx.x); i < N;
@@ -346,11 +356,12 @@ MiBuffers mi_carve(WsCarver &c, int bins) {
     return b;
 }
 
-cudaError_t launch_mi_range(const float *If, const float *Im, long long N, MiBuffers b,
+cudaError_t launch_mi_range(const float *If, const float *Im, Dims d, MiBuffers b,
                             cudaStream_t s) {
+    const long long N = d.NP();
     k_mi_range_init<<<1, 1, 0, s>>>(b.range);
     note_launch();
-    k_mi_range<<<grid_blocks(N), 256, 0, s>>>(If, Im, N, b.range);
+    k_mi_range<<<grid_blocks(N), 256, 0, s>>>(If, Im, N, d.W, d.pitch(), b.range);
     note_launch();
     return cudaGetLastError();
 }
@@ -364,7 +375,7 @@ cudaError_t launch_mi_range_set(const float *range4, MiBuffers b, cudaStream_t s
 cudaError_t launch_mi(const float *I, const float *J, const float *grad, Dims d, int bins,
                       WsHeader *h, MiBuffers b, float *loss_out, float *dJ, float *g,
                       cudaStream_t s) {
-    const long long N = d.N();
+    const long long N = d.NP();  // elements; the gradient fills a row's padding too
     const int nb = bins * bins;
     cudaError_t e = cudaMemsetAsync(b.hist, 0, sizeof(unsigned long long) * nb, s);
     if (e != cudaSuccess) return e;
@@ -374,17 +385,17 @@ cudaError_t launch_mi(const float *I, const float *J, const float *grad, Dims d,
     long long hb = (most + kHistIters - 1) / kHistIters;
     hb = hb < num_sms() ? num_sms() : hb;
     hb = hb < most ? hb : most;
-    k_mi_hist<<<(unsigned)hb, kHistThreads, ((size_t)nb << lc) * 8, s>>>(I, J, N, bins, lc,
-                                                                         b.range, b.hist, h);
+    k_mi_hist<<<(unsigned)hb, kHistThreads, ((size_t)nb << lc) * 8, s>>>(
+        I, J, N, d.W, d.pitch(), bins, lc, b.range, b.hist, h);
     note_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const size_t tab_smem = sizeof(float) * (nb + 2 * bins + 2 * 1024);
-    k_mi_table<<<1, 1024, tab_smem, s>>>(b.hist, bins, N, b.T, h, loss_out);
+    k_mi_table<<<1, 1024, tab_smem, s>>>(b.hist, bins, d.N(), b.T, h, loss_out);
     note_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (dJ || g) {
-        k_mi_grad<<<grid_blocks(N), 256, sizeof(float) * nb, s>>>(I, J, grad, N, bins, b.range,
-                                                                   b.T, dJ, g);
+        k_mi_grad<<<grid_blocks(N), 256, sizeof(float) * nb, s>>>(
+            I, J, grad, N, (float)d.N(), bins, b.range, b.T, dJ, g);
         note_launch();
     }
     return cudaGetLastError();
@@ -430,7 +441,7 @@ extern "C" fa_status fa_mi_fwd_bwd(const fa_vol *fixed, const fa_vol *warped, in
     if (range_dev_opt)
         FA_CUDA_TRY(launch_mi_range_set(range_dev_opt, b, s));
     else
-        FA_CUDA_TRY(launch_mi_range(I, J, d.N(), b, s));
+        FA_CUDA_TRY(launch_mi_range(I, J, d, b, s));
     FA_CUDA_TRY(launch_mi(I, J, nullptr, d, bins, h, b, loss_dev,
                           dL_dwarped_opt ? (float *)dL_dwarped_opt->data : nullptr, nullptr, s));
     return FA_OK;

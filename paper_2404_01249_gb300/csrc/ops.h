@@ -125,7 +125,7 @@ struct MiBuffers {
 constexpr int kMiMinBins = 6, kMiMaxBins = 64;
 MiBuffers mi_carve(WsCarver &c, int bins);
 // [lo, hi] of I_f, and of I_m with 0 included (samples outside the grid are 0)
-cudaError_t launch_mi_range(const float *If, const float *Im, long long N, MiBuffers b,
+cudaError_t launch_mi_range(const float *If, const float *Im, Dims d, MiBuffers b,
                             cudaStream_t s);
 cudaError_t launch_mi_range_set(const float *range4, MiBuffers b, cudaStream_t s);
 // L = -MI(I, J) into h->loss (and loss_out if not NULL); dJ = dL/dJ and

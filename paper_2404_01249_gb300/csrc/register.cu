@@ -93,21 +93,20 @@ static fa_status check_params(const fa_params *p) {
 }
 
 // Row pitch of a level's buffers: the width rounded up to a multiple of 4
-// (8 with an FP16 u) where the four fused LNCC kernels run every step of the
-// level, so that they take TMA tiles at any width; 0 (the width itself)
-// elsewhere.  The padding is never read as data: TMA tiles describe the
-// D x H x W grid and fill beyond it with zeros, and every other access
+// (8 with an FP16 u) where the fused iteration runs the level, so that its
+// update kernels take TMA tiles at any width; 0 (the width itself) for the
+// plain and the persistent schedule.  On dense odd rows the update kernels copy
+// per thread, which the short march of a small grid does not hide: ten
+// iterations of MSE take 222 us dense and 178 padded on 31 x 37 x 27, 537 and
+// 414 on 63 x 65 x 67; of MI 713 and 581 there.  (The padded copies of a
+// scale-1 level's images take 6 us of a call.)
+// The padding is never read as data: TMA tiles describe the D x H x W grid and
+// fill beyond it with zeros, the MI kernels skip it, and every other access
 // checks x < W.
 static int level_pitch(const fa_params *p, Dims d) {
     // FP16 u: rows of a multiple of 8 elements (16 bytes of FP16)
     if (p->field_storage == FA_F16) return d.W % 8 == 0 ? 0 : (d.W + 7) & ~7;
-    if (p->loss != FA_LOSS_LNCC || p->use_jac || d.W % 4 == 0) return 0;
-    if (p->mode == FA_MODE_PLAIN || (p->mode == FA_MODE_PERSISTENT && persistent_eligible(p, d)))
-        return 0;
-    GaussTaps tg, tw;
-    make_gauss_taps(p->sigma_grad, &tg);
-    make_gauss_taps(p->sigma_warp, &tw);
-    if (tg.R > kMaxFusedRadius || tw.R > kMaxFusedRadius) return 0;  // separable passes, unpitched
+    if (d.W % 4 == 0 || p->mode == FA_MODE_PLAIN || persistent_eligible(p, d)) return 0;
     return (d.W + 3) & ~3;
 }
 
@@ -377,7 +376,7 @@ static fa_status level_begin(Plan &P, const fa_params *p, int l, const float *u_
     // fixed-point scale of this level's images (max |I_f|, max |I_m|)
     FA_CUDA_TRY(cudaMemsetAsync(P.h->absmax_bits, 0, sizeof(P.h->absmax_bits), s));
     FA_CUDA_TRY(launch_absmax2(If, Im, d.NP(), P.h, s));  // padding (if any) holds zeros
-    if (p->loss == FA_LOSS_MI) FA_CUDA_TRY(launch_mi_range(If, Im, d.N(), P.mi, s));
+    if (p->loss == FA_LOSS_MI) FA_CUDA_TRY(launch_mi_range(If, Im, d, P.mi, s));
     if (p->mode != FA_MODE_PLAIN)
         FA_CUDA_TRY(fused_level_start(If, Im, P.u[*cur], d, p, P.h, P.fb, s));
     return FA_OK;

@@ -325,7 +325,7 @@ extern "C" fa_status fa_register_svf(const fa_vol *fixed, const fa_vol *moving,
         }
         FA_CUDA_TRY(cudaMemsetAsync(q.h->absmax_bits, 0, sizeof(q.h->absmax_bits), s));
         FA_CUDA_TRY(launch_absmax2(If, Im, d.N(), q.h, s));
-        if (p->loss == FA_LOSS_MI) FA_CUDA_TRY(launch_mi_range(If, Im, d.N(), q.mi, s));
+        if (p->loss == FA_LOSS_MI) FA_CUDA_TRY(launch_mi_range(If, Im, d, q.mi, s));
         for (int it = 0; it < p->iters[l]; ++it) {
             ++t;
             const int parity = t & 1;
@@ -383,7 +383,7 @@ extern "C" fa_status fa_svf_loss_grad(const fa_vol *fixed, const fa_vol *moving,
     const float *If = (const float *)fixed->data, *Im = (const float *)moving->data;
     FA_CUDA_TRY(launch_header_reset(q.h, s));
     FA_CUDA_TRY(launch_absmax2(If, Im, d.N(), q.h, s));
-    if (p1.loss == FA_LOSS_MI) FA_CUDA_TRY(launch_mi_range(If, Im, d.N(), q.mi, s));
+    if (p1.loss == FA_LOSS_MI) FA_CUDA_TRY(launch_mi_range(If, Im, d, q.mi, s));
     // exp(v) - id is made in the caller's field unless that holds an image the
     // loss still reads, or the gradient that is written after it
     const size_t b = sizeof(float) * 3 * d.N();

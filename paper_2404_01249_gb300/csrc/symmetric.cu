@@ -40,7 +40,8 @@ struct SymWs {
 
 // Whether the levels' rows are padded to a multiple of 4 floats, which the
 // update kernels' tile copies need (on dense odd rows, copied per thread, the
-// call above takes 35.7 ms); the MSE and Jacobian kernels take dense rows only.
+// call above takes 35.7 ms).  MSE (k_scale_channels) and the Jacobian direction
+// keep dense rows.
 bool sym_pitched(const fa_params *p) {
     GaussTaps tg, tw;
     make_gauss_taps(p->sigma_grad, &tg);

@@ -58,7 +58,7 @@ cudaError_t launch_warp_field(const float *Im, const void *u, int field, float *
 // diffeomorphisms", the use_jac option of Algorithm 1): g <- J(phi)^T g with
 // J(phi) = I + grad u, grad u by central differences inside the grid and
 // one-sided first differences at its ends (zero on an axis of length 1).
-// In place: each output reads only its own voxel of g.
+// In place: each output reads only its own voxel of g.  Rows of P elements.
 __device__ __forceinline__ float fd_axis(const float *__restrict__ f, int n, int k, long long i,
                                          long long stride) {
     if (n < 2) return 0.0f;
@@ -68,19 +68,19 @@ __device__ __forceinline__ float fd_axis(const float *__restrict__ f, int n, int
 }
 
 __global__ void __launch_bounds__(256) k_jac_direction(const float *gin, const float *__restrict__ u,
-                                                       float *gout, int D, int H, int W) {
+                                                       float *gout, int D, int H, int W, int P) {
     const int x = blockIdx.x * 32 + threadIdx.x;
     const int y = blockIdx.y * 8 + threadIdx.y;
     const int z = blockIdx.z;
     if (x >= W || y >= H) return;
-    const long long N = (long long)D * H * W, HW = (long long)H * W;
-    const long long i = (long long)z * HW + (long long)y * W + x;
+    const long long N = (long long)D * H * P, HW = (long long)H * P;
+    const long long i = (long long)z * HW + (long long)y * P + x;
     const float g0 = gin[i], g1 = gin[N + i], g2 = gin[2 * N + i];
     float out[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {  // component a: g_a + sum_j (d u_j / d x_a) g_j
         const int n = a == 0 ? D : (a == 1 ? H : W), k = a == 0 ? z : (a == 1 ? y : x);
-        const long long st = a == 0 ? HW : (a == 1 ? (long long)W : 1ll);
+        const long long st = a == 0 ? HW : (a == 1 ? (long long)P : 1ll);
         const float ga = a == 0 ? g0 : (a == 1 ? g1 : g2);
         float s = ga;
         s = fmaf(fd_axis(u, n, k, i, st), g0, s);
@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(256) k_jac_direction(const float *gin, const f
 cudaError_t launch_jac_direction(const float *gin, const float *u, float *gout, Dims d,
                                  cudaStream_t s) {
     VoxGrid g(d.D, d.H, d.W);
-    k_jac_direction<<<g.grid, g.block, 0, s>>>(gin, u, gout, d.D, d.H, d.W);
+    k_jac_direction<<<g.grid, g.block, 0, s>>>(gin, u, gout, d.D, d.H, d.W, d.pitch());
     note_launch();
     return cudaGetLastError();
 }
