@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(256) k_compose(const float *__restrict__ u,
     float dz = -e * d[i], dy = -e * d[N + i], dx = -e * d[2 * N + i];
     float gz, gy, gx;
     TriPending q[3];  // the compose's cell (the same as the fused schedule's)
-    tri_issue_step3(q, u, N, D, H, W, z, y, x, dz, dy, dx);
+    tri_issue_step3(q, u, N, D, H, W, W, z, y, x, dz, dy, dx);
 #pragma unroll
     for (int ch = 0; ch < 3; ++ch) {
         float s = tri_finish<false>(q[ch], gz, gy, gx);
@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(256) k_compose_fields(const float *__restrict_
     const float dz = delta[i], dy = delta[N + i], dx = delta[2 * N + i];
     float gz, gy, gx, r[3];
     TriPending q[3];
-    tri_issue3(q, u, N, D, H, W, z, y, x, dz, dy, dx);
+    tri_issue3(q, u, N, D, H, W, W, z, y, x, dz, dy, dx);
 #pragma unroll
     for (int ch = 0; ch < 3; ++ch) r[ch] = tri_finish<false>(q[ch], gz, gy, gx);
     uo[i] = dz + r[0];

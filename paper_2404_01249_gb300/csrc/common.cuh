@@ -192,47 +192,16 @@ __device__ __forceinline__ void tri_issue_p(TriPending &p, const T *__restrict__
     if (z1 && y1 && x1) p.c111 = ld_field(q1 + P + 1);
 }
 
-// The compose's sample u(x + delta) at a grid voxel (z, y, x): for a step
-// shorter than one voxel on every axis the cell's corners are the voxel itself
-// and its neighbours on the side of each component's sign, with the exact
-// weights |delta| (so u is sampled exactly when delta is 0 on an axis); longer
-// steps take tri_issue_p's cell.  tri_finish completes either.
-template <class T>
-__device__ __forceinline__ void tri_issue_step(TriPending &p, const T *__restrict__ v, int D,
-                                               int H, int W, int P, int z, int y, int x,
-                                               float uz, float uy, float ux) {
-    if (!(fabsf(uz) < 1.0f && fabsf(uy) < 1.0f && fabsf(ux) < 1.0f)) {
-        tri_issue_p(p, v, D, H, W, P, z, y, x, uz, uy, ux);
-        return;
-    }
-    p.tz = fabsf(uz);
-    p.ty = fabsf(uy);
-    p.tx = fabsf(ux);
-    const int sz = uz < 0.0f ? -1 : 1, sy = uy < 0.0f ? -1 : 1, sx = ux < 0.0f ? -1 : 1;
-    const bool zo = z + sz >= 0 && z + sz < D, yo = y + sy >= 0 && y + sy < H,
-               xo = x + sx >= 0 && x + sx < W;
-    // 32-bit offsets: buffers hold fewer than 2^31 elements
-    const T *q0 = v + (z * H + y) * P + x, *q1 = q0 + sz * H * P;
-    const int oy = sy * P;
-    p.c000 = ld_field(q0);
-    p.c001 = xo ? ld_field(q0 + sx) : 0.0f;
-    p.c010 = yo ? ld_field(q0 + oy) : 0.0f;
-    p.c011 = yo && xo ? ld_field(q0 + oy + sx) : 0.0f;
-    p.c100 = zo ? ld_field(q1) : 0.0f;
-    p.c101 = zo && xo ? ld_field(q1 + sx) : 0.0f;
-    p.c110 = zo && yo ? ld_field(q1 + oy) : 0.0f;
-    p.c111 = zo && yo && xo ? ld_field(q1 + oy + sx) : 0.0f;
-}
-
-// The same cells for three channels of a field, N elements apart: the cell,
-// its place and the choice of path are worked out once for all three.
+// The same cell for three channels of a field, N elements apart (rows of P
+// elements): the cell, its place and the choice of path are worked out once for
+// all three.
 template <class T>
 __device__ __forceinline__ void tri_issue3(TriPending (&p)[3], const T *__restrict__ v,
-                                           long long N, int D, int H, int W, int z, int y, int x,
-                                           float uz, float uy, float ux) {
+                                           long long N, int D, int H, int W, int P, int z, int y,
+                                           int x, float uz, float uy, float ux) {
     const float LIM = 1048576.0f;
     if (!(fabsf(uz) < LIM && fabsf(uy) < LIM && fabsf(ux) < LIM)) {
-        tri_issue_p(p[0], v, D, H, W, W, z, y, x, uz, uy, ux);
+        tri_issue_p(p[0], v, D, H, W, P, z, y, x, uz, uy, ux);
         p[1] = p[2] = p[0];
         return;
     }
@@ -242,18 +211,18 @@ __device__ __forceinline__ void tri_issue3(TriPending (&p)[3], const T *__restri
     const bool y0 = iy >= 0 && iy < H, y1 = iy + 1 >= 0 && iy + 1 < H;
     const bool x0 = ix >= 0 && ix < W, x1 = ix + 1 >= 0 && ix + 1 < W;
     // corners outside the grid read as zero
-    const T *q0 = v + ((long long)iz * H + iy) * W + ix, *q1 = q0 + (long long)H * W;
+    const T *q0 = v + ((long long)iz * H + iy) * P + ix, *q1 = q0 + (long long)H * P;
     if (z0 && z1 && y0 && y1 && x0 && x1) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             p[c].c000 = ld_field(q0);
             p[c].c001 = ld_field(q0 + 1);
-            p[c].c010 = ld_field(q0 + W);
-            p[c].c011 = ld_field(q0 + W + 1);
+            p[c].c010 = ld_field(q0 + P);
+            p[c].c011 = ld_field(q0 + P + 1);
             p[c].c100 = ld_field(q1);
             p[c].c101 = ld_field(q1 + 1);
-            p[c].c110 = ld_field(q1 + W);
-            p[c].c111 = ld_field(q1 + W + 1);
+            p[c].c110 = ld_field(q1 + P);
+            p[c].c111 = ld_field(q1 + P + 1);
             q0 += N;
             q1 += N;
         }
@@ -262,12 +231,12 @@ __device__ __forceinline__ void tri_issue3(TriPending (&p)[3], const T *__restri
         for (int c = 0; c < 3; ++c) {
             p[c].c000 = z0 && y0 && x0 ? ld_field(q0) : 0.0f;
             p[c].c001 = z0 && y0 && x1 ? ld_field(q0 + 1) : 0.0f;
-            p[c].c010 = z0 && y1 && x0 ? ld_field(q0 + W) : 0.0f;
-            p[c].c011 = z0 && y1 && x1 ? ld_field(q0 + W + 1) : 0.0f;
+            p[c].c010 = z0 && y1 && x0 ? ld_field(q0 + P) : 0.0f;
+            p[c].c011 = z0 && y1 && x1 ? ld_field(q0 + P + 1) : 0.0f;
             p[c].c100 = z1 && y0 && x0 ? ld_field(q1) : 0.0f;
             p[c].c101 = z1 && y0 && x1 ? ld_field(q1 + 1) : 0.0f;
-            p[c].c110 = z1 && y1 && x0 ? ld_field(q1 + W) : 0.0f;
-            p[c].c111 = z1 && y1 && x1 ? ld_field(q1 + W + 1) : 0.0f;
+            p[c].c110 = z1 && y1 && x0 ? ld_field(q1 + P) : 0.0f;
+            p[c].c111 = z1 && y1 && x1 ? ld_field(q1 + P + 1) : 0.0f;
             q0 += N;
             q1 += N;
         }
@@ -280,19 +249,24 @@ __device__ __forceinline__ void tri_issue3(TriPending (&p)[3], const T *__restri
     }
 }
 
+// The compose's sample u(x + delta) at a grid voxel (z, y, x): for a step
+// shorter than one voxel on every axis the cell's corners are the voxel itself
+// and its neighbours on the side of each component's sign, with the exact
+// weights |delta| (so u is sampled exactly when delta is 0 on an axis); longer
+// steps take tri_issue3's cell.  tri_finish completes either.
 template <class T>
 __device__ __forceinline__ void tri_issue_step3(TriPending (&p)[3], const T *__restrict__ v,
-                                                long long N, int D, int H, int W, int z, int y,
-                                                int x, float uz, float uy, float ux) {
+                                                long long N, int D, int H, int W, int P, int z,
+                                                int y, int x, float uz, float uy, float ux) {
     if (!(fabsf(uz) < 1.0f && fabsf(uy) < 1.0f && fabsf(ux) < 1.0f)) {
-        tri_issue3(p, v, N, D, H, W, z, y, x, uz, uy, ux);
+        tri_issue3(p, v, N, D, H, W, P, z, y, x, uz, uy, ux);
         return;
     }
     const int sz = uz < 0.0f ? -1 : 1, sy = uy < 0.0f ? -1 : 1, sx = ux < 0.0f ? -1 : 1;
     const bool zo = z + sz >= 0 && z + sz < D, yo = y + sy >= 0 && y + sy < H,
                xo = x + sx >= 0 && x + sx < W;
-    const T *q0 = v + ((long long)z * H + y) * W + x, *q1 = q0 + (long long)sz * H * W;
-    const int oy = sy * W;
+    const T *q0 = v + ((long long)z * H + y) * P + x, *q1 = q0 + (long long)sz * H * P;
+    const int oy = sy * P;
     if (zo && yo && xo) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {

@@ -74,11 +74,11 @@ __global__ void __launch_bounds__(256) k_inverse_terms(const float *__restrict__
         const float wz = w[i], wy = w[N + i], wx = w[2 * N + i];
         float A[3], B[3], G[3][3], gz, gy, gx;
         TriPending q[3];
-        tri_issue3(q, w, N, D, H, W, z, y, x, uz, uy, ux);
+        tri_issue3(q, w, N, D, H, W, W, z, y, x, uz, uy, ux);
         A[0] = uz + tri_finish<false>(q[0], gz, gy, gx);
         A[1] = uy + tri_finish<false>(q[1], gz, gy, gx);
         A[2] = ux + tri_finish<false>(q[2], gz, gy, gx);
-        tri_issue3(q, u, N, D, H, W, z, y, x, wz, wy, wx);
+        tri_issue3(q, u, N, D, H, W, W, z, y, x, wz, wy, wx);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const float wc = c == 0 ? wz : (c == 1 ? wy : wx);

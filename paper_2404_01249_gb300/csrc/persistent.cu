@@ -196,7 +196,7 @@ __device__ __forceinline__ void tri_issue_cg(TriPending &p, const float *v, int 
 }
 
 // The compose's sample of a field written inside this launch: the cell and
-// weights of tri_issue_step (this voxel and its neighbours on the side of the
+// weights of tri_issue_step3 (this voxel and its neighbours on the side of the
 // step's sign for a step shorter than one voxel, tri_issue_cg's cell
 // otherwise), L2 loads.
 __device__ __forceinline__ void tri_issue_step_cg(TriPending &p, const float *v, int D, int H,

@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(256) k_square_adjoint(const float *__restrict_
         b[2] = gb[2 * N + i];
         float G[3][3];
         TriPending t[3];
-        tri_issue3(t, u, N, D, H, W, z, y, x, uz, uy, ux);
+        tri_issue3(t, u, N, D, H, W, W, z, y, x, uz, uy, ux);
 #pragma unroll
         for (int c = 0; c < 3; ++c) tri_finish<true>(t[c], G[c][0], G[c][1], G[c][2]);
 #pragma unroll
