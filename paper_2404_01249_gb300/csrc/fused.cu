@@ -38,8 +38,13 @@ thread_local const TileChoice *g_force = nullptr;  // a candidate under measurem
 // a CTA: there the shorter march of 32 x 8 tiles counts (a 32^3 pair: 1.80 ms
 // with 32 x 16 tiles on both levels, 1.70 with 32 x 8; K4 on 16 x 32 x 32
 // voxels 14.4 against 12.3 us, but on 32 x 64 x 64 voxels 22.6 against 24.3).
-int default_wide(int kernel, Dims d) {
+// Without smoothing K4 has no halo that the taller tile would save, and takes
+// 32 x 8 tiles with their three CTAs per SM (ten MSE iterations without either
+// smoothing: 160 x 192 x 224 3,367 us on 32 x 16 tiles, 3,271 on 32 x 8, 40 x 24 x 64
+// 113 and 103; before the passes were pipelined 3,393 and 106).
+int default_wide(int kernel, int radius, Dims d) {
     const long long tiles = (long long)((d.W + FX - 1) / FX) * ((d.H + 15) / 16);
+    if (kernel == 3 && radius == 0) return 0;
     return kernel >= 2 && tiles * d.D >= num_sms();
 }
 
@@ -48,7 +53,7 @@ TileChoice tile_choice(int kernel, int radius, int su, Dims d) {
     std::lock_guard<std::mutex> lock(g_tune_mu);
     auto it = g_tune.find(TuneKey{kernel, radius, su, d.D, d.H, d.W});
     if (it != g_tune.end()) return it->second;
-    return TileChoice{default_wide(kernel, d), 0};
+    return TileChoice{default_wide(kernel, radius, d), 0};
 }
 
 inline LaunchGeom geometry(int occ, int nw, int ty, float extra, Dims d, int tz) {
@@ -472,7 +477,7 @@ fa_status fused_autotune_level(FusedBuffers &fb, WsHeader *h, const fa_params *p
     for (int kernel = (p->loss == FA_LOSS_LNCC ? 0 : 2); kernel < 4 && result == FA_OK; ++kernel) {
         const int radius = kernel < 2 ? p->window / 2 : (kernel == 2 ? g3.R : g4.R);
         const int sukey = kernel == 3 && su ? 1 : 0;
-        TileChoice best{default_wide(kernel, d), 0};
+        TileChoice best{default_wide(kernel, radius, d), 0};
         float best_ms = -1.0f;
         for (int wide = 0; wide < (kernel >= 2 ? 2 : 1) && result == FA_OK; ++wide)
             for (int tz : tzs) {
