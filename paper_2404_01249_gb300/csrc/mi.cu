@@ -157,12 +157,16 @@ __global__ void __launch_bounds__(256) k_mi_range(const float *__restrict__ If,
 // non-zero bins to the global histogram.
 // Bound: the shared-memory atomics, 32 per voxel.  6.9 M voxels, 32 bins:
 // 590 us with one copy per warp (lanes of a warp serialised on the few bins
-// of a smooth region), 88 us with 16 copies.
+// of a smooth region), 88 us with 16 copies.  Where 152 blocks of 512 threads
+// cover the volume with one voxel per thread, zeroing and reading out the copies
+// counts: four of them then (the loss and its gradient on 13,440 voxels, 16, 32
+// and 64 bins: 20.5, 19.8 and 29.0 us against 21.9, 21.9 and 29.7 with up to 16
+// in blocks of 1,024; on 107,604 voxels 22.6 and 22.7, the line).
 constexpr int kHistThreads = 1024, kHistIters = 64;
 constexpr size_t kHistSmem = 196 * 1024;
+constexpr long long kMiGradOne = 1ll << 20;  // the gradient's one-voxel form up to here
 
-int hist_log_copies(int nb) {
-    int lc = 5;
+int hist_log_copies(int nb, int lc) {  // at most 2^lc
     while (lc > 0 && ((size_t)nb << lc) * 8 > kHistSmem) --lc;
     return lc;
 }
@@ -274,10 +278,27 @@ __global__ void __launch_bounds__(1024) k_mi_table(const unsigned long long *__r
     }
 }
 
+// The values of V voxels from i on (V = 4: as load4).
+template <int V>
+__device__ __forceinline__ void load_v(float (&v)[V], const float *__restrict__ p, long long i,
+                                       long long N) {
+    if constexpr (V == 4)
+        load4(v, p, i, N);
+    else
+        v[0] = __ldg(p + i);
+}
+
+// V adjacent voxels per thread and step.  With four their loads and table reads
+// overlap, bound by the table's shared-memory reads; with one, a small volume
+// has four times the threads.  The loss and its gradient, 32 bins, one against
+// four (us): 13,440 voxels 18.9 and 19.8, 512,000 31.5 and 31.9, 1.4 M 49.7 and
+// 49.2, 6.9 M 160 and 154: hence kMiGradOne.
+template <int V>
 __global__ void __launch_bounds__(256) k_mi_grad(const float *__restrict__ I,
                                                  const float *__restrict__ J,
                                                  const float *__restrict__ grad, long long N,
-                                                 float count, int B, const unsigned *__restrict__ keys,
+                                                 float count, int B,
+                                                 const unsigned *__restrict__ keys,
                                                  const float *__restrict__ Tg, float *dJ,
                                                  float *g) {
     extern __shared__ float T[];
@@ -285,15 +306,13 @@ __global__ void __launch_bounds__(256) k_mi_grad(const float *__restrict__ I,
     __syncthreads();
     const MiMap mf = mi_map(keys, 0, B), mm = mi_map(keys, 1, B);
     const float c = -mm.s / count;
-    // four adjacent voxels per thread and step: their loads and table reads
-    // overlap (one voxel: 48 us on 6.9 M voxels; four: 40 us, bound by the table's shared-memory reads)
-    for (long long i = 4 * ((long long)blockIdx.x * blockDim.x + threadIdx.x); i < N;
-         i += 4ll * gridDim.x * blockDim.x) {
-        float Iv[4], Jv[4], dj[4];
-        load4(Iv, I, i, N);
-        load4(Jv, J, i, N);
+    for (long long i = V * ((long long)blockIdx.x * blockDim.x + threadIdx.x); i < N;
+         i += (long long)V * gridDim.x * blockDim.x) {
+        float Iv[V], Jv[V], dj[V];
+        load_v(Iv, I, i, N);
+        load_v(Jv, J, i, N);
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
+        for (int e = 0; e < V; ++e) {
             const float xf = mf.coord(Iv[e]), xm = mm.coord(Jv[e]);
             const float ff = floorf(xf), fm = floorf(xm);
             float wf[4], dm[4];
@@ -312,28 +331,29 @@ __global__ void __launch_bounds__(256) k_mi_grad(const float *__restrict__ I,
             }
             dj[e] = c * acc;
         }
-        const bool four = i + 4 <= N;
+        const bool all = i + V <= N;
         if (dJ) {
-            if (four) {
-                *(float4 *)(dJ + i) = make_float4(dj[0], dj[1], dj[2], dj[3]);
+            if (V == 4 && all) {
+                *(float4 *)(dJ + i) = make_float4(dj[0], dj[1 % V], dj[2 % V], dj[3 % V]);
             } else {
 #pragma unroll
-                for (int e = 0; e < 4; ++e)
+                for (int e = 0; e < V; ++e)
                     if (i + e < N) dJ[i + e] = dj[e];
             }
         }
         if (g) {
-            const bool vec = four && (N & 3) == 0;  // the other channels start on 16 bytes too
+            const bool vec = V == 4 && all && (N & 3) == 0;  // the other channels start on 16 bytes too
 #pragma unroll
             for (int ch = 0; ch < 3; ++ch) {
                 const float *src = grad + ch * N + i;
                 float *dst = g + ch * N + i;
                 if (vec) {
                     const float4 q = *(const float4 *)src;
-                    *(float4 *)dst = make_float4(dj[0] * q.x, dj[1] * q.y, dj[2] * q.z, dj[3] * q.w);
+                    *(float4 *)dst = make_float4(dj[0] * q.x, dj[1 % V] * q.y, dj[2 % V] * q.z,
+                                                 dj[3 % V] * q.w);
                 } else {
 #pragma unroll
-                    for (int e = 0; e < 4; ++e)
+                    for (int e = 0; e < V; ++e)
                         if (i + e < N) dst[e] = dj[e] * src[e];
                 }
             }
@@ -379,13 +399,15 @@ cudaError_t launch_mi(const float *I, const float *J, const float *grad, Dims d,
     const int nb = bins * bins;
     cudaError_t e = cudaMemsetAsync(b.hist, 0, sizeof(unsigned long long) * nb, s);
     if (e != cudaSuccess) return e;
-    const int lc = hist_log_copies(nb);
     prepare(k_mi_hist, kHistSmem, kHistThreads);
-    const long long most = (N + kHistThreads - 1) / kHistThreads;
+    const bool one_pass = N <= 512ll * num_sms();
+    const int threads = one_pass ? 512 : kHistThreads;
+    const int lc = hist_log_copies(nb, one_pass ? 2 : 5);
+    const long long most = (N + threads - 1) / threads;
     long long hb = (most + kHistIters - 1) / kHistIters;
     hb = hb < num_sms() ? num_sms() : hb;
     hb = hb < most ? hb : most;
-    k_mi_hist<<<(unsigned)hb, kHistThreads, ((size_t)nb << lc) * 8, s>>>(
+    k_mi_hist<<<(unsigned)hb, threads, ((size_t)nb << lc) * 8, s>>>(
         I, J, N, d.W, d.pitch(), bins, lc, b.range, b.hist, h);
     note_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -394,8 +416,15 @@ cudaError_t launch_mi(const float *I, const float *J, const float *grad, Dims d,
     note_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (dJ || g) {
-        k_mi_grad<<<grid_blocks(N), 256, sizeof(float) * nb, s>>>(
-            I, J, grad, N, (float)d.N(), bins, b.range, b.T, dJ, g);
+        if (N <= kMiGradOne) {
+            long long gb = (N + 255) / 256;
+            gb = gb < 152 * 4 ? gb : 152 * 4;
+            k_mi_grad<1><<<(unsigned)gb, 256, sizeof(float) * nb, s>>>(
+                I, J, grad, N, (float)d.N(), bins, b.range, b.T, dJ, g);
+        } else {
+            k_mi_grad<4><<<grid_blocks(N), 256, sizeof(float) * nb, s>>>(
+                I, J, grad, N, (float)d.N(), bins, b.range, b.T, dJ, g);
+        }
         note_launch();
     }
     return cudaGetLastError();
