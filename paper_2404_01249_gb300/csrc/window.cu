@@ -6,11 +6,17 @@ namespace fa {
 
 namespace {
 
+// Deepest slab.  A thread of the forward kernel adds two terms per plane whose
+// lower limb is up to 2^19 in magnitude in 32 bits: 2^11 planes could overflow.
+// (The cost model stays below 64; a caller's tile table may ask for any depth.)
+constexpr int kMaxSlab = 1024;
+
 template <int R>
 LaunchGeom window_geom(Dims d, int tz, int occ) {
     using G = WinTile<R>;
     LaunchGeom g;
     const int gx = (d.W + FX - 1) / FX, gy = (d.H + G::TY - 1) / G::TY;
+    tz = tz < kMaxSlab ? tz : kMaxSlab;
     g.tz = tz > 0 ? (tz < d.D ? tz : d.D) : choose_tz(d.D, gx * gy, window_slab_extra(R), occ);
     g.grid = dim3(gx, gy, (d.D + g.tz - 1) / g.tz);
     g.block = dim3(G::NT);
