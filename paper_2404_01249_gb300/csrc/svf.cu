@@ -384,15 +384,17 @@ extern "C" fa_status fa_svf_loss_grad(const fa_vol *fixed, const fa_vol *moving,
     FA_CUDA_TRY(launch_header_reset(q.h, s));
     FA_CUDA_TRY(launch_absmax2(If, Im, d.N(), q.h, s));
     if (p1.loss == FA_LOSS_MI) FA_CUDA_TRY(launch_mi_range(If, Im, d, q.mi, s));
-    // exp(v) - id is made in the caller's field unless that holds an image the
-    // loss still reads, or the gradient that is written after it
+    // exp(v) - id is made in the caller's field unless that holds v (whose
+    // scaling would read what it has written), an image the loss still reads,
+    // or the gradient that is written after it
     const size_t b = sizeof(float) * 3 * d.N();
     auto apart = [&](const void *p, size_t n) {
         const char *x = (const char *)u_out_opt->data, *y = (const char *)p;
         return x + b <= y || y + n <= x;
     };
     float *uM = nullptr;
-    if (u_out_opt && apart(If, b / 3) && apart(Im, b / 3) && apart(grad_v_out->data, b))
+    if (u_out_opt && apart(v->data, b) && apart(If, b / 3) && apart(Im, b / 3) &&
+        apart(grad_v_out->data, b))
         uM = (float *)u_out_opt->data;
     FA_TRY(svf_eval(q, &p1, steps, d, If, Im, (const float *)v->data, true, loss_dev, s, uM,
                     (float *)grad_v_out->data));

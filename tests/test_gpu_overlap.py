@@ -45,3 +45,27 @@ def test_adjoint_field_gradient_over_the_fixed_image(fa, shape, channel):
     assert torch.equal(du, ref["dL_du"])
     assert torch.equal(dI, ref["dL_dfixed"])
     assert torch.equal(dM, ref["dL_dmoving"])
+
+
+@pytest.mark.parametrize("steps", [0, 3])
+@pytest.mark.parametrize("shift", [0, 0.5])  # u_out starts this much of a field behind v
+def test_svf_displacement_over_the_velocity(fa, steps, shift):
+    shape = (40, 52, 64)
+    n3 = 3 * shape[0] * shape[1] * shape[2]
+    f, m, _ = synth.blobs_pair(shape=shape, sigma=3.0)
+    f, m = torch.from_numpy(f).cuda(), torch.from_numpy(m).cuda()
+    v = torch.from_numpy(synth.random_field(shape, 4.0, 1.5, seed=6)).float().cuda()
+    L, g, u = fa.fa_svf_loss_grad(f, m, v, steps)
+    off = int(shift * n3)
+    buf = torch.empty(n3 + off, device="cuda")
+    # early elements of u_out go where late ones of v are
+    vo, uo = buf[:n3].view((3,) + shape), buf[off:].view((3,) + shape)
+    vo.copy_(v)
+    lib, p = fa.load(), fa.RegParams(scales=(1,), iters=(0,)).to_c()
+    ws = fa.workspace(lib.fa_register_svf_workspace_size(*shape, ctypes.byref(p), steps))
+    go, loss = torch.empty_like(v), torch.empty((), device="cuda")
+    fa._check(lib.fa_svf_loss_grad(fa._vol(f, 1), fa._vol(m, 1), fa._vol(vo, 3), ctypes.byref(p),
+                                   steps, fa._ptr(loss), fa._vol(go, 3), fa._vol(uo, 3),
+                                   fa._ptr(ws), ws.numel(), fa._stream()))
+    assert float(loss) == float(L)
+    assert torch.equal(go, g) and torch.equal(uo, u)
