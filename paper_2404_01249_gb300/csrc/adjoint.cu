@@ -9,16 +9,16 @@
 //   dL/dI_m(p) = sum_x dL/dJ(x) w_p(x)            (the adjoint of the warp:
 //                w_p(x) is the trilinear weight of corner p at x + u(x))
 //
-// Without dL/dI_f the call runs on the window kernels: the warp (J and grad
-// I_m at x + u), the forward sums of both images (cc, the adjoint
-// coefficients, the loss) and K2 (the adjoint window sums, dL/du, and dL/dJ
-// for the scatter).  With
-// dL/dI_f it runs the per-op LNCC kernels, which also form the fixed image's
-// coefficients.  The scatter of dL/dI_m accumulates quantised contributions
+// The call runs on the window kernels: the warp (J and, for dL/du, grad I_m at
+// x + u), the forward sums of both images (cc, the adjoint coefficients, the
+// loss) and the adjoint sums (dL/du, and dL/dJ for the scatter), once more with
+// the images' roles exchanged for dL/dI_f.  One forward pass over both images
+// takes 134 us on 160 x 192 x 224; the fixed image's statistics in a pass of
+// their own, which a loop makes once per level, cost 27 us more.
+// The scatter of dL/dI_m accumulates quantised contributions
 // in int64 with integer atomics, so the result does not depend on the order
 // in which threads add (the same fixed-point scheme as the window sums).
 #include "ops.h"
-#include "register.h"
 #include "scatter.cuh"
 #include "validate.h"
 
@@ -34,26 +34,6 @@ struct AdjointBuffers {
     float *J, *grad, *dJ;
     long long *acc;
 };
-
-// The fused route (no dL/dI_f): the fused kernels' buffers, dL/dJ and the
-// scatter accumulator.
-struct AdjointFusedBuffers {
-    WsHeader *h;
-    FusedBuffers fb;
-    float *dJ;
-    long long *acc;
-};
-
-AdjointFusedBuffers adjoint_fused_carve(void *base, size_t cap, long long N, size_t *bytes) {
-    WsCarver c(base, cap);
-    AdjointFusedBuffers b;
-    b.h = c.take<WsHeader>(1);
-    fused_carve(c, N, &b.fb);
-    b.dJ = c.take<float>(N);
-    b.acc = c.take<long long>(N);
-    *bytes = c.off;
-    return b;
-}
 
 AdjointBuffers adjoint_carve(void *base, size_t cap, long long N, size_t *bytes) {
     WsCarver c(base, cap);
@@ -146,10 +126,9 @@ fa_status scatter_to_moving(const float *dJ, const float *u, long long *acc, WsH
 extern "C" size_t fa_warp_lncc_adjoint_workspace_size(int32_t D, int32_t H, int32_t W) {
     fa::clear_error();
     if (D < 1 || H < 1 || W < 1) return 0;
-    size_t plain = 0, fused = 0;
-    fa::adjoint_carve(nullptr, ~size_t(0), (long long)D * H * W, &plain);
-    fa::adjoint_fused_carve(nullptr, ~size_t(0), (long long)D * H * W, &fused);
-    return plain > fused ? plain : fused;
+    size_t bytes = 0;
+    fa::adjoint_carve(nullptr, ~size_t(0), (long long)D * H * W, &bytes);
+    return bytes;
 }
 
 extern "C" fa_status fa_warp_lncc_adjoint(const fa_vol *fixed, const fa_vol *moving,
@@ -195,25 +174,13 @@ extern "C" fa_status fa_warp_lncc_adjoint(const fa_vol *fixed, const fa_vol *mov
     float *dIf = dL_dfixed_opt ? (float *)dL_dfixed_opt->data : nullptr;
     float *dIm = dL_dmoving_opt ? (float *)dL_dmoving_opt->data : nullptr;
 
-    if (!dIf) {  // the fused kernels: warp, K1 (forward), K2 (dL/du and dL/dJ), scatter
-        size_t need = 0;
-        AdjointFusedBuffers b = adjoint_fused_carve(ws, ws_bytes, N, &need);
-        FA_CUDA_TRY(launch_header_reset(b.h, s));
-        float *g = du ? du : (dIm ? b.fb.g : nullptr);
-        FA_CUDA_TRY(fused_warp_lncc_adjoint(I, Im, uu, b.fb, d, window, cc_eps, b.h, loss_dev, g,
-                                            dIm ? b.dJ : nullptr, s));
-        if (dIm) FA_TRY(scatter_to_moving(b.dJ, uu, b.acc, b.h, d, dIm, s));
-        return FA_OK;
-    }
-
     size_t need = 0;
     AdjointBuffers b = adjoint_carve(ws, ws_bytes, N, &need);
-
     FA_CUDA_TRY(launch_header_reset(b.h, s));
     FA_CUDA_TRY(launch_warp(Im, uu, b.J, du ? b.grad : nullptr, d, s));
     FA_CUDA_TRY(launch_absmax2(I, b.J, N, b.h, s));
-    FA_CUDA_TRY(launch_lncc_forward(I, b.J, d, window, cc_eps, true, dIf != nullptr, b.h, b.lb,
-                                    s));
+    FA_CUDA_TRY(launch_lncc_forward(I, b.J, d, window, cc_eps, du || dIf || dIm, dIf != nullptr,
+                                    b.h, b.lb, s));
     FA_CUDA_TRY(launch_loss_finalize(b.h, N, -1.0f, loss_dev, s));
     if (du || dIf || dIm)
         FA_CUDA_TRY(launch_lncc_backward(I, b.J, du ? b.grad : nullptr, d, window, b.h, b.lb,

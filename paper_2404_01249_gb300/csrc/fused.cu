@@ -160,10 +160,8 @@ cudaError_t launch_k1(const float *If, const float *J, const long long *sI, cons
     return launch_window_fwd(kFwdGiven, a, d, window, tile_choice(0, window / 2, 0, d).tz, s);
 }
 
-// dJout (may be NULL): also write dL/dJ, which the adjoint's scatter needs.
 cudaError_t launch_k2(const float *If, const float *gJ, const float *J, const float *coef,
-                      const WsHeader *h, float *g, float *dJout, Dims d, int window,
-                      cudaStream_t s) {
+                      const WsHeader *h, float *g, Dims d, int window, cudaStream_t s) {
     GradArgs a{};
     a.I = If;
     a.J = J;
@@ -171,7 +169,6 @@ cudaError_t launch_k2(const float *If, const float *gJ, const float *J, const fl
     a.coef = coef;
     a.h = h;
     a.g = g;
-    a.dJ = dJout;
     return launch_window_grad(false, a, d, window, tile_choice(1, window / 2, 0, d).tz, s);
 }
 
@@ -385,7 +382,7 @@ fa_status fused_iteration(FusedBuffers &fb, WsHeader *h, const fa_params *p, Dim
                                 true, s));
         FA_CUDA_TRY(stop(FA_K_FUSED_WARP_LNCC));
         FA_CUDA_TRY(start(FA_K_FUSED_LNCC_GRAD));
-        FA_CUDA_TRY(launch_k2(it.If, fb.gJ, fb.J, fb.coef, h, fb.g, nullptr, d, p->window, s));
+        FA_CUDA_TRY(launch_k2(it.If, fb.gJ, fb.J, fb.coef, h, fb.g, d, p->window, s));
         FA_CUDA_TRY(stop(FA_K_FUSED_LNCC_GRAD));
     } else if (p->loss == FA_LOSS_MI) {
         FA_CUDA_TRY(start(FA_K_FUSED_LNCC_GRAD));
@@ -461,7 +458,7 @@ fa_status fused_autotune_level(FusedBuffers &fb, WsHeader *h, const fa_params *p
             case 0:
                 return launch_k1(If, fb.J, fb.sI, fb.varI, fb.coef, h, d, p->window, p->cc_eps,
                                    true, s);
-            case 1: return launch_k2(If, fb.gJ, fb.J, fb.coef, h, fb.g, nullptr, d, p->window, s);
+            case 1: return launch_k2(If, fb.gJ, fb.J, fb.coef, h, fb.g, d, p->window, s);
             case 2: return dispatch_k3(fb.g, m, v, p->state_storage, fb.dir, h, d, g3, ac, 0, s);
             default:
                 return dispatch_k4(u, fb.dir, u_alt, p->field_storage, Im, fb.J, fb.gJ, h, d, g4,
@@ -546,28 +543,6 @@ int fused_tile_choices(int32_t *out, int capacity) {
 cudaError_t fused_lncc_forward_only(const float *If, const FusedBuffers &fb, Dims d, int window,
                                     float cc_eps, WsHeader *h, cudaStream_t s) {
     return launch_k1(If, fb.J, fb.sI, fb.varI, nullptr, h, d, window, cc_eps, false, s);
-}
-
-cudaError_t fused_warp_lncc_adjoint(const float *If, const float *Im, const float *u,
-                                    const FusedBuffers &fb, Dims d, int window, float cc_eps,
-                                    WsHeader *h, float *loss_dev, float *g, float *dJ,
-                                    cudaStream_t s) {
-    cudaError_t e;
-    if ((e = launch_warp(Im, u, fb.J, g ? fb.gJ : nullptr, d, s)) != cudaSuccess) return e;
-    if ((e = launch_absmax2(If, fb.J, d.N(), h, s)) != cudaSuccess) return e;
-    // one pass over both images (134 us on 160 x 192 x 224): the fixed image's
-    // own pass, which a loop makes once per level, cost 27 us more here
-    FwdArgs a{};
-    a.I = If;
-    a.J = fb.J;
-    a.coef = fb.coef;
-    a.h = h;
-    a.cc_eps = cc_eps;
-    a.write_coef = g != nullptr;
-    if ((e = launch_window_fwd(kFwdBoth, a, d, window, 0, s)) != cudaSuccess) return e;
-    if ((e = launch_loss_finalize(h, d.N(), -1.0f, loss_dev, s)) != cudaSuccess) return e;
-    if (!g) return cudaSuccess;
-    return launch_k2(If, fb.gJ, fb.J, fb.coef, h, g, dJ, d, window, s);
 }
 
 // Self-test of the bounded wait: one thread waits on an mbarrier that no
