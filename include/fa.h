@@ -597,8 +597,10 @@ fa_status fa_inverse_energy_grad(const fa_vol *u, const fa_vol *w, float *energy
  * fixed/moving: C=1 volumes of p->storage; u_out and the optional uF_out,
  * uM_out: C=3 FA_F32 on the last level's grid.  final_loss_dev receives
  * L(I_f, I_m o (id + u_out)), mid_loss_dev L(I_f o phi_F, I_m o phi_M)
- * (device floats, either may be NULL).  Per-op kernels, no graph
- * recording (p->mode and p->graph are ignored).  Asynchronous; workspace of
+ * (device floats, either may be NULL).  No graph recording (p->mode and
+ * p->graph are ignored); each map's update runs as the two update kernels of
+ * the fused schedule where the rows and the Gaussians allow it, whose bounded
+ * waits report through the status word.  Asynchronous; workspace of
  * fa_register_symmetric_workspace_size bytes (0: invalid arguments).
  *
  * fa_symmetric_loss_grad evaluates L(I_f o phi_F, I_m o phi_M) and both

@@ -15,9 +15,10 @@ namespace {
 
 // ------------------------------------------------------------- tile choices
 // Per (kernel, radius, compose variant, level grid): the slab depth TZ
-// (0: the cost model above) and, for K3/K4 on the TMA path, 32 x 16 tiles
-// of 16 warps instead of 32 x 8.  fa_autotune measures candidates and fills
-// the table; every choice computes the same bits.
+// (0: the cost model of launch.cuh) and, for K3/K4 on the TMA path, 32 x 16
+// tiles instead of 32 x 8 (both of 8 warps: two rows per thread, or one).
+// fa_autotune measures candidates and fills the table; every choice computes
+// the same bits.
 struct TileChoice {
     int wide, tz;
 };
@@ -103,7 +104,7 @@ struct MapKeyHash {
 
 }  // namespace
 
-// Map of a [C][D][H][W] field of 2- (FP16), 4- or 8-byte elements (rows of d.pitch()
+// Map of a [C][D][H][W] field of 2- (FP16) or 4-byte elements (rows of d.pitch()
 // elements) with a {bx, by, 1, bc} box, zero fill outside the D x H x W grid
 // (so a padded row's tail is never read).  Encoded maps are kept per host
 // thread (a map is a function of its key alone; a lockstep batch reuses a
@@ -128,9 +129,8 @@ bool tmap(CUtensorMap *m, const void *base, int esize, Dims d, int C, int bx, in
     cuuint32_t box[4] = {(cuuint32_t)bx, (cuuint32_t)by, 1u, (cuuint32_t)bc};
     cuuint32_t es[4] = {1u, 1u, 1u, 1u};
     CUtensorMap tm;
-    const CUtensorMapDataType dt = esize == 8   ? CU_TENSOR_MAP_DATA_TYPE_INT64
-                                   : esize == 2 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
-                                                : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
+    const CUtensorMapDataType dt =
+        esize == 2 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
     CUresult r = fn(&tm, dt,
                     4, const_cast<void *>(base), dims, strides, box, es,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,

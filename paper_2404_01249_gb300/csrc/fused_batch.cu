@@ -122,7 +122,7 @@ __device__ __forceinline__ void window_tile(const A &a, int t, int &bx, int &by,
 }
 
 template <int R>
-__global__ void __launch_bounds__(WinTile<R>::NT, fwd_min_ctas(R, kFwdGiven))
+__global__ void __launch_bounds__(WinTile<R>::NT, fwd_min_ctas(R))
     k_lncc_fwd_batch(const __grid_constant__ K1Batch b) {
     const int k = batch_job(b.first, b.n, (int)blockIdx.x);
     int bx, by, bz;

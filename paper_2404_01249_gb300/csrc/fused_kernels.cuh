@@ -143,7 +143,7 @@ __device__ __forceinline__ void tma4(void *dst, const CUtensorMap *m, int x, int
 
 // Tensor maps of one launch (the ones a kernel does not use stay zero).
 struct Maps {
-    CUtensorMap a, b, c, d;
+    CUtensorMap a, b, c;
 };
 
 // The tensor maps a CTA's body loads through: generic addresses of maps in
@@ -155,7 +155,7 @@ struct MapRef {
 __device__ __forceinline__ MapRef map_ref(const Maps &m) { return MapRef{&m.a, &m.b, &m.c}; }
 
 }  // namespace
-// Map of a [C][D][H][W] field of 4- or 8-byte elements with rows of
+// Map of a [C][D][H][W] field of 2- (FP16) or 4-byte elements with rows of
 // d.pitch() elements, a {bx, by, 1, bc} box and zero fill outside the grid;
 // false when the field does not meet TMA's alignment rules.
 bool tmap(CUtensorMap *m, const void *base, int esize, Dims d, int C, int bx, int by, int bc);

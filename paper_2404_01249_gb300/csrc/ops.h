@@ -77,9 +77,10 @@ cudaError_t launch_window_grad(bool swap, GradArgs g, Dims d, int window, int tz
 // ---- plain LNCC / MSE (lncc.cu)
 // Header fields used: absmax_bits, coef_max_bits, loss_acc, status.
 struct LnccBuffers {
-    // [5][N] int64 each: part of the workspace sizes callers allocate by; the
-    // window sums stay on the chip, so only p0 is used, as scratch for a
-    // gradient that overlaps an input
+    // [5][N] int64 each.  The window sums stay on the chip: only p0 is used, as
+    // scratch for gradients that overlap an input.  fa_lncc_workspace_size
+    // counts both, and the limit of fa_lncc_fwd_bwd_noalloc (621,376 voxels in
+    // 64 MiB) is documented and tested by that size.
     long long *p0, *p1;
     float *coef;          // [7][N]: A, B, C hi, C lo, B', C' hi, C' lo
 };

@@ -24,7 +24,9 @@
 // 160 x 192 x 224: forward 155 -> 116 us, gradient 143 -> 119; on 40 x 48 x 56
 // 14 -> 9 and 12 -> 7 us; windows of 7 on 128 x 256 x 256: 215 -> 155 and
 // 250 -> 205 us; the loss with both gradients as a layer on 127 x 181 x 159:
-// 691 -> 227 us.
+// 691 -> 227 us, and at windows of 9, 11, 13 and 15 there 885 -> 351, 999 -> 408,
+// 1,105 -> 467 and 1,222 -> 532; ten iterations on 96 x 112 x 104 at these windows
+// 2,078 -> 1,477, 2,645 -> 1,652, 3,194 -> 1,970 and 3,575 -> 2,137 us.
 //
 // What bounds them: latency at 16 warps per SM (2.0 and 1.5 warp instructions
 // per clock and SM, no pipe above half of its rate).  24 warps at 80
@@ -69,9 +71,7 @@ struct WinTile {
 __host__ __device__ constexpr float window_slab_extra(int R) { return 1.0f + 0.35f * 2 * R; }
 
 // Resident CTAs the register allocation aims at.
-__host__ __device__ constexpr int fwd_min_ctas(int R, FwdMode m) {
-    return R <= 3 ? 2 : 1;
-}
+__host__ __device__ constexpr int fwd_min_ctas(int R) { return R <= 3 ? 2 : 1; }
 __host__ __device__ constexpr int grad_min_ctas(int R) { return R <= 3 ? 2 : 1; }
 
 // A thread's positions.  One outside the grid reads its nearest voxel inside
@@ -505,7 +505,7 @@ __device__ __forceinline__ void lncc_fwd_body(const FwdArgs &g, int bx, int by, 
 }
 
 template <int R, FwdMode M>
-__global__ void __launch_bounds__(WinTile<R>::NT, fwd_min_ctas(R, M)) k_lncc_fwd(const __grid_constant__ FwdArgs g) {
+__global__ void __launch_bounds__(WinTile<R>::NT, fwd_min_ctas(R)) k_lncc_fwd(const __grid_constant__ FwdArgs g) {
     lncc_fwd_body<R, M>(g, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
