@@ -80,11 +80,15 @@ __device__ __forceinline__ void load4(float (&v)[4], const float *__restrict__ p
     }
 }
 
+// PAD: rows hold W voxels and P elements, P a multiple of 4 (such volumes have
+// fewer than 2^32 elements); else P = W.  The dense forms keep their registers
+// (36 instead of 32 would leave the range kernel 7 of its 8 blocks per SM: 1.5
+// us of 148 for the loss and its gradient on 6.9 M voxels).
 // Which of the values i .. i + 3 (i a multiple of 4) of a volume of N elements
-// are voxels: the first so many.  Rows hold W voxels and P elements, P == W or
-// a multiple of 4 (volumes with such rows hold fewer than 2^32 elements).
+// are voxels: the first so many.
+template <bool PAD>
 __device__ __forceinline__ int voxels4(long long i, long long N, int W, int P) {
-    if (P == W) return i + 4 <= N ? 4 : (int)(N - i);
+    if (!PAD) return i + 4 <= N ? 4 : (int)(N - i);
     return min(4, max(0, W - (int)((unsigned)i % (unsigned)P)));
 }
 
@@ -99,6 +103,7 @@ __global__ void k_mi_range_set(const float *range, unsigned *keys) {
     if (threadIdx.x < 4) keys[threadIdx.x] = fkey(range[threadIdx.x]);
 }
 
+template <bool PAD>
 __global__ void __launch_bounds__(256) k_mi_range(const float *__restrict__ If,
                                                   const float *__restrict__ Im, long long N,
                                                   int W, int P, unsigned *keys) {
@@ -108,7 +113,7 @@ __global__ void __launch_bounds__(256) k_mi_range(const float *__restrict__ If,
         float a[4], b[4];
         load4(a, If, i, N);
         load4(b, Im, i, N);
-        const int n = voxels4(i, N, W, P);
+        const int n = voxels4<PAD>(i, N, W, P);
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             if (e >= n) break;
@@ -171,6 +176,7 @@ int hist_log_copies(int nb, int lc) {  // at most 2^lc
     return lc;
 }
 
+template <bool PAD>
 __global__ void __launch_bounds__(kHistThreads) k_mi_hist(const float *__restrict__ I,
                                                           const float *__restrict__ J, long long N,
                                                           int W, int P, int B, int lc,
@@ -185,7 +191,7 @@ __global__ void __launch_bounds__(kHistThreads) k_mi_hist(const float *__restric
     bool bad = false;
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += stride) {
-        if (P != W && (int)((unsigned)i % (unsigned)P) >= W) continue;  // a row's padding
+        if (PAD && (int)((unsigned)i % (unsigned)P) >= W) continue;
         const float a = I[i], b = J[i];
         if (!(fabsf(a) <= 3.4e38f && fabsf(b) <= 3.4e38f)) {
             bad = true;
@@ -381,7 +387,8 @@ cudaError_t launch_mi_range(const float *If, const float *Im, Dims d, MiBuffers 
     const long long N = d.NP();
     k_mi_range_init<<<1, 1, 0, s>>>(b.range);
     note_launch();
-    k_mi_range<<<grid_blocks(N), 256, 0, s>>>(If, Im, N, d.W, d.pitch(), b.range);
+    auto range = d.pitch() != d.W ? k_mi_range<true> : k_mi_range<false>;
+    range<<<grid_blocks(N), 256, 0, s>>>(If, Im, N, d.W, d.pitch(), b.range);
     note_launch();
     return cudaGetLastError();
 }
@@ -399,7 +406,8 @@ cudaError_t launch_mi(const float *I, const float *J, const float *grad, Dims d,
     const int nb = bins * bins;
     cudaError_t e = cudaMemsetAsync(b.hist, 0, sizeof(unsigned long long) * nb, s);
     if (e != cudaSuccess) return e;
-    prepare(k_mi_hist, kHistSmem, kHistThreads);
+    auto hist = d.pitch() != d.W ? k_mi_hist<true> : k_mi_hist<false>;
+    prepare(hist, kHistSmem, kHistThreads);
     const bool one_pass = N <= 512ll * num_sms();
     const int threads = one_pass ? 512 : kHistThreads;
     const int lc = hist_log_copies(nb, one_pass ? 2 : 5);
@@ -407,7 +415,7 @@ cudaError_t launch_mi(const float *I, const float *J, const float *grad, Dims d,
     long long hb = (most + kHistIters - 1) / kHistIters;
     hb = hb < num_sms() ? num_sms() : hb;
     hb = hb < most ? hb : most;
-    k_mi_hist<<<(unsigned)hb, threads, ((size_t)nb << lc) * 8, s>>>(
+    hist<<<(unsigned)hb, threads, ((size_t)nb << lc) * 8, s>>>(
         I, J, N, d.W, d.pitch(), bins, lc, b.range, b.hist, h);
     note_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
