@@ -261,10 +261,13 @@ static cudaError_t onepass(const float *in, float *out, int C, Dims d, const Gau
 }
 
 // The one-pass kernel takes unpadded grids that its launch limits allow (65,535
-// layers of tiles along y and of slabs); anything else goes axis by axis.
+// layers of tiles along y and of slabs) and that have more than five rows; anything
+// else goes axis by axis.  With fewer rows its tiles of 32 are mostly empty (three
+// channels of 600 x H x 701, sigma 1, one pass against three, us: H = 1 87 and 44,
+// 2 87 and 53, 4 87 and 76; sigma 2: H = 4 150 and 98, 6 152 and 146).
 static bool onepass_takes(int C, Dims d, const GaussTaps &t) {
-    return t.R >= 1 && t.R <= kOnePassRadius && d.pitch() == d.W && (d.H + 31) / 32 <= 65535 &&
-           (long long)C * d.D <= 65535;
+    return t.R >= 1 && t.R <= kOnePassRadius && d.pitch() == d.W && d.H > 5 &&
+           (d.H + 31) / 32 <= 65535 && (long long)C * d.D <= 65535;
 }
 
 cudaError_t launch_gauss3(const float *in, float *out, float *t1, float *t2, int C, Dims d,
