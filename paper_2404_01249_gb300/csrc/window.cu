@@ -23,34 +23,46 @@ LaunchGeom window_geom(Dims d, int tz, int occ) {
     return g;
 }
 
-template <int R, FwdMode M>
+template <int R, FwdMode M, int RZ>
 cudaError_t fwd(FwdArgs &a, Dims d, int tz, cudaStream_t s) {
-    using S = FwdSmem<R, M>;
-    auto kern = k_lncc_fwd<R, M>;
+    using S = FwdSmem<R, M, RZ>;
+    auto kern = k_lncc_fwd<R, M, RZ>;
     const int occ = prepare(kern, S::bytes, WinTile<R>::NT);
     const LaunchGeom g = window_geom<R>(d, tz, occ);
     a.TZ = g.tz;
     return launch_pdl(kern, g, S::bytes, s, a);
 }
 
-template <int R, bool SWAP>
+template <int R, bool SWAP, int RZ>
 cudaError_t grad(GradArgs &a, Dims d, int tz, cudaStream_t s) {
-    using S = GradTile<R>;
-    auto kern = k_lncc_grad<R, SWAP>;
+    using S = GradTile<R, RZ>;
+    auto kern = k_lncc_grad<R, SWAP, RZ>;
     const int occ = prepare(kern, S::bytes, WinTile<R>::NT);
     const LaunchGeom g = window_geom<R>(d, tz, occ);
     a.TZ = g.tz;
     return launch_pdl(kern, g, S::bytes, s, a);
 }
 
-template <int R>
+template <int R, int RZ>
 cudaError_t fwd_mode(FwdMode m, FwdArgs &a, Dims d, int tz, cudaStream_t s) {
     switch (m) {
-        case kFwdGiven: return fwd<R, kFwdGiven>(a, d, tz, s);
-        case kFwdBoth: return fwd<R, kFwdBoth>(a, d, tz, s);
-        case kFwdStats: return fwd<R, kFwdStats>(a, d, tz, s);
+        case kFwdGiven: return fwd<R, kFwdGiven, RZ>(a, d, tz, s);
+        case kFwdBoth: return fwd<R, kFwdBoth, RZ>(a, d, tz, s);
+        case kFwdStats: return fwd<R, kFwdStats, RZ>(a, d, tz, s);
     }
     return cudaErrorInvalidValue;
+}
+
+template <int R, int RZ>
+cudaError_t grad_swap(bool swap, GradArgs &a, Dims d, int tz, cudaStream_t s) {
+    return swap ? grad<R, true, RZ>(a, d, tz, s) : grad<R, false, RZ>(a, d, tz, s);
+}
+
+// Planes of one row each are one plane of these rows, in memory and to windows
+// that are cubes: the sums are exact, so their order does not show.  (The rows'
+// tiles must fit the launch grid.)
+Dims as_plane(Dims d) {
+    return d.H == 1 && d.D <= 8 * 65535 ? Dims{1, d.D, d.W, d.P} : d;
 }
 
 template <class A>
@@ -77,22 +89,24 @@ void fill_grid(A &a, Dims d) {
 
 cudaError_t launch_window_fwd(FwdMode mode, FwdArgs a, Dims d, int window, int tz,
                               cudaStream_t s) {
+    d = as_plane(d);
     fill_grid(a, d);
     a.window = window;
     a.bits = lncc_image_bits(window);
     cudaError_t e = cudaErrorInvalidValue;
-    FA_EACH_R((fwd_mode<RR>(mode, a, d, tz, s)))
+    FA_EACH_R((d.D == 1 ? fwd_mode<RR, 0>(mode, a, d, tz, s) : fwd_mode<RR, RR>(mode, a, d, tz, s)))
     note_launch();
     return e;
 }
 
 cudaError_t launch_window_grad(bool swap, GradArgs a, Dims d, int window, int tz,
                                cudaStream_t s) {
+    d = as_plane(d);
     fill_grid(a, d);
     a.n = window * window * window;
     a.cbits = lncc_coef_bits(window);
     cudaError_t e = cudaErrorInvalidValue;
-    FA_EACH_R((swap ? grad<RR, true>(a, d, tz, s) : grad<RR, false>(a, d, tz, s)))
+    FA_EACH_R((d.D == 1 ? grad_swap<RR, 0>(swap, a, d, tz, s) : grad_swap<RR, RR>(swap, a, d, tz, s)))
     note_launch();
     return e;
 }

@@ -62,9 +62,14 @@ struct WinTile {
     static constexpr int RX = FX + 2 * R, RY = TY + 2 * R, NPOS = RX * RY;
     static constexpr int PP = (NPOS + NT - 1) / NT;  // positions per thread
     static constexpr int NPAD = PP * NT;             // their slots in shared memory
-    static constexpr int HS = 2 * R;                 // planes a ring holds
     static constexpr int CG = TY / 8;                // column items per column
 };
+
+// RZ, the radius along z of the bodies below, is R, or 0 for a volume of one
+// plane: there the windows' other planes add nothing, and the march of 2 R + 1
+// planes with its ring is left out (1 x 1024 x 1024, both gradients: windows of 9
+// to 15 294, 381, 447 and 543 us marching, 96, 109, 130 and 137 so; 249, 279, 302 and 326
+// before the sums ran z first).
 
 // What a slab costs beyond its output planes, in output planes: the 2R planes
 // before its first output take the z sums only (about a third of a plane).
@@ -265,22 +270,23 @@ __device__ __forceinline__ void store2(float *p, long long N, const float2 (&v)[
 // ============================================================== forward (K1)
 constexpr int fwd_channels(FwdMode m) { return m == kFwdGiven ? 3 : (m == kFwdBoth ? 5 : 2); }
 
-template <int R, FwdMode M>
+template <int R, FwdMode M, int RZ = R>
 struct FwdSmem {
     using G = WinTile<R>;
     static constexpr int NCH = fwd_channels(M);
-    static constexpr size_t ring = (size_t)G::HS * G::NPAD * (M == kFwdStats ? 4 : 8);
+    static constexpr int HS = 2 * RZ;  // planes the ring holds
+    static constexpr size_t ring = (size_t)HS * G::NPAD * (M == kFwdStats ? 4 : 8);
     static constexpr size_t o_zs = (ring + 15) / 16 * 16;
     static constexpr size_t o_ys = o_zs + (size_t)NCH * G::NPAD * 8;
     static constexpr size_t bytes = o_ys + (size_t)NCH * G::TY * G::RX * 8;
     static_assert(bytes + 512 <= 227 * 1024, "a CTA's shared memory");
 };
 
-template <int R, FwdMode M>
+template <int R, FwdMode M, int RZ = R>
 __device__ __forceinline__ void lncc_fwd_body(const FwdArgs &g, int bx, int by, int bz) {
     using G = WinTile<R>;
-    using S = FwdSmem<R, M>;
-    constexpr int NT = G::NT, PP = G::PP, NPAD = G::NPAD, HS = G::HS, NCH = S::NCH;
+    using S = FwdSmem<R, M, RZ>;
+    constexpr int NT = G::NT, PP = G::PP, NPAD = G::NPAD, HS = S::HS, NCH = S::NCH;
     constexpr bool HASJ = M != kFwdStats;
     extern __shared__ __align__(128) unsigned char smem[];
     int2 *ring2 = (int2 *)smem;  // [HS][NPAD]: q_I, q_J
@@ -293,7 +299,7 @@ __device__ __forceinline__ void lncc_fwd_body(const FwdArgs &g, int bx, int by, 
     const int x0 = bx * FX, y0 = by * G::TY, z0 = bz * g.TZ;
     const int zend = min(z0 + g.TZ, g.D);
     const long long HW = (long long)g.H * g.P, N = HW * g.D;
-    const int zs0 = z0 - R, np = zend - z0 + 2 * R;
+    const int zs0 = z0 - RZ, np = zend - z0 + 2 * RZ;
     WinPos<R> wp;
     wp.init(tid, x0, y0, g.H, g.W, g.P);
     const int ox = x0 + 2 * pair, oy = y0 + row;
@@ -348,7 +354,7 @@ __device__ __forceinline__ void lncc_fwd_body(const FwdArgs &g, int bx, int by, 
         fetch(i + 1);
         Two<long long> sI2[1] = {{0, 0}};
         Two<float> vI2[1] = {{0.f, 0.f}};
-        const long long zo = (long long)(zp - R) * HW;
+        const long long zo = (long long)(zp - RZ) * HW;
         if (M == kFwdGiven && emit && live) {
             load2(sI2, g.SI + zo + ooff, N, both, vec);
             load2(vI2, g.varI + zo + ooff, N, both, vec);
@@ -504,9 +510,9 @@ __device__ __forceinline__ void lncc_fwd_body(const FwdArgs &g, int bx, int by, 
     }
 }
 
-template <int R, FwdMode M>
+template <int R, FwdMode M, int RZ = R>
 __global__ void __launch_bounds__(WinTile<R>::NT, fwd_min_ctas(R)) k_lncc_fwd(const __grid_constant__ FwdArgs g) {
-    lncc_fwd_body<R, M>(g, blockIdx.x, blockIdx.y, blockIdx.z);
+    lncc_fwd_body<R, M, RZ>(g, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
 // ============================================================= gradient (K2)
@@ -518,25 +524,26 @@ __global__ void __launch_bounds__(WinTile<R>::NT, fwd_min_ctas(R)) k_lncc_fwd(co
 // the bits of floats in [2^23, 2^24) (adding 1.5 2^23 rounds to an integer);
 // the constant exponent bits are added along with them and n of them are
 // subtracted from the finished sum (all arithmetic is modulo 2^32).
-template <int R>
+template <int R, int RZ = R>
 struct GradTile {
     using G = WinTile<R>;
+    static constexpr int HS = 2 * RZ;  // planes between a plane's coming and leaving
     static constexpr int RB = R <= 5 ? 20 : 18;
     // windows of 13 and 15: the ring would not fit, so the plane that leaves
     // the window is loaded and quantised again
-    static constexpr bool RING = R <= 5 && R > 0;
-    static constexpr size_t ring = RING ? (size_t)G::HS * G::NPAD * 3 * 8 : 0;  // [HS][3][NPAD]
+    static constexpr bool RING = R <= 5 && RZ > 0;
+    static constexpr size_t ring = RING ? (size_t)HS * G::NPAD * 3 * 8 : 0;  // [HS][3][NPAD]
     static constexpr size_t o_zs = (ring + 15) / 16 * 16;
     static constexpr size_t o_ys = o_zs + (size_t)3 * G::NPAD * 8;
     static constexpr size_t bytes = o_ys + (size_t)3 * G::TY * G::RX * 8;
     static_assert(bytes + 512 <= 227 * 1024, "a CTA's shared memory");
 };
 
-template <int R, bool SWAP>
+template <int R, bool SWAP, int RZ = R>
 __device__ __forceinline__ void lncc_grad_body(const GradArgs &g, int bx, int by, int bz) {
     using G = WinTile<R>;
-    using S = GradTile<R>;
-    constexpr int NT = G::NT, PP = G::PP, NPAD = G::NPAD, HS = G::HS;
+    using S = GradTile<R, RZ>;
+    constexpr int NT = G::NT, PP = G::PP, NPAD = G::NPAD, HS = S::HS;
     constexpr int CB = SWAP ? 4 : 1;  // channel of B; C hi and lo follow
     extern __shared__ __align__(128) unsigned char smem[];
     Limb2 *ring = (Limb2 *)smem;
@@ -546,7 +553,7 @@ __device__ __forceinline__ void lncc_grad_body(const GradArgs &g, int bx, int by
     const int x0 = bx * FX, y0 = by * G::TY, z0 = bz * g.TZ;
     const int zend = min(z0 + g.TZ, g.D);
     const long long HW = (long long)g.H * g.P, N = HW * g.D;
-    const int zs0 = z0 - R, np = zend - z0 + 2 * R;
+    const int zs0 = z0 - RZ, np = zend - z0 + 2 * RZ;
     WinPos<R> wp;
     wp.init(tid, x0, y0, g.H, g.W, g.P);
     const int ox = x0 + 2 * pair, oy = y0 + row;
@@ -597,7 +604,7 @@ __device__ __forceinline__ void lncc_grad_body(const GradArgs &g, int bx, int by
     }
     auto ask = [&](int i) {
         const int z = zs0 + i + kAhead;
-        if (line && z >= 0 && z < min(zend + R, g.D))
+        if (line && z >= 0 && z < min(zend + RZ, g.D))
             asm volatile("prefetch.global.L2 [%0];" ::"l"(line + (long long)z * HW));
     };
     auto quant = [&](const Raw &f, int i, Limb2 (&q)[PP][3]) {
@@ -628,7 +635,7 @@ __device__ __forceinline__ void lncc_grad_body(const GradArgs &g, int bx, int by
             fetch(f, i - HS);
             quant(f, i - HS, old);
         }
-        const long long zo = (long long)(zs0 + i - R) * HW;
+        const long long zo = (long long)(zs0 + i - RZ) * HW;
         Two<float> Iv[1], Jv[1], gv[3];
         if (emit && live) {
             load2(Iv, g.I + zo + ooff, N, both, vec);
@@ -662,7 +669,8 @@ __device__ __forceinline__ void lncc_grad_body(const GradArgs &g, int bx, int by
         float2 hi[3], lo[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const unsigned base = kLimbBits * (unsigned)g.n * (c == 2 ? 2u : 1u);
+            const unsigned terms = (unsigned)(RZ == R ? g.n : (2 * R + 1) * (2 * R + 1));
+            const unsigned base = kLimbBits * terms * (c == 2 ? 2u : 1u);
             long long x[2];
 #pragma unroll
             for (int e = 0; e < 2; ++e)
@@ -689,9 +697,9 @@ __device__ __forceinline__ void lncc_grad_body(const GradArgs &g, int bx, int by
     }
 }
 
-template <int R, bool SWAP>
+template <int R, bool SWAP, int RZ = R>
 __global__ void __launch_bounds__(WinTile<R>::NT, grad_min_ctas(R)) k_lncc_grad(const __grid_constant__ GradArgs g) {
-    lncc_grad_body<R, SWAP>(g, blockIdx.x, blockIdx.y, blockIdx.z);
+    lncc_grad_body<R, SWAP, RZ>(g, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
 }  // namespace
