@@ -43,9 +43,15 @@ thread_local const TileChoice *g_force = nullptr;  // a candidate under measurem
 // 32 x 8 tiles with their three CTAs per SM (ten MSE iterations without either
 // smoothing: 160 x 192 x 224 3,367 us on 32 x 16 tiles, 3,271 on 32 x 8, 40 x 24 x 64
 // 113 and 103; before the passes were pipelined 3,393 and 106).
+// With eight rows or fewer the second half of the taller tile is empty (ten
+// iterations, 32 x 16 and 32 x 8, us: MSE on 600 x 2 x 701 1,597 and 1,036, 300 x 8 x 401
+// 730 and 637, 300 x 8 x 8 215 and 208; LNCC on 300 x 8 x 401 1,216 and 1,120,
+// 200 x 8 x 64 374 and 372, but on 300 x 8 x 8 304 and 328: its CTAs, a narrow tile of
+// one plane each, start during the kernel before and crowd on the SMs that are
+// free first).
 int default_wide(int kernel, int radius, Dims d) {
     const long long tiles = (long long)((d.W + FX - 1) / FX) * ((d.H + 15) / 16);
-    if (kernel == 3 && radius == 0) return 0;
+    if (d.H <= 8 || (kernel == 3 && radius == 0)) return 0;
     return kernel >= 2 && tiles * d.D >= num_sms();
 }
 
